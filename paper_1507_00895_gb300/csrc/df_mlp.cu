@@ -18,167 +18,408 @@
 #include <cuda_bf16.h>
 
 #include "df_tcgj_dev.cuh"
+#include "df_tcr_dev.cuh"
 
 namespace df {
 
-constexpr int kGm = 128, kGn = 128, kGk = 64;  // block tile: M x N outputs, K per stage
-constexpr int kGemmThreads = 256;               // 8 warps: staging, epilogue; thread 0 issues the MMAs
-constexpr int kGemmTmemCols = 128;              // the FP32 accumulator tile (N = 128 columns)
-constexpr int kGemmStage = kGm * kGk * 2;       // bytes of one operand tile (128 rows x 64 bf16)
-constexpr int kGemmSmem = 4 * kGemmStage + 1024;   // two stages of (A, B) + alignment slack
+// ---- BF16 operands as swizzled atoms ---------------------------------------
+// A BF16 matrix X[r][c] that a product reads is kept in global memory as
+// 1 KB atoms of 8 rows x 64 columns, the 128-byte-swizzled layout of the
+// tensor cores' shared-memory operands: 16-byte chunk q of row r at chunk
+// q ^ (r & 7).  Atom (r / 8, c / 64) is at index (c / 64) * rg + r / 8, rg the
+// number of 8-row groups (rows and columns padded to 128 with zeros).  A
+// run of row groups of one 64-column block is one contiguous piece, so
+// that a bulk asynchronous copy brings a whole tile, and the same atoms
+// serve a product that sums over the columns (K-major operand) and one that
+// sums over the rows (MN-major operand): the network's three products per
+// layer read activations, dZ and weights in both ways without a transpose.
+__host__ __device__ constexpr long pad128(long x) { return (x + 127) / 128 * 128; }
+__host__ __device__ constexpr size_t atoms_bytes(long rows, long cols) { return (size_t)pad128(rows) * pad128(cols) * 2; }
+// byte offset of the 16-byte chunk holding columns c .. c + 7 (c a multiple of 8) of row r
+__device__ __forceinline__ size_t atom_chunk(int r, int c, int rg) {
+  return ((size_t)(c >> 6) * rg + (r >> 3)) * 1024 + (size_t)((r & 7) * 128 + ((((c & 63) >> 3) ^ (r & 7)) << 4));
+}
+__device__ __forceinline__ unsigned pack_bf16(float lo, float hi) {
+  const __nv_bfloat162 p = __floats2bfloat162_rn(lo, hi);
+  return *reinterpret_cast<const unsigned*>(&p);
+}
 
-// C[m][n] = act(sum_k bf16(A(m,k)) bf16(B(k,n)) + bias[n]) (+ C[m][n] if accumulate)
-// A(m,k) = A[m sam + k sak], B(k,n) = B[k sbk + n sbn], C row-major with ldc.
-// act: 0 identity, 1 tanh.  One 128 x 128 output tile per block on the tensor
-// cores (tcgen05, M = 128, N = 128, K = 16 per MMA, FP32 accumulator in tensor
-// memory): per stage of 64 k the block rounds its A and B tiles to BF16 into
-// shared memory (K-major, 128-byte swizzle), thread 0 issues 4 MMAs and commits
-// them to the stage buffer's barrier, and the next stage is staged into the
-// other buffer meanwhile.  The epilogue reads the accumulator from tensor
-// memory (warp w: lanes 32 (w % 4) .., columns 64 (w / 4) ..).  Waits are
-// bounded; one that gives up sets *err.
-__global__ void __launch_bounds__(kGemmThreads)
-gemm_tc_kernel(int M, int N, int K, const float* __restrict__ A, long sam, long sak, const float* __restrict__ B,
-               long sbk, long sbn, float* __restrict__ C, long ldc, const float* __restrict__ bias, int act,
-               int accumulate, int* __restrict__ err) {
+// ---- the products ------------------------------------------------------------
+// One kernel for every product D[m][n] = sum_k A(m, k) B(k, n) of the network,
+// an output tile of TM x TN per block, K in stages of KB blocks of 64:
+//   warp 8 (one lane) streams the operand tiles into a ring of NS stages by
+//   bulk asynchronous copies; warp 9 (one lane) issues the MMAs (M = TM,
+//   N = TN, K = 16, FP32 accumulator in tensor memory) and its commits hand
+//   the stages back; warps 0-7 run the epilogue, and where B is the FP32
+//   weights (WF32: the forward products) they round the weight tile to BF16
+//   into the stage, loading one stage ahead in registers, and with wsh leave
+//   the rounded tile in global memory for the backward product.
+// AMN / BMN: the operand's M / N index is the atoms' column (MN-major), the
+// sum runs over the atoms' rows; else K-major.
+// The accumulation runs over k in order whatever the tile, so every tile
+// shape gives the same bits.
+// A 256-row batch at 512 x 71808 (before: FP32 operands rounded and transposed
+// by every block with two-byte stores, two stages, 128 x 128 tiles throughout):
+//   forward with the loss     0.11 ms   147 MB of weights, 74 MB of targets read
+//   weight gradient           0.056 ms  147 MB of gradients written (HBM: 0.03)
+//   activation gradient       0.23 ms   K = 71808; one block per 64 x 16 outputs so that
+//                                       128 of the 152 SMs work, bound by the L2 -> shared
+//                                       memory traffic of its 1.5 GB of tiles (was 8 blocks,
+//                                       ~10 ms); a split K would change the summation order
+//                                       and with it BF16 roundings downstream
+// and the whole training step 13.1 -> 0.70 ms.
+enum GemmEpi {
+  kEpiStore = 0,     // C = D
+  kEpiTanh = 1,      // a = tanh(D + bias): C = a, Cb = bf16(a)
+  kEpiLinear = 2,    // C = D + bias
+  kEpiLoss = 3,      // y = D + bias, dZ = 2 (y - aux) scale: Cb = bf16(dZ), column and loss partials
+  kEpiBack = 4,      // dZ = D (1 - aux^2): Cb = bf16(dZ), column partials
+};
+
+struct GemmArgs {
+  int M, N, nkb;                 // outputs; K in 64-blocks
+  const unsigned char* A;        // atoms, a_rg row groups
+  int a_rg;
+  const unsigned char* B;        // atoms, b_rg row groups (not WF32)
+  int b_rg;
+  const float* W;                // WF32: W[k][n], k < kw rows, ldw = N
+  int kw, wvec;
+  unsigned char* wsh;            // WF32: the rounded weights' atoms (NULL: not kept)
+  int wsh_rg;
+  int epi;
+  float* C;                      // FP32 output, row stride N
+  unsigned char* Cb;             // BF16 atoms of the output
+  int cb_rg;
+  const float* bias;
+  const float* aux;              // kEpiLoss: target, kEpiBack: activations; row stride N
+  float scale;
+  float* part_col;               // [m tiles * 4][N] sums of dZ over a quadrant's rows
+  float* part_loss;              // [blocks] sums of (y - target)^2
+  int* err;
+};
+
+constexpr int kGemmThreads = 320;
+
+__host__ __device__ constexpr int gemm_stage_bytes(int TM, int TN, int KB) { return (TM + TN) * 128 * KB; }
+__host__ __device__ constexpr int gemm_smem_bytes(int TM, int TN, int KB, int NS) {
+  const int ring = NS * gemm_stage_bytes(TM, TN, KB), epi = 8 * 32 * 33 * 4;
+  return (ring > epi ? ring : epi) + 1024;
+}
+
+// shared-memory descriptor of an MN-major operand of 128-byte-swizzled atoms:
+// atoms along K 1024 B apart, along M / N (64 elements) 8192 B apart
+__device__ __forceinline__ uint64_t umma_desc_mn(unsigned saddr) {
+  return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)(8192 >> 4) << 16) | ((uint64_t)(1024 >> 4) << 32) |
+         ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
+}
+
+__device__ __forceinline__ void bulk_g2s(unsigned dst, const void* src, unsigned bytes, uint64_t* mbar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+               "l"(src), "r"(bytes), "r"(smem_u32(mbar))
+               : "memory");
+}
+__device__ __forceinline__ void mbar_init(uint64_t* b, unsigned count) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(b)), "r"(count) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive(uint64_t* b) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(b)) : "memory");
+}
+__device__ __forceinline__ void mbar_expect(uint64_t* b, unsigned bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(b)), "r"(bytes) : "memory");
+}
+
+// the tile's loads of one operand for stage `it`: T rows of the product
+// (m or n) from t0, KB 64-blocks of k
+template <int T, int KB, bool MN>
+__device__ __forceinline__ void load_operand(const unsigned char* X, int rg, int t0, int it, unsigned dst,
+                                             uint64_t* full) {
+  if constexpr (MN) {
+    static_assert(KB == 1 && T % 64 == 0, "MN-major tiles are 64-column blocks of 8 row groups");
+#pragma unroll
+    for (int cb = 0; cb < T / 64; ++cb)
+      bulk_g2s(dst + cb * 8192, X + ((size_t)(t0 / 64 + cb) * rg + it * 8) * 1024, 8192, full);
+  } else {
+#pragma unroll
+    for (int kb = 0; kb < KB; ++kb)
+      bulk_g2s(dst + kb * T * 128, X + ((size_t)(it * KB + kb) * rg + t0 / 8) * 1024, T * 128, full);
+  }
+}
+
+template <int TM, int TN, int KB, int NS, bool AMN, bool BMN, bool WF32>
+__global__ void __launch_bounds__(kGemmThreads, TM == 128 ? 2 : 1)
+gemm_tc_kernel(const GemmArgs g) {
+  static_assert(!WF32 || (BMN && KB == 1 && !AMN), "FP32 weights are the forward products' B operand");
   extern __shared__ unsigned char gsm_raw[];
-  __shared__ uint64_t bar_s[2];
+  __shared__ uint64_t full_s[NS], empty_s[NS], done_s;
   __shared__ unsigned tslot_s;
+  __shared__ int fail_s;
+  __shared__ float loss_s[8];
   unsigned char* gsm = reinterpret_cast<unsigned char*>(((uintptr_t)gsm_raw + 1023) & ~(uintptr_t)1023);
-  const int m0 = blockIdx.y * kGm, n0 = blockIdx.x * kGn;
+  constexpr int kA = TM * 128 * KB, kB = TN * 128 * KB, kStage = kA + kB;
+  constexpr int kTmem = TN < 32 ? 32 : TN;
+  const int m0 = blockIdx.x * TM, n0 = blockIdx.y * TN;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  if (warp == 0) tmem_alloc_cols<kGemmTmemCols>(&tslot_s);
+  const int nit = (g.nkb + KB - 1) / KB;
+  if (warp == 0) tmem_alloc_cols<kTmem>(&tslot_s);
   if (tid == 0) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&bar_s[0])) : "memory");
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&bar_s[1])) : "memory");
+    for (int s = 0; s < NS; ++s) {
+      mbar_init(&full_s[s], WF32 ? 9 : 1);      // the copies' thread, and the eight converting warps
+      mbar_init(&empty_s[s], 1);
+    }
+    mbar_init(&done_s, 1);
+    fail_s = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   tc05_fence_before();
   __syncthreads();
   tc05_fence_after();
-  const unsigned tmem = tslot_s;
-  const unsigned idesc = umma_idesc_bf16(kGm, kGn);
-  unsigned ph = 0u;                                  // bit b: the phase of buffer b's barrier
-  bool ok = true;
-  const int nst = (K + kGk - 1) / kGk;
-  for (int st = 0; st < nst; ++st) {
-    const int b = st & 1, k0 = st * kGk;
-    if (st >= 2) {                                   // the MMAs that read this buffer are done
-      ok = ok && mbar_wait(&bar_s[b], (ph >> b) & 1u);
-      ph ^= 1u << b;
+  const unsigned tmem = tslot_s, ring = smem_u32(gsm);
+
+  if (warp == 8) {
+    if (lane == 0) {
+      int it = 0;
+      for (; it < nit; ++it) {
+        const int s = it % NS;
+        if (it >= NS && !mbar_wait(&empty_s[s], (unsigned)((it / NS - 1) & 1))) break;
+        mbar_expect(&full_s[s], WF32 ? kA : kStage);
+        load_operand<TM, KB, AMN>(g.A, g.a_rg, m0, it, ring + s * kStage, &full_s[s]);
+        if constexpr (!WF32) load_operand<TN, KB, BMN>(g.B, g.b_rg, n0, it, ring + s * kStage + kA, &full_s[s]);
+      }
+      if (it < nit) {                           // gave up: its copies in flight land first (bounded)
+        fail_s = 1;
+        for (int k = it - NS < 0 ? 0 : it - NS; k < it; ++k) mbar_wait(&full_s[k % NS], (unsigned)((k / NS) & 1));
+      }
     }
-    if (__syncthreads_or(!ok)) break;
-    __nv_bfloat16* As = reinterpret_cast<__nv_bfloat16*>(gsm + b * 2 * kGemmStage);
-    __nv_bfloat16* Bs = reinterpret_cast<__nv_bfloat16*>(gsm + b * 2 * kGemmStage + kGemmStage);
-    // A tile [m][k]: k fastest when A's rows are contiguous, m fastest otherwise
-    for (int idx = tid; idx < kGm * kGk; idx += kGemmThreads) {
-      const int r = sak == 1 ? idx / kGk : idx % kGm, k = sak == 1 ? idx % kGk : idx / kGm;
-      const int gm = m0 + r, gk = k0 + k;
-      const float v = (gm < M && gk < K) ? A[gm * sam + gk * sak] : 0.f;
-      As[swz(r, k)] = __float2bfloat16_rn(v);
-    }
-    // B tile [n][k]: n fastest when B's rows (over n) are contiguous, k fastest otherwise
-    for (int idx = tid; idx < kGn * kGk; idx += kGemmThreads) {
-      const int nn = sbn == 1 ? idx % kGn : idx / kGk, k = sbn == 1 ? idx / kGn : idx % kGk;
-      const int gn = n0 + nn, gk = k0 + k;
-      const float v = (gn < N && gk < K) ? B[gk * sbk + gn * sbn] : 0.f;
-      Bs[swz(nn, k)] = __float2bfloat16_rn(v);
-    }
-    fence_async_smem();
-    tc05_fence_before();
-    __syncthreads();
-    if (tid == 0) {
-      tc05_fence_after();
-      const unsigned a = smem_u32(As), bb = smem_u32(Bs);
+  } else if (warp == 9) {
+    if (lane == 0) {
+      const unsigned idesc = umma_idesc_bf16(TM, TN) | (AMN ? 1u << 15 : 0u) | (BMN ? 1u << 16 : 0u);
+      int it = 0;
+      for (; it < nit; ++it) {
+        const int s = it % NS;
+        if (!mbar_wait(&full_s[s], (unsigned)((it / NS) & 1))) break;
+        tc05_fence_after();
+        const unsigned a = ring + s * kStage, b = a + kA;
 #pragma unroll
-      for (int ks = 0; ks < kGk / 16; ++ks)
-        umma_bf16(tmem, umma_desc_sw128(a + 32 * ks), umma_desc_sw128(bb + 32 * ks), idesc,
-                  (st > 0 || ks > 0) ? 1u : 0u);
-      umma_commit(&bar_s[b]);
+        for (int kb = 0; kb < KB; ++kb)
+#pragma unroll
+          for (int ks = 0; ks < 4; ++ks) {
+            const uint64_t da = AMN ? umma_desc_mn(a + 2048 * ks) : umma_desc_sw128(a + kb * TM * 128 + 32 * ks);
+            const uint64_t db = BMN ? umma_desc_mn(b + 2048 * ks) : umma_desc_sw128(b + kb * TN * 128 + 32 * ks);
+            umma_bf16(tmem, da, db, idesc, (it > 0 || kb > 0 || ks > 0) ? 1u : 0u);
+          }
+        umma_commit(&empty_s[s]);
+      }
+      if (it < nit) fail_s = 1;
+      umma_commit(&done_s);
     }
-  }
-  // the last one or two commits: every MMA done before the epilogue
-  for (int st = nst - 2 < 0 ? 0 : nst - 2; ok && st < nst; ++st) {
-    const int b = st & 1;
-    ok = mbar_wait(&bar_s[b], (ph >> b) & 1u);
-    ph ^= 1u << b;
-  }
-  tc05_fence_after();
-  if (__syncthreads_or(!ok)) {
-    if (tid == 0) atomicOr(err, 1);
   } else {
-    const int q = warp & 3, half = warp >> 2;
-    const int r = m0 + 32 * q + lane;
-    const unsigned tl = tmem + ((32u * q) << 16) + (unsigned)(64 * half);
+    if constexpr (WF32) {
+      // the weight tile: 64 k x TN n, float4 along n
+      constexpr int kPer = 64 * TN / 4 / 256;
+      float4 w[kPer];
+      auto fetch = [&](int it) {
 #pragma unroll
-    for (int c16 = 0; c16 < 4; ++c16) {
-      float v[16];
-      tmem_ld16(tl + 16 * c16, v);
-      if (r < M) {
-#pragma unroll
-        for (int e = 0; e < 16; ++e) {
-          const int cn = n0 + 64 * half + 16 * c16 + e;
-          if (cn < N) {
-            float x = v[e];
-            if (bias) x += bias[cn];
-            if (act == 1) x = tanhf(x);
-            float* dst = C + (long)r * ldc + cn;
-            *dst = accumulate ? *dst + x : x;
+        for (int e = 0; e < kPer; ++e) {
+          const int f = tid + 256 * e, k = it * 64 + f / (TN / 4), n = n0 + (f % (TN / 4)) * 4;
+          w[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (k < g.kw) {
+            const float* src = g.W + (size_t)k * g.N + n;
+            if (g.wvec && n + 3 < g.N) {
+              w[e] = __ldcs(reinterpret_cast<const float4*>(src));
+            } else {
+              if (n < g.N) w[e].x = src[0];
+              if (n + 1 < g.N) w[e].y = src[1];
+              if (n + 2 < g.N) w[e].z = src[2];
+              if (n + 3 < g.N) w[e].w = src[3];
+            }
           }
         }
+      };
+      fetch(0);
+      bool ok = true;
+      for (int it = 0; it < nit; ++it) {
+        const int s = it % NS;
+        if (it >= NS && !(ok = mbar_wait(&empty_s[s], (unsigned)((it / NS - 1) & 1)))) break;
+        unsigned char* bt = gsm + s * kStage + kA;
+#pragma unroll
+        for (int e = 0; e < kPer; ++e) {
+          const int f = tid + 256 * e, k = f / (TN / 4), c = (f % (TN / 4)) * 4;
+          const uint2 v = make_uint2(pack_bf16(w[e].x, w[e].y), pack_bf16(w[e].z, w[e].w));
+          const unsigned o = (unsigned)((k & 7) * 128 + ((((c & 63) >> 3) ^ (k & 7)) << 4) + (c & 4) * 2);
+          *reinterpret_cast<uint2*>(bt + (c >> 6) * 8192 + (k >> 3) * 1024 + o) = v;
+          if (g.wsh && blockIdx.x == 0)
+            *reinterpret_cast<uint2*>(g.wsh + ((size_t)((n0 + c) >> 6) * g.wsh_rg + it * 8 + (k >> 3)) * 1024 + o) = v;
+        }
+        if (it + 1 < nit) fetch(it + 1);
+        fence_async_smem();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&full_s[s]);
       }
+      if (!ok) fail_s = 1;
+    }
+    if (!mbar_wait(&done_s, 0u)) fail_s = 1;
+    tc05_fence_after();
+  }
+  __syncthreads();
+  const bool fail = fail_s != 0;
+  if (fail) {
+    if (tid == 0) atomicOr(g.err, 1);
+  } else if (warp < 8) {
+    // epilogue: warp w takes lane quadrant w % 4 and every second group of CW columns
+    constexpr int CW = TN >= 64 ? 32 : 16;
+    const int q = warp & 3;
+    const bool live = TM == 128 || lane < 16;             // TM = 64: rows 16 q .. 16 q + 15 in lanes 0-15
+    const int r = m0 + (TM == 128 ? 32 * q + lane : 16 * q + lane);
+    const bool in = live && r < g.M;
+    float* stg = reinterpret_cast<float*>(gsm) + warp * 32 * 33;
+    float loss = 0.f;
+#pragma unroll 1
+    for (int ci = warp >> 2; ci < TN / CW; ci += 2) {
+      float v[CW];
+      const unsigned ta = tmem + ((32u * q) << 16) + (unsigned)(CW * ci);
+      tmem_ld16(ta, v);
+      if constexpr (CW == 32) tmem_ld16(ta + 16, v + 16);
+      const int nb = n0 + CW * ci;
+      if (g.epi == kEpiTanh || g.epi == kEpiLinear || g.epi == kEpiLoss) {
+#pragma unroll
+        for (int e = 0; e < CW; ++e)
+          if (nb + e < g.N) v[e] += __ldg(g.bias + nb + e);
+      }
+      if (g.epi == kEpiTanh) {
+#pragma unroll
+        for (int e = 0; e < CW; ++e) v[e] = tanhf(v[e]);
+      }
+      const bool dz = g.epi == kEpiLoss || g.epi == kEpiBack;
+      if (dz || g.C) {                         // through shared memory: a lane per column, rows coalesced
+        constexpr int kRows = TM == 128 ? 32 : 16;
+        const int n = nb + lane, rq = m0 + kRows * q, rows = max(0, min(kRows, g.M - rq));
+        __syncwarp();
+#pragma unroll
+        for (int e = 0; e < CW; ++e) stg[lane * 33 + e] = v[e];
+        __syncwarp();
+        if (lane < CW && n < g.N) {
+          if (g.C) {
+            float* dst = g.C + (size_t)rq * g.N + n;
+            for (int k = 0; k < rows; ++k) __stcs(dst + (size_t)k * g.N, stg[k * 33 + lane]);
+          }
+          if (dz) {
+            const float* ax = g.aux + (size_t)rq * g.N + n;
+            float s = 0.f;
+#pragma unroll
+            for (int k0 = 0; k0 < kRows; k0 += 16) {
+              float x[16];
+#pragma unroll
+              for (int k = 0; k < 16; ++k) x[k] = k0 + k < rows ? __ldg(ax + (size_t)(k0 + k) * g.N) : 0.f;
+#pragma unroll
+              for (int k = 0; k < 16; ++k) {
+                float& y = stg[(k0 + k) * 33 + lane];
+                float z = 0.f;
+                if (k0 + k < rows) {
+                  if (g.epi == kEpiLoss) {
+                    const float d = y - x[k];
+                    z = 2.f * d * g.scale;
+                    loss += d * d;
+                  } else {
+                    z = y * (1.f - x[k] * x[k]);
+                  }
+                }
+                y = z;
+                s += z;
+              }
+            }
+            g.part_col[(size_t)(blockIdx.x * 4 + q) * g.N + n] = s;
+          }
+        }
+        if (dz) {
+          __syncwarp();
+#pragma unroll
+          for (int e = 0; e < CW; ++e) v[e] = stg[lane * 33 + e];
+        }
+      }
+      if (g.Cb) {                              // padding rows and columns as zeros
+#pragma unroll
+        for (int e = 0; e < CW; ++e)
+          if (!in || nb + e >= g.N) v[e] = 0.f;
+        if (live) {
+#pragma unroll
+          for (int e = 0; e < CW; e += 8)
+            *reinterpret_cast<uint4*>(g.Cb + atom_chunk(r, nb + e, g.cb_rg)) =
+                make_uint4(pack_bf16(v[e], v[e + 1]), pack_bf16(v[e + 2], v[e + 3]), pack_bf16(v[e + 4], v[e + 5]),
+                           pack_bf16(v[e + 6], v[e + 7]));
+        }
+      }
+    }
+    if (g.epi == kEpiLoss) {
+      for (int o = 16; o > 0; o >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, o);
+      if (lane == 0) loss_s[warp] = loss;
     }
   }
   tc05_fence_before();
   __syncthreads();
   tc05_fence_after();
-  if (warp == 0) tmem_dealloc_cols<kGemmTmemCols>(tmem);
-}
-
-// dY = 2 (Y - T) / (B n_out); per-block partial sums of (Y - T)^2
-__global__ void mse_grad_kernel(long count, const float* __restrict__ y, const float* __restrict__ t,
-                                float* __restrict__ dy, float scale, float* __restrict__ partial) {
-  __shared__ float sred[32];
-  float s = 0.f;
-  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < count; i += (long)gridDim.x * blockDim.x) {
-    const float d = y[i] - t[i];
-    dy[i] = 2.f * d * scale;
-    s += d * d;
+  if (!fail && g.epi == kEpiLoss && tid == 0) {
+    float s = 0.f;
+    for (int w = 0; w < 8; ++w) s += loss_s[w];
+    g.part_loss[blockIdx.y * gridDim.x + blockIdx.x] = s;
   }
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if ((threadIdx.x & 31) == 0) sred[threadIdx.x >> 5] = s;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    s = (threadIdx.x < blockDim.x / 32) ? sred[threadIdx.x] : 0.f;
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (threadIdx.x == 0) partial[blockIdx.x] = s;
+  if (warp == 0) tmem_dealloc_cols<kTmem>(tmem);
+}
+
+// x [M][N] FP32 -> BF16 atoms, rows up to the next multiple of 128 and padding columns zero
+__global__ void to_atoms_kernel(int M, int N, const float* __restrict__ x, unsigned char* __restrict__ out, int rg) {
+  const int cols8 = (int)(pad128(N) / 8);
+  const long total = pad128(M) * cols8;
+  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < total; i += (long)gridDim.x * blockDim.x) {
+    const int r = (int)(i / cols8), c = (int)(i - (long)r * cols8) * 8;
+    float v[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) v[e] = (r < M && c + e < N) ? x[(size_t)r * N + c + e] : 0.f;
+    *reinterpret_cast<uint4*>(out + atom_chunk(r, c, rg)) =
+        make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
   }
 }
 
-// dZ = dA (1 - A^2)  (tanh layers)
-__global__ void tanh_back_kernel(long count, const float* __restrict__ a, float* __restrict__ dz) {
-  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < count; i += (long)gridDim.x * blockDim.x)
-    dz[i] = dz[i] * (1.f - a[i] * a[i]);
+// db_l[n] = sum of the layer's row-quadrant partials of dZ (blockIdx.y = layer)
+struct BiasGrads {
+  const float* part[4];
+  float* db[4];
+  int n[4], parts[4];
+};
+__global__ void bias_grad_kernel(const BiasGrads b) {
+  const int l = blockIdx.y, N = b.n[l];
+  for (int n = blockIdx.x * blockDim.x + threadIdx.x; n < N; n += gridDim.x * blockDim.x) {
+    float s = 0.f;
+    for (int p = 0; p < b.parts[l]; ++p) s += b.part[l][(size_t)p * N + n];
+    b.db[l][n] = s;
+  }
 }
 
-// db[n] = sum_m dZ[m][n]
-__global__ void colsum_kernel(int M, int N, const float* __restrict__ dz, float* __restrict__ db) {
-  const int n = blockIdx.x * blockDim.x + threadIdx.x;
-  if (n >= N) return;
-  float s = 0.f;
-  for (int m = 0; m < M; ++m) s += dz[(long)m * N + n];
-  db[n] = s;
+// bound by HBM: 16 B read and 12 B written per parameter, four parameters per thread and step
+__device__ __forceinline__ void adam_one(float& p, float gv, float& m1, float& m2, float lr, float b1, float b2,
+                                         float eps, float c1, float c2) {
+  const float a = b1 * m1 + (1.f - b1) * gv;
+  const float b = b2 * m2 + (1.f - b2) * gv * gv;
+  m1 = a;
+  m2 = b;
+  p -= lr * (a / c1) / (sqrtf(b / c2) + eps);
 }
-
-__global__ void adam_kernel(long count, float* __restrict__ p, const float* __restrict__ gr, float* __restrict__ m1,
-                            float* __restrict__ m2, float lr, float b1, float b2, float eps, float c1, float c2) {
-  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < count; i += (long)gridDim.x * blockDim.x) {
-    const float gv = gr[i];
-    const float a = b1 * m1[i] + (1.f - b1) * gv;
-    const float b = b2 * m2[i] + (1.f - b2) * gv * gv;
-    m1[i] = a;
-    m2[i] = b;
-    p[i] -= lr * (a / c1) / (sqrtf(b / c2) + eps);
+__global__ void __launch_bounds__(256)
+adam_kernel(long count, float* __restrict__ p, const float* __restrict__ gr, float* __restrict__ m1,
+            float* __restrict__ m2, float lr, float b1, float b2, float eps, float c1, float c2) {
+  const long i = (blockIdx.x * (long)blockDim.x + threadIdx.x) * 4;
+  if (i + 3 < count) {
+    float4 pv = *reinterpret_cast<const float4*>(p + i), av = *reinterpret_cast<const float4*>(m1 + i),
+           bv = *reinterpret_cast<const float4*>(m2 + i);
+    const float4 gv = *reinterpret_cast<const float4*>(gr + i);
+    adam_one(pv.x, gv.x, av.x, bv.x, lr, b1, b2, eps, c1, c2);
+    adam_one(pv.y, gv.y, av.y, bv.y, lr, b1, b2, eps, c1, c2);
+    adam_one(pv.z, gv.z, av.z, bv.z, lr, b1, b2, eps, c1, c2);
+    adam_one(pv.w, gv.w, av.w, bv.w, lr, b1, b2, eps, c1, c2);
+    *reinterpret_cast<float4*>(p + i) = pv;
+    *reinterpret_cast<float4*>(m1 + i) = av;
+    *reinterpret_cast<float4*>(m2 + i) = bv;
+  } else {
+    for (long k = i; k < count; ++k) adam_one(p[k], gr[k], m1[k], m2[k], lr, b1, b2, eps, c1, c2);
   }
 }
 
@@ -216,10 +457,13 @@ struct df_mlp {
   float* m2 = nullptr;
   long nparam = 0;
   long off_w[4], off_b[4];
-  float* act[5] = {};        // act[0] = input copy, act[l] = layer-l output
-  float* dact = nullptr;     // scratch for dA / dZ (max width)
-  float* dact2 = nullptr;
-  float* partial = nullptr;
+  float* act[4] = {};        // act[l] = output of hidden layer l (l = 1, 2, 3)
+  unsigned char* actb[4] = {};  // BF16 atoms: the input (0) and the hidden layers' outputs
+  unsigned char* dzb[4] = {};   // BF16 atoms of dZ of layer l's output
+  unsigned char* wb[4] = {};    // BF16 atoms of W_l (l >= 1), left by the forward products of a gradient
+  float* part_col[4] = {};      // dZ's column sums per row quadrant (bias gradients)
+  float* part_loss = nullptr;
+  long loss_blocks = 0;         // capacity of part_loss
   int* d_timeout = nullptr;  // set by a tensor-core GEMM whose bounded wait gave up
   float* h_loss = nullptr;
   long step = 0;
@@ -243,64 +487,93 @@ df_status mfail(df_mlp* m, df_status s, const char* what, cudaError_t e = cudaSu
       return mfail((m), e__ == cudaErrorMemoryAllocation ? DF_ERR_OOM : DF_ERR_CUDA, (what), e__); \
   } while (0)
 
-// err: the handle's device flag a GEMM sets when a bounded tensor-core wait gave up
-cudaError_t gemm(cudaStream_t s, int* err, int M, int N, int K, const float* A, long sam, long sak, const float* B,
-                 long sbk, long sbn, float* C, long ldc, const float* bias, int act, int accumulate) {
-  static bool attr = false;
-  if (!attr) {
-    const cudaError_t e = cudaFuncSetAttribute((const void*)gemm_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               kGemmSmem);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
-  dim3 grid((N + kGn - 1) / kGn, (M + kGm - 1) / kGm);
-  gemm_tc_kernel<<<grid, kGemmThreads, kGemmSmem, s>>>(M, N, K, A, sam, sak, B, sbk, sbn, C, ldc, bias, act, accumulate,
-                                                       err);
+template <int TM, int TN, int KB, int NS, bool AMN, bool BMN, bool WF32>
+cudaError_t launch_gemm(cudaStream_t s, const GemmArgs& g) {
+  constexpr int smem = gemm_smem_bytes(TM, TN, KB, NS);
+  auto fn = gemm_tc_kernel<TM, TN, KB, NS, AMN, BMN, WF32>;
+  cudaError_t e = cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  const dim3 grid((g.M + TM - 1) / TM, (g.N + TN - 1) / TN);
+  fn<<<grid, kGemmThreads, smem, s>>>(g);
   return cudaGetLastError();
 }
 
-int blocks_for(long n) { return (int)std::min<long>(1024, (n + 255) / 256); }
+// forward and weight-gradient tiles: 128 columns, or 64 when 128 leave the
+// 152 SMs without a block each (the width-512 layers)
+bool wide_tiles(int M, int N) { return (long)((M + 127) / 128) * ((N + 127) / 128) >= 152; }
 
-df_status forward(df_mlp* m, const float* x, int B) {
-  M_CUDA(m, cudaMemcpyAsync(m->act[0], x, sizeof(float) * B * m->dims[0], cudaMemcpyDeviceToDevice, m->stream),
-         "copy input");
+int rg_of(long rows) { return (int)(pad128(rows) / 8); }
+bool vec4(const float* p, int ld) { return ((uintptr_t)p & 15) == 0 && ld % 4 == 0; }
+
+// y: the FP32 output [B][n_out], or with target (and y NULL) dZ of the loss
+df_status forward(df_mlp* m, const float* x, int B, float* y, const float* target, bool keep_w) {
+  const int rb = rg_of(m->max_batch);
+  const long chunks = pad128(B) * (pad128(m->dims[0]) / 8);
+  to_atoms_kernel<<<(int)std::min<long>(1024, (chunks + 255) / 256), 256, 0, m->stream>>>(B, m->dims[0], x, m->actb[0],
+                                                                                         rb);
+  M_CUDA(m, cudaGetLastError(), "input to BF16");
   for (int l = 0; l < 4; ++l) {
     const int in = m->dims[l], out = m->dims[l + 1];
-    M_CUDA(m, gemm(m->stream, m->d_timeout, B, out, in, m->act[l], in, 1, m->params + m->off_w[l], out, 1, m->act[l + 1], out,
-                   m->params + m->off_b[l], l < 3 ? 1 : 0, 0),
+    GemmArgs g{};
+    g.M = B; g.N = out; g.nkb = (in + 63) / 64;
+    g.A = m->actb[l]; g.a_rg = rb;
+    g.W = m->params + m->off_w[l]; g.kw = in; g.wvec = vec4(g.W, out);
+    if (keep_w && l > 0) { g.wsh = m->wb[l]; g.wsh_rg = rg_of(in); }
+    g.bias = m->params + m->off_b[l];
+    g.err = m->d_timeout;
+    if (l < 3) {
+      g.epi = kEpiTanh; g.C = m->act[l + 1]; g.Cb = m->actb[l + 1]; g.cb_rg = rb;
+    } else if (target) {
+      g.epi = kEpiLoss; g.aux = target; g.scale = 1.f / (float)((long)B * out);
+      g.Cb = m->dzb[3]; g.cb_rg = rb; g.part_col = m->part_col[3]; g.part_loss = m->part_loss;
+    } else {
+      g.epi = kEpiLinear; g.C = y;
+    }
+    M_CUDA(m, wide_tiles(B, out) ? (launch_gemm<128, 128, 1, 3, false, true, true>(m->stream, g))
+                                 : (launch_gemm<128, 64, 1, 4, false, true, true>(m->stream, g)),
            "forward GEMM");
   }
   return DF_OK;
 }
 
-df_status backward(df_mlp* m, const float* target, int B, float* loss_host) {
-  const int nout = m->dims[4];
-  const long count = (long)B * nout;
-  const int nb = blocks_for(count);
-  mse_grad_kernel<<<nb, 256, 0, m->stream>>>(count, m->act[4], target, m->dact, 1.f / (float)count, m->partial);
-  M_CUDA(m, cudaGetLastError(), "loss");
-  float* dz = m->dact;      // dZ of the current layer [B][out]
-  float* da = m->dact2;     // dA of the layer below
+df_status backward(df_mlp* m, int B, float* loss_host) {
+  const int rb = rg_of(m->max_batch);
+  BiasGrads bg{};
+  int nmax = 0;
   for (int l = 3; l >= 0; --l) {
     const int in = m->dims[l], out = m->dims[l + 1];
-    // dW_l[in][out] = A_{l}^T dZ   (M = in, N = out, K = B)
-    M_CUDA(m, gemm(m->stream, m->d_timeout, in, out, B, m->act[l], 1, in, dz, out, 1, m->grads + m->off_w[l], out, nullptr, 0, 0),
+    bg.part[l] = m->part_col[l];
+    bg.db[l] = m->grads + m->off_b[l];
+    bg.n[l] = out;
+    bg.parts[l] = 4 * (l == 3 ? (B + 127) / 128 : (B + 63) / 64);
+    nmax = std::max(nmax, out);
+    // dW_l[in][out] = A_l^T dZ_l   (M = in, N = out, K = B)
+    GemmArgs w{};
+    w.M = in; w.N = out; w.nkb = (B + 63) / 64;
+    w.A = m->actb[l]; w.a_rg = rb;
+    w.B = m->dzb[l]; w.b_rg = rb;
+    w.epi = kEpiStore; w.C = m->grads + m->off_w[l]; w.err = m->d_timeout;
+    M_CUDA(m, wide_tiles(in, out) ? (launch_gemm<128, 128, 1, 3, true, true, false>(m->stream, w))
+                                  : (launch_gemm<128, 64, 1, 4, true, true, false>(m->stream, w)),
            "weight gradient");
-    colsum_kernel<<<(out + 255) / 256, 256, 0, m->stream>>>(B, out, dz, m->grads + m->off_b[l]);
-    M_CUDA(m, cudaGetLastError(), "bias gradient");
     if (l == 0) break;
-    // dA_{l} [B][in] = dZ W_l^T   (M = B, N = in, K = out; B(k, n) = W[n][k])
-    M_CUDA(m, gemm(m->stream, m->d_timeout, B, in, out, dz, out, 1, m->params + m->off_w[l], 1, out, da, in, nullptr, 0, 0),
-           "activation gradient");
-    tanh_back_kernel<<<blocks_for((long)B * in), 256, 0, m->stream>>>((long)B * in, m->act[l], da);
-    M_CUDA(m, cudaGetLastError(), "tanh backward");
-    float* t = dz;
-    dz = da;
-    da = t;
+    // dZ_{l-1} = (dZ_l W_l^T) (1 - A_l^2)   (M = B, N = in, K = out)
+    GemmArgs d{};
+    d.M = B; d.N = in; d.nkb = (int)(pad128(out) / 64);
+    d.A = m->dzb[l]; d.a_rg = rb;
+    d.B = m->wb[l]; d.b_rg = rg_of(in);
+    d.epi = kEpiBack; d.aux = m->act[l];
+    d.Cb = m->dzb[l - 1]; d.cb_rg = rb; d.part_col = m->part_col[l - 1]; d.err = m->d_timeout;
+    M_CUDA(m, (launch_gemm<64, 16, 2, 8, false, false, false>(m->stream, d)), "activation gradient");
   }
+  bias_grad_kernel<<<dim3((nmax + 255) / 256, 4), 256, 0, m->stream>>>(bg);
+  M_CUDA(m, cudaGetLastError(), "bias gradients");
   if (loss_host) {
+    const int nout = m->dims[4];
+    const int tn = wide_tiles(B, nout) ? 128 : 64;
+    const long nb = (long)((B + 127) / 128) * ((nout + tn - 1) / tn);
     std::vector<float> part(nb);
-    M_CUDA(m, cudaMemcpyAsync(part.data(), m->partial, sizeof(float) * nb, cudaMemcpyDeviceToHost, m->stream),
+    M_CUDA(m, cudaMemcpyAsync(part.data(), m->part_loss, sizeof(float) * nb, cudaMemcpyDeviceToHost, m->stream),
            "loss copy");
     int timeout = 0;
     M_CUDA(m, cudaMemcpyAsync(&timeout, m->d_timeout, sizeof(int), cudaMemcpyDeviceToHost, m->stream), "flag copy");
@@ -308,7 +581,7 @@ df_status backward(df_mlp* m, const float* target, int B, float* loss_host) {
     if (timeout) return mfail(m, DF_ERR_TIMEOUT, "a tensor-core GEMM's completion wait gave up");
     double s = 0.0;
     for (float v : part) s += v;
-    *loss_host = (float)(s / (double)count);
+    *loss_host = (float)(s / (double)((long)B * nout));
   }
   return DF_OK;
 }
@@ -343,23 +616,33 @@ df_status df_mlp_create(df_mlp** out, int n_in, int width, int n_out, int max_ba
     std::uniform_real_distribution<float> U(-lim, lim);
     for (long i = 0; i < (long)d[l] * d[l + 1]; ++i) h[m->off_w[l] + i] = U(rng);
   }
-  int maxw = std::max(std::max(n_in, width), n_out);
   cudaError_t e;
   df_status st = DF_OK;
   if ((e = cudaMalloc(&m->params, sizeof(float) * o)) != cudaSuccess ||
       (e = cudaMalloc(&m->grads, sizeof(float) * o)) != cudaSuccess ||
       (e = cudaMalloc(&m->m1, sizeof(float) * o)) != cudaSuccess ||
       (e = cudaMalloc(&m->m2, sizeof(float) * o)) != cudaSuccess ||
-      (e = cudaMalloc(&m->dact, sizeof(float) * (long)max_batch * maxw)) != cudaSuccess ||
-      (e = cudaMalloc(&m->dact2, sizeof(float) * (long)max_batch * maxw)) != cudaSuccess ||
-      (e = cudaMalloc(&m->partial, sizeof(float) * 1024)) != cudaSuccess ||
       (e = cudaMalloc(&m->d_timeout, sizeof(int))) != cudaSuccess ||
       (e = cudaMemset(m->d_timeout, 0, sizeof(int))) != cudaSuccess) {
     st = mfail(m, DF_ERR_OOM, "cudaMalloc", e);
   }
-  for (int l = 0; l < 5 && st == DF_OK; ++l)
-    if ((e = cudaMalloc(&m->act[l], sizeof(float) * (long)max_batch * d[l])) != cudaSuccess)
+  const long pb = pad128(max_batch);
+  m->loss_blocks = pb / 128 * ((n_out + 63) / 64);
+  auto zalloc = [&](void** p, size_t bytes) {    // the atoms' padding stays zero
+    if (st != DF_OK) return;
+    if ((e = cudaMalloc(p, bytes)) != cudaSuccess || (e = cudaMemset(*p, 0, bytes)) != cudaSuccess)
       st = mfail(m, DF_ERR_OOM, "cudaMalloc activations", e);
+  };
+  for (int l = 0; l < 4; ++l) {
+    zalloc((void**)&m->actb[l], atoms_bytes(max_batch, d[l]));
+    zalloc((void**)&m->dzb[l], atoms_bytes(max_batch, d[l + 1]));
+    zalloc((void**)&m->part_col[l], sizeof(float) * (size_t)(pb / 64 * 4) * d[l + 1]);
+    if (l > 0) {
+      zalloc((void**)&m->act[l], sizeof(float) * (size_t)max_batch * d[l]);
+      zalloc((void**)&m->wb[l], atoms_bytes(d[l], d[l + 1]));
+    }
+  }
+  zalloc((void**)&m->part_loss, sizeof(float) * m->loss_blocks);
   if (st == DF_OK &&
       ((e = cudaMemcpy(m->params, h.data(), sizeof(float) * o, cudaMemcpyHostToDevice)) != cudaSuccess ||
        (e = cudaMemset(m->m1, 0, sizeof(float) * o)) != cudaSuccess ||
@@ -381,11 +664,15 @@ void df_mlp_destroy(df_mlp* m) {
   cudaFree(m->grads);
   cudaFree(m->m1);
   cudaFree(m->m2);
-  cudaFree(m->dact);
-  cudaFree(m->dact2);
-  cudaFree(m->partial);
+  cudaFree(m->part_loss);
   cudaFree(m->d_timeout);
-  for (auto* a : m->act) cudaFree(a);
+  for (int l = 0; l < 4; ++l) {
+    cudaFree(m->act[l]);
+    cudaFree(m->actb[l]);
+    cudaFree(m->dzb[l]);
+    cudaFree(m->wb[l]);
+    cudaFree(m->part_col[l]);
+  }
   delete m;
 }
 
@@ -397,25 +684,21 @@ df_status df_mlp_param_count(const df_mlp* m, long* count) {
 
 df_status df_mlp_forward(df_mlp* m, const float* x, int batch, float* y) {
   if (!m || !x || !y || batch < 1 || batch > m->max_batch) return DF_ERR_ARG;
-  df_status s = forward(m, x, batch);
-  if (s != DF_OK) return s;
-  M_CUDA(m, cudaMemcpyAsync(y, m->act[4], sizeof(float) * batch * m->dims[4], cudaMemcpyDeviceToDevice, m->stream),
-         "copy output");
-  return DF_OK;
+  return forward(m, x, batch, y, nullptr, false);
 }
 
 df_status df_mlp_gradients(df_mlp* m, const float* x, const float* target, int batch, float* loss_host) {
   if (!m || !x || !target || batch < 1 || batch > m->max_batch) return DF_ERR_ARG;
-  df_status s = forward(m, x, batch);
+  df_status s = forward(m, x, batch, nullptr, target, true);
   if (s != DF_OK) return s;
-  return backward(m, target, batch, loss_host);
+  return backward(m, batch, loss_host);
 }
 
 df_status df_mlp_adam_step(df_mlp* m, float lr, float beta1, float beta2, float eps) {
   if (!m) return DF_ERR_ARG;
   ++m->step;
   const float c1 = 1.f - std::pow(beta1, (float)m->step), c2 = 1.f - std::pow(beta2, (float)m->step);
-  adam_kernel<<<blocks_for(m->nparam), 256, 0, m->stream>>>(m->nparam, m->params, m->grads, m->m1, m->m2, lr, beta1,
+  adam_kernel<<<(unsigned)((m->nparam + 1023) / 1024), 256, 0, m->stream>>>(m->nparam, m->params, m->grads, m->m1, m->m2, lr, beta1,
                                                            beta2, eps, c1, c2);
   M_CUDA(m, cudaGetLastError(), "adam");
   return DF_OK;

@@ -114,3 +114,41 @@ def test_warm_start_cuts_passes(env):
     assert not any(r["fallback"] for r in rows)
     assert warm < cold
     assert err < 0.5
+
+
+@pytest.mark.parametrize("dims, batch, max_batch", [
+    ((1, 2, 2, 2, 1), 1, 1),                      # one element of every tile
+    ((65, 130, 130, 130, 129), 64, 64),           # one past a 64-block of k, one past a tile of n
+    ((137, 200, 200, 200, 1000), 130, 256),       # two row tiles, row strides of the output odd multiples of 4
+    ((64, 128, 128, 128, 19459), 5, 200),         # 128-column tiles, rows that are not 16-byte aligned
+])
+def test_products_at_tile_edges(env, dims, batch, max_batch):
+    """Forward and gradients against the oracle where the product tiles end: sizes one past a
+    64-block of the sum, one past a tile, and a smaller batch after a full one (the larger
+    batch's rows must not enter the sums over the batch).  Bounds: the oracle has the same BF16
+    operands, so FP32 against FP64 accumulation leaves sqrt(K) 2^-24 except where a hidden
+    value sits on a BF16 rounding boundary: one flip moves it by 2^-8."""
+    df, torch = env
+    net = df.MLP(dims[0], dims[-1], width=dims[1], max_batch=max_batch, seed=3)
+    rng = np.random.default_rng(7)
+    big = rng.normal(size=(max_batch, dims[0])).astype(np.float32) * 50
+    tbig = rng.normal(size=(max_batch, dims[-1])).astype(np.float32) * 50
+    net.gradients(torch.from_numpy(big).cuda(), torch.from_numpy(tbig).cuda())
+    x = rng.normal(size=(batch, dims[0])).astype(np.float32)
+    t = rng.normal(size=(batch, dims[-1])).astype(np.float32)
+    xd, td = torch.from_numpy(x).cuda(), torch.from_numpy(t).cuda()
+    p = net.params().astype(np.float64)
+    y = torch.empty((batch, dims[-1]), dtype=torch.float32, device="cuda")
+    net.forward(xd, y)
+    torch.cuda.synchronize()
+    assert nrel(y.cpu().numpy(), M.forward(p, dims, x, rounding=True)[-1]) < 5e-3
+    loss = net.gradients(xd, td)
+    g = net.grads()
+    ref_loss, ref = M.loss_and_grads(p, dims, x, t, rounding=True)
+    assert abs(loss - ref_loss) < 1e-3 * ref_loss
+    o = 0
+    for l in range(4):
+        nw = dims[l] * dims[l + 1]
+        for part in (slice(o, o + nw), slice(o + nw, o + nw + dims[l + 1])):
+            assert nrel(g[part], ref[part]) < 1e-2, (l, part)
+        o += nw + dims[l + 1]
