@@ -19,6 +19,7 @@
 
 #include "df_bse_dev.cuh"
 #include "df_fft_dev.cuh"
+#include "df_mixed64_dev.cuh"
 #include "df_mixed_dev.cuh"
 #include "df_mixed_large_dev.cuh"
 
@@ -154,7 +155,10 @@ __global__ void batch_setup_elem_kernel(const PointDev* __restrict__ pts, int p)
       P.gg_lo[idx] = make_float2((float)(t.x - (double)hx), (float)(t.y - (double)hy));
     }
   }
-  if (P.gdig)
+  if (P.gdig && mixed_pad(n) == 64)
+    gamma_digits_cols(n, 2 * P.dm.nb, P.gam, P.gdig, (blockIdx.x * blockDim.x + threadIdx.x) >> 5,
+                      (gridDim.x * blockDim.x) >> 5, threadIdx.x & 31);
+  else if (P.gdig)
     gamma_digits_rows(n, mixed_pad(n), 2 * P.dm.nb, P.gam, P.gdig, (blockIdx.x * blockDim.x + threadIdx.x) >> 5,
                       (gridDim.x * blockDim.x) >> 5, threadIdx.x & 31);
 }
@@ -261,24 +265,13 @@ __global__ void batch_wedge_scatter_kernel(const PointDev* __restrict__ pts) {
 }
 
 template <int NP>
-__global__ void __launch_bounds__(mixed_block_threads(NP), use_umma_residual(NP) ? 1 : 0)
+__global__ void __launch_bounds__(mixed_block_threads(NP))
 batch_bse_mixed_kernel(const PointDev* __restrict__ pts, const int* __restrict__ order, const long* __restrict__ start,
                        int nseg, int chunk, unsigned long long* __restrict__ counter, int* __restrict__ redo) {
   extern __shared__ __align__(1024) float2 smf[];
   __shared__ int piv_s[128];
   __shared__ unsigned long long item_s;
-  __shared__ uint64_t mbar_s[2];
-  __shared__ unsigned tslot_s;
   const MixedPtrs sp = mixed_ptrs(smf, NP, piv_s);
-  Tc05 tc{};
-  if constexpr (use_umma_residual(NP)) {
-    // the swizzled operand tiles need a 1024-aligned work area
-    if (smem_u32(sp.work) & 1023u) {
-      if (threadIdx.x == 0) atomicOr(pts[0].flags, kFlagTcLayout);
-      return;
-    }
-    tc05_setup(tc, mbar_s, &tslot_s);
-  }
   const long total = start[nseg];
   long cur = -1;                       // (point, channel, W) whose gamma digits are in shared memory
   for (;;) {
@@ -299,16 +292,62 @@ batch_bse_mixed_kernel(const PointDev* __restrict__ pts, const int* __restrict__
       const int rem = (int)(local - (long)c * per_ch);
       const int a = dm.a0 + rem / dm.N, q = rem - (a - dm.a0) * dm.N;
       const long key = (long)k * 256 + c * dm.nb + a;
-      if (use_umma_residual(NP) && (threadIdx.x >> 5) == mixed_compute_threads(NP) / 32)
-        mixed_producer(sp, &tc);                      // warp 8: the tensor-core MMAs
-      else
-        bse_mixed_system<NP>(dm, c, a, q, P.gam, P.gam_hi, P.gam_lo, P.gg_hi, P.gg_lo, P.lchi, P.lkc, P.flags, sp,
-                             P.gdig ? P.gdig + (size_t)(c * dm.nb + a) * gdig_bytes(NP) : nullptr, key != cur, &tc,
-                             batch_check(redo, order[k]));
+      bse_mixed_system<NP>(dm, c, a, q, P.gam, P.gam_hi, P.gam_lo, P.gg_hi, P.gg_lo, P.lchi, P.lkc, P.flags, sp,
+                           P.gdig ? P.gdig + (size_t)(c * dm.nb + a) * gdig_bytes(NP) : nullptr, key != cur,
+                           batch_check(redo, order[k]));
       cur = key;
     }
   }
-  if constexpr (use_umma_residual(NP)) tc05_teardown(tc, mixed_compute_threads(NP));
+}
+
+// orders 33-64: two ladders of one (point, channel, W) at a time per block.  A
+// block takes kBatch64Take chunks of systems at once (gamma's 98 KB of digits are loaded per
+// (point, channel, W), so a longer run of one plane loads them less often)
+constexpr int kBatch64Take = 8;
+__global__ void __launch_bounds__(kM64Threads, 1)
+batch_bse_mixed64_kernel(const PointDev* __restrict__ pts, const int* __restrict__ order,
+                         const long* __restrict__ start, int nseg, int chunk,
+                         unsigned long long* __restrict__ counter, int* __restrict__ redo) {
+  extern __shared__ __align__(1024) unsigned char sm64[];
+  __shared__ uint64_t mbar_s[2 * kM64Groups];
+  __shared__ unsigned tslot_s;
+  __shared__ unsigned long long item_s;
+  if (smem_u32(sm64) & 1023u) {                  // the swizzled operand tiles need 1024-byte alignment
+    if (threadIdx.x == 0) atomicOr(pts[0].flags, kFlagTcLayout);
+    return;
+  }
+  M64Block blk;
+  m64_setup(blk, sm64, mbar_s, &tslot_s);
+  const long total = start[nseg];
+  long cur = -1;                       // (point, channel, W) whose gamma digits are in shared memory
+  for (;;) {
+    __syncthreads();
+    if (threadIdx.x == 0) item_s = atomicAdd(counter, (unsigned long long)(kBatch64Take * chunk));
+    __syncthreads();
+    long s = (long)item_s;
+    if (s >= total) break;
+    const long last = min(s + (long)(kBatch64Take * chunk), total);
+    while (s < last) {
+      const int k = find_segment(start, nseg, s);
+      const PointDev& P = pts[order[k]];
+      const Dims& dm = P.ldm;
+      const long plane = (s - start[k]) / dm.N;    // (channel, view plane) of the point
+      const long base = start[k] + plane * dm.N, end = min(last, base + dm.N);
+      if (P.active) {
+        const int c = (int)(plane / dm.na), a = dm.a0 + (int)(plane % dm.na), key = c * dm.nb + a;
+        const long id = (long)k * 256 + key;
+        if (id != cur) m64_load_digits(blk, P.gdig + (size_t)key * kM64DigBytes);
+        cur = id;
+        const size_t mat = (size_t)key * dm.n_w * dm.n_w;
+        for (long x = s + blk.gr.g; x < end; x += kM64Groups)
+          m64_system(dm, c, a, (int)(x - base), P.gam_hi + mat, P.gam_lo + mat, P.gg_hi + mat, P.gg_lo + mat, P.lchi,
+                     P.lkc, P.flags, blk.gr, smem_u32(sm64), reinterpret_cast<const float*>(sm64 + kM64Gexp),
+                     batch_check(redo, order[k]));
+      }
+      s = end;
+    }
+  }
+  m64_teardown(blk);
 }
 
 // mixed ladders of order 64 < n <= 128 (the shared-memory Gauss-Jordan body),
@@ -363,7 +402,7 @@ MixedKernel mixed_kernel_of(int np) {
     case 8: return batch_bse_mixed_kernel<8>;
     case 16: return batch_bse_mixed_kernel<16>;
     case 32: return batch_bse_mixed_kernel<32>;
-    default: return batch_bse_mixed_kernel<64>;
+    default: return batch_bse_mixed64_kernel;
   }
 }
 
@@ -526,8 +565,8 @@ df_status configure_groups(df_batch* b) {
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, batch_bse_gj_kernel, g.threads, g.smem);
       g.grid = b->sms * std::max(1, per);
     } else if (g.mixed) {
-      g.threads = mixed_block_threads(g.np);
-      g.smem = sizeof(float2) * (size_t)mixed_layout(g.np).total;
+      g.threads = g.np == 64 ? kM64Threads : mixed_block_threads(g.np);
+      g.smem = g.np == 64 ? (size_t)kM64Smem : sizeof(float2) * (size_t)mixed_layout(g.np).total;
       B_CUDA(b, cudaFuncSetAttribute((const void*)mixed_kernel_of(g.np), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)g.smem),
              "mixed smem attribute");
@@ -691,8 +730,7 @@ df_status df_batch_init(df_batch** out, int npts, const df_point* pts, int preci
     total += align_up(sizeof(double) * (2 * dm.n_w + 4));
     total += align_up(sizeof(int) * 4);
     if (P.mixed) total += align_up(sizeof(float2) * nv) * 4;      // gam hi, lo; gg hi, lo
-    if (P.mixed && use_tc_residual(mixed_pad(dm.n_w)))
-      total += align_up((size_t)2 * dm.nb * gdig_bytes(mixed_pad(dm.n_w)));   // gamma's digits
+    if (P.mixed) total += align_up((size_t)2 * dm.nb * mixed_digit_bytes(mixed_pad(dm.n_w)));   // gamma's digits
     if (P.sym) {
       const size_t nw = (size_t)dm.nb * dm.n_w * P.n_orb;
       total += align_up(sizeof(double2) * nw) * 3;                // compact chi, kc (2)
@@ -734,8 +772,7 @@ df_status df_batch_init(df_batch** out, int npts, const df_point* pts, int preci
       P.gam_lo = (float2*)take(sizeof(float2) * nv);
       P.gg_hi = (float2*)take(sizeof(float2) * nv);
       P.gg_lo = (float2*)take(sizeof(float2) * nv);
-      if (use_tc_residual(mixed_pad(dm.n_w)))
-        P.gdig = (unsigned char*)take((size_t)2 * dm.nb * gdig_bytes(mixed_pad(dm.n_w)));
+      if (const size_t db = mixed_digit_bytes(mixed_pad(dm.n_w))) P.gdig = (unsigned char*)take((size_t)2 * dm.nb * db);
     }
     if (P.sym) {
       const size_t nw = (size_t)dm.nb * dm.n_w * P.n_orb;

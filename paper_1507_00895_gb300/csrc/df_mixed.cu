@@ -1,28 +1,8 @@
-// Mixed-precision ladder solves (DF_FP32_IR): Eq. lin_alg_inv factorised in
-// FP32 (complex64) and corrected once with an FP64-accurate residual.
-//
-// Per (q, W, channel) system, with D = 1 - gamma diag(chi~):
-//   1. LU with partial pivoting of D in FP32 on the augmented [D | gamma]
-//      (forward substitution of the n right-hand sides fused into the
-//      elimination), then back substitution: X0 ~ D^-1 gamma in FP32.
-//   2. R = gamma - D X0 = gamma - X0 + gamma (chi o X0), evaluated with
-//      gamma and chi~ split into FP32 (hi, lo) pairs, exact FP32 products
-//      (fma) and double-float (TwoSum) accumulation: ~48-bit accurate.
-//   3. E = D^-1 R with the same FP32 LU; diag Gamma = diag X0 + diag E in FP64.
-// One correction step leaves an error ~(kappa u32)^2 |Gamma| plus kappa times
-// the residual's own accuracy, i.e. FP64-level for the condition numbers of
-// the ladder matrices met here (up to ~1e6).
-//
-// Layout: the whole [D | RHS] lives in registers.  The block is a P x P
-// grid of threads, P = n_pad / 4; thread (tr, tc) owns rows tr + P i and
-// columns tc + P j (i, j < 4) of D and of the right-hand sides (2D cyclic,
-// so that the shrinking active part of the elimination stays balanced).
-// Row pivoting is implicit: rows never move; pivot rows are marked used and
-// their order is kept in piv[] (logical row k of the factorisation is
-// physical row piv[k]).  Matrices of order n < n_pad are padded with an
-// identity block (gamma = 0, chi~ = 0 there), which leaves the solution of
-// the first n rows unchanged.
-#include "df_mixed_dev.cuh"
+// Mixed-precision ladder solves (DF_FP32_IR) of one problem: the kernels around
+// the per-ladder bodies of df_mixed64_dev.cuh (orders 33-64, two ladders of
+// one (channel, W) at a time per block) and df_mixed_dev.cuh (orders up to 32),
+// gamma's words and digits, and the launchers.
+#include "df_mixed64_dev.cuh"
 
 namespace df {
 
@@ -49,10 +29,16 @@ __global__ void gamma_digits_kernel(int n, int np, int count, const double2* __r
                     (gridDim.x * blockDim.x) >> 5, threadIdx.x & 31);
 }
 
+__global__ void gamma_digits64_kernel(int n, int count, const double2* __restrict__ gam,
+                                      unsigned char* __restrict__ out) {
+  gamma_digits_cols(n, count, gam, out, (blockIdx.x * blockDim.x + threadIdx.x) >> 5, (gridDim.x * blockDim.x) >> 5,
+                    threadIdx.x & 31);
+}
+
 // One contiguous range of systems per block (so that consecutive systems
 // share (channel, W) and gamma's digits stay in shared memory).
 template <int NP>
-__global__ void __launch_bounds__(mixed_block_threads(NP), use_umma_residual(NP) ? 1 : 0)
+__global__ void __launch_bounds__(mixed_block_threads(NP))
 bse_mixed_kernel(Dims dm, int ch0, int nch, const double2* __restrict__ gam,
                  const float2* __restrict__ gam_hi, const float2* __restrict__ gam_lo,
                  const float2* __restrict__ gg_hi, const float2* __restrict__ gg_lo,
@@ -60,18 +46,7 @@ bse_mixed_kernel(Dims dm, int ch0, int nch, const double2* __restrict__ gam,
                  const unsigned char* __restrict__ gdig, int* __restrict__ flags, MixedCheck mc) {
   extern __shared__ __align__(1024) float2 smf[];
   __shared__ int piv_s[128];
-  __shared__ uint64_t mbar_s[2];
-  __shared__ unsigned tslot_s;
   const MixedPtrs sp = mixed_ptrs(smf, NP, piv_s);
-  Tc05 tc{};
-  if constexpr (use_umma_residual(NP)) {
-    // the swizzled operand tiles need a 1024-aligned work area
-    if (smem_u32(sp.work) & 1023u) {
-      if (threadIdx.x == 0) atomicOr(flags, kFlagTcLayout);
-      return;
-    }
-    tc05_setup(tc, mbar_s, &tslot_s);
-  }
   const int N = dm.N, nb = dm.nb, na = dm.na;
   const long systems = (long)nch * na * N;
   const long per = (systems + gridDim.x - 1) / gridDim.x;
@@ -82,14 +57,43 @@ bse_mixed_kernel(Dims dm, int ch0, int nch, const double2* __restrict__ gam,
     const int rem = (int)(sys - (long)(c - ch0) * na * N);
     const int a = dm.a0 + rem / N, q = rem - (a - dm.a0) * N;
     const int key = c * nb + a;
-    if (use_umma_residual(NP) && (threadIdx.x >> 5) == mixed_compute_threads(NP) / 32)
-      mixed_producer(sp, &tc);                        // warp 8: the tensor-core MMAs
-    else
-      bse_mixed_system<NP>(dm, c, a, q, gam, gam_hi, gam_lo, gg_hi, gg_lo, chi, kc, flags, sp,
-                           gdig ? gdig + (size_t)key * gdig_bytes(NP) : nullptr, key != cur, &tc, mc);
+    bse_mixed_system<NP>(dm, c, a, q, gam, gam_hi, gam_lo, gg_hi, gg_lo, chi, kc, flags, sp,
+                         gdig ? gdig + (size_t)key * gdig_bytes(NP) : nullptr, key != cur, mc);
     cur = key;
   }
-  if constexpr (use_umma_residual(NP)) tc05_teardown(tc, mixed_compute_threads(NP));
+}
+
+// Orders 33-64: one contiguous range of systems per block, split where
+// (channel, W) changes; the two groups of a block take its systems in turn.
+__global__ void __launch_bounds__(kM64Threads, 1)
+bse_mixed64_kernel(Dims dm, int ch0, int nch, const float2* __restrict__ gam_hi, const float2* __restrict__ gam_lo,
+                   const float2* __restrict__ gg_hi, const float2* __restrict__ gg_lo,
+                   const double2* __restrict__ chi, double2* __restrict__ kc, const unsigned char* __restrict__ gdig,
+                   int* __restrict__ flags, MixedCheck mc) {
+  extern __shared__ __align__(1024) unsigned char sm64[];
+  __shared__ uint64_t mbar_s[2 * kM64Groups];
+  __shared__ unsigned tslot_s;
+  if (smem_u32(sm64) & 1023u) {                  // the swizzled operand tiles need 1024-byte alignment
+    if (threadIdx.x == 0) atomicOr(flags, kFlagTcLayout);
+    return;
+  }
+  M64Block blk;
+  m64_setup(blk, sm64, mbar_s, &tslot_s);
+  const int N = dm.N, nb = dm.nb, na = dm.na;
+  const long systems = (long)nch * na * N;
+  const long s1 = systems * (blockIdx.x + 1) / gridDim.x;
+  long s = systems * blockIdx.x / gridDim.x;
+  while (s < s1) {
+    const long plane = s / N, end = min(s1, (plane + 1) * N);
+    const int c = ch0 + (int)(plane / na), a = dm.a0 + (int)(plane % na), key = c * nb + a;
+    m64_load_digits(blk, gdig + (size_t)key * kM64DigBytes);
+    const size_t mat = (size_t)key * dm.n_w * dm.n_w;
+    for (long x = s + blk.gr.g; x < end; x += kM64Groups)
+      m64_system(dm, c, a, (int)(x - plane * N), gam_hi + mat, gam_lo + mat, gg_hi + mat, gg_lo + mat, chi, kc, flags,
+                 blk.gr, smem_u32(sm64), reinterpret_cast<const float*>(sm64 + kM64Gexp), mc);
+    s = end;
+  }
+  m64_teardown(blk);
 }
 
 // Self-test of the bounded wait the tensor-core residual uses: one warp
@@ -129,7 +133,7 @@ bool mixed_supported(int n_w) { return mixed_np(n_w) <= 128; }
 // largest rho^2 and the hand-back list (count + 2 N_W N system indices)
 static size_t mixed_check_offset(const Dims& dm) {
   const int np = mixed_np(dm.n_w);
-  const size_t digits = use_tc_residual(np) ? (size_t)2 * dm.nb * gdig_bytes(np) : 0;
+  const size_t digits = (size_t)2 * dm.nb * mixed_digit_bytes(np);
   return ((size_t)4 * 2 * dm.nb * dm.n_w * dm.n_w * sizeof(float2) + digits + 15) & ~(size_t)15;
 }
 size_t mixed_tcr_offset(const Dims& dm) {
@@ -151,7 +155,7 @@ MixedCheck mixed_check(df_ctx* c) {
 
 static unsigned char* gdig_ptr(df_ctx* c) {
   const int np = mixed_np(c->dm.n_w);
-  if (!use_tc_residual(np)) return nullptr;
+  if (!mixed_digit_bytes(np)) return nullptr;
   return (unsigned char*)c->mixed_ws + (size_t)4 * 2 * c->dm.nb * c->dm.n_w * c->dm.n_w * sizeof(float2);
 }
 
@@ -165,7 +169,10 @@ cudaError_t launch_split_gamma(df_ctx* c, const double2* gg) {
   if (mixed_np(dm.n_w) > 64) return launch_split_gamma_t(c);   // slots 2, 3: gamma^T's words
   if (unsigned char* gd = gdig_ptr(c)) {
     const int np = mixed_np(dm.n_w), rows = 2 * dm.nb * np;
-    gamma_digits_kernel<<<(rows + 7) / 8, 256, 0, c->stream>>>(dm.n_w, np, 2 * dm.nb, c->gam, gd);
+    if (np == 64)
+      gamma_digits64_kernel<<<(rows + 7) / 8, 256, 0, c->stream>>>(dm.n_w, 2 * dm.nb, c->gam, gd);
+    else
+      gamma_digits_kernel<<<(rows + 7) / 8, 256, 0, c->stream>>>(dm.n_w, np, 2 * dm.nb, c->gam, gd);
     e = cudaGetLastError();
   }
   return e;
@@ -174,7 +181,7 @@ cudaError_t launch_split_gamma(df_ctx* c, const double2* gg) {
 template <int NP>
 static cudaError_t launch_bse_mixed_np(df_ctx* c, int channel_mask, int* flags) {
   const Dims& dm = c->dm;
-  constexpr int threads = mixed_block_threads(NP);   // + the producer warp at n_pad = 64
+  constexpr int threads = mixed_block_threads(NP);
   const size_t smem = sizeof(float2) * (size_t)mixed_layout(NP).total;
   cudaError_t e = cudaFuncSetAttribute((const void*)bse_mixed_kernel<NP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)smem);
@@ -206,6 +213,24 @@ static cudaError_t launch_bse_mixed_np(df_ctx* c, int channel_mask, int* flags) 
   return cudaSuccess;
 }
 
+// orders 33-64: one block of two ladder groups per SM
+static cudaError_t launch_bse_mixed64(df_ctx* c, int channel_mask, int* flags) {
+  const Dims& dm = c->dm;
+  cudaError_t e = cudaFuncSetAttribute((const void*)bse_mixed64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       kM64Smem);
+  if (e != cudaSuccess) return e;
+  int sms = 0;
+  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device)) != cudaSuccess) return e;
+  const size_t count = (size_t)2 * dm.nb * dm.n_w * dm.n_w;
+  const float2* hi = (const float2*)c->mixed_ws;
+  const MixedCheck mc = mixed_check(c);
+  const int nch = (channel_mask & 1) + ((channel_mask >> 1) & 1), ch0 = (channel_mask & 1) ? 0 : 1;
+  const long pairs = ((long)nch * dm.na * dm.N + kM64Groups - 1) / kM64Groups;
+  bse_mixed64_kernel<<<(int)(pairs < sms ? pairs : sms), kM64Threads, kM64Smem, c->stream>>>(
+      dm, ch0, nch, hi, hi + count, hi + 2 * count, hi + 3 * count, c->chi, c->kc, gdig_ptr(c), flags, mc);
+  return cudaGetLastError();
+}
+
 // the mixed-precision ladder solves of one df_bse call, then the FP64 LU over
 // the ladders whose predicted error exceeded the bound (none: its blocks exit
 // at once).  The caller zeroes the check words before (run_ladders).
@@ -215,7 +240,7 @@ cudaError_t launch_bse_mixed(df_ctx* c, int channel_mask, int* flags) {
     case 8: e = launch_bse_mixed_np<8>(c, channel_mask, flags); break;
     case 16: e = launch_bse_mixed_np<16>(c, channel_mask, flags); break;
     case 32: e = launch_bse_mixed_np<32>(c, channel_mask, flags); break;
-    case 64: e = launch_bse_mixed_np<64>(c, channel_mask, flags); break;
+    case 64: e = launch_bse_mixed64(c, channel_mask, flags); break;
     case 128: e = launch_bse_mixed_large(c, channel_mask, flags); break;   // df_mixed_large.cu
     default: return cudaErrorInvalidValue;
   }

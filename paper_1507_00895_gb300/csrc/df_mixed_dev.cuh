@@ -172,21 +172,13 @@ __device__ __forceinline__ void mma_bf16(float* d, const unsigned* a, unsigned b
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
-// ---- tcgen05 (5th-generation tensor core) helpers for the np = 64 residual ----
+// ---- tcgen05 (5th-generation tensor core) helpers ----
 // Operands are K-major bf16 tiles in shared memory with 128-byte rows in the
 // 128-byte swizzle (16-byte chunk c of row r at chunk c ^ (r & 7); 8-row groups
 // 1024 bytes apart, group base 1024-aligned) -- the layout swz() writes.  The
 // FP32 accumulators live in tensor memory (TMEM): row i of D in TMEM lane i,
 // column j in TMEM column (base + j).
-constexpr int kTmemCols = 512;      // two buffers of 8 weight groups x 32 columns
 constexpr unsigned kMbarSpin = 1u << 22;   // try_wait rounds before giving up
-
-struct Tc05 {
-  unsigned tmem;        // TMEM base address (lane 0, first allocated column)
-  uint64_t* mbar;       // completion barrier of the MMA batches
-  unsigned phase;       // parity of the next completion (the same in every thread)
-  uint64_t* fin;        // the tear-down's barrier: every queued MMA done before TMEM is freed
-};
 
 __device__ __forceinline__ unsigned smem_u32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
 
@@ -243,44 +235,6 @@ __device__ __forceinline__ void tmem_ld16(unsigned taddr, float* v) {
 #pragma unroll
   for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[j]);
 }
-// block-level set-up / tear-down (all threads call; warp 0 owns the TMEM allocation);
-// mbar: two barriers (the MMA batches', the tear-down's)
-__device__ __forceinline__ void tc05_setup(Tc05& tc, uint64_t* mbar, unsigned* tslot) {
-  if ((threadIdx.x >> 5) == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tslot)),
-                 "n"(kTmemCols)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-  }
-  if (threadIdx.x == 0) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(mbar)) : "memory");
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(mbar + 1)) : "memory");
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  tc05_fence_before();
-  __syncthreads();
-  tc05_fence_after();
-  tc.tmem = *tslot;
-  tc.mbar = mbar;
-  tc.phase = 0;
-  tc.fin = mbar + 1;
-}
-// issuer: the thread that issued the block's MMAs.  Its one more commit, to
-// the tear-down's barrier, completes once every MMA it queued has (also after
-// a completion wait that gave up earlier); the wait for it is bounded.
-__device__ __forceinline__ void tc05_teardown(const Tc05& tc, int issuer) {
-  if ((int)threadIdx.x == issuer) {
-    tc05_fence_before();
-    umma_commit(tc.fin);
-    mbar_wait(tc.fin, 0u);
-  }
-  tc05_fence_before();
-  __syncthreads();
-  tc05_fence_after();
-  if ((threadIdx.x >> 5) == 0)
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tc.tmem), "n"(kTmemCols) : "memory");
-}
-
 __device__ __forceinline__ void dd_add(float& hi, float& lo, float v) {
   float s, e;
   two_sum(hi, v, s, e);
@@ -385,80 +339,6 @@ __device__ __forceinline__ void gj_panel(float2* pan, int k0, int lane, unsigned
   }
 }
 
-// The same b = 8 steps for np = 64 on two warps (threads 0..63), one row per
-// lane: each warp's best unused row (its warp max) goes to cand / ckey, a
-// 64-thread named barrier, then both warps take the better of the two.  The
-// candidate slots alternate between steps, so one barrier per step suffices.
-__device__ __forceinline__ void gj_panel2(float2* pan, int k0, int w, int lane, unsigned& used0, int* piv_s,
-                                          int* rowstep, int* flags, float4* cand, unsigned* ckey) {
-  constexpr int np = 64;
-  const int r = 32 * w + lane;
-  float2 pv[kPanel];
-#pragma unroll
-  for (int c2 = 0; c2 < kPanel; ++c2) pv[c2] = pan[r * kPanelLd + c2];
-  int pivs[kPanel];
-  bool sing = false;
-#pragma unroll
-  for (int i = 0; i < kPanel; ++i) {
-    const float m0 = fabsf(pv[i].x) + fabsf(pv[i].y);
-    const unsigned key = (used0 & 1u) ? 0u : ((__float_as_uint(m0) & ~0x7Fu) | (unsigned)(127 - r));
-    const unsigned kw = __reduce_max_sync(0xffffffffu, key);
-    const int par = i & 1;
-    if (key == kw && kw != 0u) {
-      float4* cs = cand + (par * 2 + w) * (kPanel / 2);
-#pragma unroll
-      for (int c4 = 0; c4 < kPanel / 2; ++c4)
-        cs[c4] = make_float4(pv[2 * c4].x, pv[2 * c4].y, pv[2 * c4 + 1].x, pv[2 * c4 + 1].y);
-    }
-    if (lane == 0) ckey[par * 2 + w] = kw;
-    asm volatile("bar.sync 1, 64;" ::: "memory");
-    const unsigned ka = ckey[par * 2], kb = ckey[par * 2 + 1];
-    const int wb = kb > ka ? 1 : 0;
-    const unsigned kbest = kb > ka ? kb : ka;
-    int p = 127 - (int)(kbest & 0x7Fu);
-    const float bm = __uint_as_float(kbest & ~0x7Fu);
-    const bool singular = !(bm > 0.f) || p >= np;
-    if (p >= np) p = 0;
-    const float4* cb = cand + (par * 2 + wb) * (kPanel / 2);
-    float2 u[kPanel];
-#pragma unroll
-    for (int c4 = 0; c4 < kPanel / 2; ++c4) {
-      const float4 q = cb[c4];
-      u[2 * c4] = make_float2(q.x, q.y);
-      u[2 * c4 + 1] = make_float2(q.z, q.w);
-    }
-    float2 ainv = make_float2(0.f, 0.f);
-    if (!singular) {
-      const float2 z = u[i];
-      const float d = __fdividef(1.f, fmaf(z.x, z.x, z.y * z.y));
-      ainv = make_float2(z.x * d, -z.y * d);
-    }
-#pragma unroll
-    for (int c2 = 0; c2 < kPanel; ++c2) u[c2] = (c2 == i) ? ainv : cmulf(u[c2], ainv);
-    pivs[i] = p;
-    sing |= singular;
-    const bool isp = (r == p);
-    used0 |= isp ? 1u : 0u;
-    const float2 m = pv[i];
-#pragma unroll
-    for (int c2 = 0; c2 < kPanel; ++c2) {
-      const float2 base = (c2 == i) ? make_float2(0.f, 0.f) : pv[c2];
-      const float2 e = cfmsf(m, u[c2], base);
-      pv[c2] = isp ? u[c2] : e;
-    }
-  }
-#pragma unroll
-  for (int c2 = 0; c2 < kPanel; ++c2) pan[r * kPanelLd + c2] = pv[c2];
-  if (w == 0 && lane == 0) {
-#pragma unroll
-    for (int i = 0; i < kPanel; ++i) {
-      piv_s[k0 + i] = pivs[i];
-      rowstep[pivs[i]] = k0 + i;
-    }
-    if (sing) atomicOr(flags, 1);
-  }
-}
-
 // bf16 bit pattern of the signed digit (sign16 = 0 or 0x8000, 0 <= d < 256),
 // exact and without a conversion unit: the float 2^23 + d minus 2^23
 __device__ __forceinline__ unsigned bf16_digit(unsigned d, unsigned sign16) {
@@ -558,21 +438,14 @@ struct MixedSmem {
   int x0, chih, chil, invu, x0d, chi64, work, gt_h, gt_l, yh, yl, total;
 };
 
-__host__ __device__ constexpr bool use_tc_residual(int np) { return np == 32 || np == 64; }
-// np = 64: the digit products run as tcgen05 MMAs (M = 128 = [Zr; Zi] rows)
-__host__ __device__ constexpr bool use_umma_residual(int np) { return np == 64; }
-// offset of the Y digits in the work area (1024-aligned for the tcgen05 operands)
-__host__ __device__ constexpr int xs_offset(int np) {
-  return use_umma_residual(np) ? ((gdig_bytes(np) + 1023) & ~1023) : gdig_bytes(np);
-}
-// bytes of the tensor-core residual's work area (n_pad in {32, 64}): the
+__host__ __device__ constexpr bool use_tc_residual(int np) { return np == 32; }
+// offset of the Y digits in the work area
+__host__ __device__ constexpr int xs_offset(int np) { return gdig_bytes(np); }
+// bytes of the tensor-core residual's work area (n_pad = 32): the
 // gamma digits of the current (channel, W) (kept across systems), then the
 // Y digits of one column block and their column exponents
 __host__ __device__ constexpr int tc_work_bytes(int np) {
-  // np = 64 adds a second column-exponent slot, the re/im exchange
-  // [2][np][kCB + 1] (double-float) and per-warp column exponents [8][kCB]
-  return xs_offset(np) + 2 * kSlices * 2 * kCB * 64 + 4 * kCB +
-         (use_umma_residual(np) ? 4 * kCB + 2 * np * (kCB + 1) * 8 + 4 * 8 * kCB : 0);
+  return xs_offset(np) + 2 * kSlices * 2 * kCB * 64 + 4 * kCB;
 }
 
 // row stride of X0 / R in shared memory (float2): np + 1 spreads a column
@@ -588,7 +461,6 @@ __host__ __device__ inline MixedSmem mixed_layout(int np) {
   L.invu = o; o += np;
   L.x0d = o;  o += np;             // diag X0 (FP32)
   L.chi64 = o; o += 2 * np;        // chi~ in FP64 (double2 = two float2 slots)
-  if (use_umma_residual(np)) o = (o + 127) & ~127;   // tcgen05 operand tiles: 1024-byte aligned
   L.work = o;                      // residual work area (one of the two layouts below)
   // SIMT residual: gamma tiles and Y = chi o X0 as double-float
   L.gt_h = o;
@@ -599,8 +471,7 @@ __host__ __device__ inline MixedSmem mixed_layout(int np) {
   const int tc = (tc_work_bytes(np) + 7) / 8;
   // Gauss-Jordan panels [2][np][kPanelLd] and pivot rows [kPanel][2 np]; with
   // the tensor-core residual they sit in the Y-digit area, past gamma's digits
-  const int gj = (use_tc_residual(np) ? gdig_bytes(np) / 8 : 0) + 2 * np * kPanelLd + kPanel * 2 * np +
-                 2 * 2 * kPanel + 2;   // + the two-warp panel's candidate rows and keys
+  const int gj = (use_tc_residual(np) ? gdig_bytes(np) / 8 : 0) + 2 * np * kPanelLd + kPanel * 2 * np;
   const int res = use_tc_residual(np) ? tc : simt;
   o += res > gj ? res : gj;
   L.total = o;
@@ -633,30 +504,7 @@ __device__ __forceinline__ MixedPtrs mixed_ptrs(float2* smf, int np, int* piv_s)
   return m;
 }
 
-// n_pad = 64 runs 9 warps: warps 0-7 compute (their own 256-thread barrier),
-// warp 8 issues the tensor-core MMAs.  Per column block the compute warps
-// arrive on barrier kBarHandoff once the block's Y digits are in shared
-// memory; the producer waits there, issues the block's MMAs and commits them
-// to the mbarrier the compute warps wait on before they read TMEM.
-constexpr int kBarCompute = 2;    // named barrier of the 256 compute threads
-constexpr int kBarHandoff = 3;    // compute warps -> producer warp (288 threads)
-__host__ __device__ constexpr int mixed_compute_threads(int np) { return (np / kTile) * (np / kTile); }
-__host__ __device__ constexpr int mixed_block_threads(int np) {
-  return mixed_compute_threads(np) + (use_umma_residual(np) ? 32 : 0);
-}
-template <int NP>
-__device__ __forceinline__ void block_sync() {
-  if constexpr (use_umma_residual(NP))
-    asm volatile("bar.sync %0, %1;" ::"n"(kBarCompute), "n"(mixed_compute_threads(NP)) : "memory");
-  else
-    __syncthreads();
-}
-__device__ __forceinline__ void handoff_arrive() {
-  asm volatile("bar.arrive %0, %1;" ::"n"(kBarHandoff), "n"(mixed_compute_threads(64) + 32) : "memory");
-}
-__device__ __forceinline__ void handoff_wait() {
-  asm volatile("bar.sync %0, %1;" ::"n"(kBarHandoff), "n"(mixed_compute_threads(64) + 32) : "memory");
-}
+__host__ __device__ constexpr int mixed_block_threads(int np) { return (np / kTile) * (np / kTile); }
 
 // One (q, W, channel) ladder in mixed precision; all P*P threads of the
 // block (P = np / 4) must call it.  Writes kc[c][a][:][q].
@@ -670,10 +518,10 @@ __device__ __forceinline__ void bse_mixed_system(const Dims& dm, int c, int a, i
                                                  const double2* __restrict__ chi, double2* __restrict__ kc,
                                                  int* __restrict__ flags, const MixedPtrs& sp,
                                                  const unsigned char* __restrict__ gdig, bool reload,
-                                                 Tc05* umma, const MixedCheck& mc) {
+                                                 const MixedCheck& mc) {
   const int n = dm.n_w, N = dm.N, nb = dm.nb;
   constexpr int np = NP, P = NP / kTile;
-  constexpr int kThr = mixed_compute_threads(NP);       // threads taking part (the producer warp does not)
+  constexpr int kThr = mixed_block_threads(NP);       // threads taking part (the producer warp does not)
   constexpr int ld = x0_ld(NP);
   float2* X0s = sp.X0s;
   float2* chih = sp.chih;
@@ -697,7 +545,6 @@ __device__ __forceinline__ void bse_mixed_system(const Dims& dm, int c, int a, i
       const uint4* src = reinterpret_cast<const uint4*>(gdig);
       uint4* dst = reinterpret_cast<uint4*>(sp.work);
       for (int i = t; i < gdig_bytes(NP) / 16; i += kThr) dst[i] = __ldg(src + i);
-      if constexpr (use_umma_residual(NP)) fence_async_smem();
     }
   }
   for (int i = t; i < np; i += kThr) {
@@ -707,7 +554,7 @@ __device__ __forceinline__ void bse_mixed_system(const Dims& dm, int c, int a, i
     chil[i] = make_float2((float)(x.x - (double)hx), (float)(x.y - (double)hy));
     sp.chi64[i] = x;
   }
-  block_sync<NP>();
+  __syncthreads();
 
   // ---- load [D | gamma] (FP32) into registers ----
   float2 A[kTile][2 * kTile];
@@ -737,8 +584,7 @@ __device__ __forceinline__ void bse_mixed_system(const Dims& dm, int c, int a, i
   // The b GJ steps of a panel change every other column j by a rank-b
   // update, A[:, j] += W A[piv, j], where W = (panel after its own in-place
   // GJ steps) - (unit columns at the pivot rows).  Per panel: (1) the owners
-  // of the panel columns copy them to pan; (2) warp 0 (warps 0 and 1 for
-  // np = 64, one row per lane) runs the b steps on pan in registers (pivot =
+  // of the panel columns copy them to pan; (2) warp 0 runs the b steps on pan in registers (pivot =
   // max of a (|a| bits, ~row) key); (3) the pivot rows' current values go to
   // prs; (4) every thread applies the rank-b update to its whole tile, then
   // the panel columns take the panel's new values (their updated ones are
@@ -750,8 +596,6 @@ __device__ __forceinline__ void bse_mixed_system(const Dims& dm, int c, int a, i
   constexpr int pb = P < kPanel ? P : kPanel;        // panel width b
   float2* panbuf = reinterpret_cast<float2*>(sp.work + (use_tc_residual(NP) ? gdig_bytes(NP) : 0));   // [2][np][kPanelLd]
   float2* prs = panbuf + 2 * np * kPanelLd;                      // [kPanel][2 np]
-  float4* cand = reinterpret_cast<float4*>(prs + kPanel * 2 * np);  // two-warp panel: [2][2][kPanel / 2]
-  unsigned* ckey = reinterpret_cast<unsigned*>(cand + 2 * kPanel);   // [2][2]
   int* rowstep = reinterpret_cast<int*>(invu);                   // pivot step of each row, -1 if none
   for (int i = t; i < np; i += kThr) rowstep[i] = -1;
   unsigned used0 = 0;                                            // panel warps: their rows already pivots
@@ -772,14 +616,10 @@ __device__ __forceinline__ void bse_mixed_system(const Dims& dm, int c, int a, i
         pan[(tr + P * ii) * kPanelLd + (tc - kc)] = v;
       }
     }
-    block_sync<NP>();
-    // (2) b GJ steps on the panel: warps 0 and 1 for np = 64, else warp 0
-    if constexpr (NP == 64) {
-      if (warp < 2) gj_panel2(pan, k0, warp, lane, used0, piv_s, rowstep, flags, cand, ckey);
-    } else {
-      if (warp == 0) gj_panel<NP>(pan, k0, lane, used0, piv_s, rowstep, flags);
-    }
-    block_sync<NP>();
+    __syncthreads();
+    // (2) b GJ steps on the panel: warp 0
+    if (warp == 0) gj_panel<NP>(pan, k0, lane, used0, piv_s, rowstep, flags);
+    __syncthreads();
     // (3) current values of the pivot rows
 #pragma unroll
     for (int ii = 0; ii < kTile; ++ii) {
@@ -792,7 +632,7 @@ __device__ __forceinline__ void bse_mixed_system(const Dims& dm, int c, int a, i
         }
       }
     }
-    block_sync<NP>();
+    __syncthreads();
     // (4) rank-b update (the panel columns too: they take their new values after)
     for (int l = 0; l < pb; ++l) {
       const int pl = piv_s[k0 + l];
@@ -824,7 +664,7 @@ __device__ __forceinline__ void bse_mixed_system(const Dims& dm, int c, int a, i
       }
     }
   }
-  block_sync<NP>();
+  __syncthreads();
 #pragma unroll
   for (int ii = 0; ii < kTile; ++ii) rowpos[ii] = rowstep[tr + P * ii];
   // X0 in logical row order: row r of the sweep is X0 row rowpos (its pivot step)
@@ -835,173 +675,9 @@ __device__ __forceinline__ void bse_mixed_system(const Dims& dm, int c, int a, i
       for (int jj = 0; jj < kTile; ++jj) X0s[rowpos[ii] * ld + tc + P * jj] = A[ii][kTile + jj];
     }
   }
-  block_sync<NP>();
+  __syncthreads();
   for (int j = t; j < np; j += kThr) x0d[j] = X0s[j * ld + j];
-  if constexpr (use_umma_residual(NP)) {
-    // ---- residual R = gamma - X0 + gamma Y with tcgen05, Y = diag(chi~) X0 ----
-    // gamma's digits (8 signed base-128 digits relative to per-row powers of
-    // two, cut once per input upload) are in zs / rowe; Y is formed in
-    // double-float and cut the same way relative to per-column powers of two,
-    // kCB columns at a time.  For each gamma slice sa one MMA per K step of
-    // 16: A = [Zr; Zi] of slice sa (M = 128), B = the Y slices 0 .. 7 - sa
-    // stacked along N (32 rows each: the block's Yr then Yi columns), D at
-    // TMEM column 32 sa, so that Y slice sb lands in accumulator d = sa + sb
-    // (weight 2^-7(d+2)), columns 32 d .. 32 d + 31 = [Yr | Yi]; lanes 0-63
-    // hold the Zr rows, 64-127 the Zi rows.  Every accumulator is exact (<= 8
-    // pairs x 64 x 127^2 < 2^23), and the pairs with weight < 2^-63 are never
-    // formed.  Column block b's MMAs run in TMEM buffer b & 1 while block
-    // b - 1 is folded and assembled.
-    __nv_bfloat16* zs = reinterpret_cast<__nv_bfloat16*>(sp.work);                       // [kSlices][2][np][64]
-    const int* rowe = reinterpret_cast<const int*>(zs + (size_t)kSlices * 2 * np * 64);   // [np]
-    __nv_bfloat16* xs = reinterpret_cast<__nv_bfloat16*>(sp.work + xs_offset(NP));       // [kSlices][2][kCB][64]
-    int* cole2 = reinterpret_cast<int*>(xs + (size_t)kSlices * 2 * kCB * 64);            // [2][kCB]
-    float2* E = reinterpret_cast<float2*>(cole2 + 2 * kCB);                              // [2][np][kCB + 1]
-    int* cw = reinterpret_cast<int*>(E + 2 * np * (kCB + 1));                            // [8][kCB]
-    unsigned* xw = reinterpret_cast<unsigned*>(xs);
-    const int warp = t >> 5, lane = t & 31;
-    const int yc = t & (kCB - 1), yp = t >> 4;          // Y map: column yc, rows 2 yp (+1) (+32)
-    // fold of column block bb (TMEM buffer bb & 1) and R = gamma - X0 + S for it
-    auto finish = [&](int bb) {
-      const int* ce = cole2 + (bb & 1) * kCB;
-      // gamma (hi, lo) of this thread's four R entries, loaded ahead of the fold
-      float2 ghv[4], glv[4];
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const int row = yp + 16 * k, j = bb * kCB + yc;
-        const bool in = (row < n && j < n);
-        ghv[k] = in ? Gh[row * n + j] : make_float2(0.f, 0.f);
-        glv[k] = in ? Gl[row * n + j] : make_float2(0.f, 0.f);
-      }
-      // warp w reads lane quadrant q = w % 4 (gamma row i; Zr or Zi) and column
-      // half h = w / 4 (Yr or Yi) of the 8 accumulators.  Weights 2^-7d for
-      // d = 4..7 are summed in FP32 (Horner; their sum is < 2^-4.9 of the
-      // d = 0 scale, rounding error < 2^-27 of it), d = 0..3 in double-float.
-      const int qd = warp & 3, h = warp >> 2;
-      const int i = ((qd & 1) << 5) + lane;
-      const bool zi = qd >= 2;
-      const unsigned tl = umma->tmem + ((unsigned)(32 * qd) << 16) + (unsigned)(256 * (bb & 1) + 16 * h);
-      float fh[kCB], fl[kCB];
-      {
-        float v[kCB];
-        tmem_ld16(tl + 32 * 7, fh);
-#pragma unroll
-        for (int d = 6; d >= 4; --d) {
-          tmem_ld16(tl + 32 * d, v);
-#pragma unroll
-          for (int c2 = 0; c2 < kCB; ++c2) fh[c2] = fmaf(fh[c2], 0.0078125f, v[c2]);
-        }
-#pragma unroll
-        for (int c2 = 0; c2 < kCB; ++c2) {
-          fh[c2] *= 3.7252902984619141e-09f;      // 2^-28
-          fl[c2] = 0.f;
-        }
-#pragma unroll
-        for (int d = 3; d >= 0; --d) {
-          tmem_ld16(tl + 32 * d, v);
-          const float sc = __int_as_float((127 - 7 * d) << 23);     // 2^-7d
-#pragma unroll
-          for (int c2 = 0; c2 < kCB; ++c2) dd_add(fh[c2], fl[c2], v[c2] * sc);
-        }
-      }
-      tc05_fence_before();
-      // scale by 2^(e_i + e_j - 14); the Zi rows' parts go to E first (ZiYi
-      // negated: it enters the real part with a minus), then the Zr rows add
-      // theirs: E[0] = S real, E[1] = S imaginary, row stride kCB + 1
-      const int ei = rowe[i];
-#pragma unroll
-      for (int c2 = 0; c2 < kCB; ++c2) {
-        const int ej = ce[c2];
-        const float w = (ei > -1000 && ej > -1000) ? pow2f(ei + ej - 14) : 0.f;
-        fh[c2] *= w;
-        fl[c2] *= w;
-      }
-      if (zi) {
-        const float sg = h ? -1.f : 1.f;
-        float2* Eo = E + (1 - h) * np * (kCB + 1) + i * (kCB + 1);   // ZiYr -> imaginary, ZiYi -> real
-#pragma unroll
-        for (int c2 = 0; c2 < kCB; ++c2) Eo[c2] = make_float2(sg * fh[c2], sg * fl[c2]);
-      }
-      block_sync<NP>();
-      if (!zi) {
-        float2* Eo = E + h * np * (kCB + 1) + i * (kCB + 1);         // ZrYr -> real, ZrYi -> imaginary
-#pragma unroll
-        for (int c2 = 0; c2 < kCB; ++c2) {
-          const float2 o = Eo[c2];
-          float sh, se;
-          two_sum(fh[c2], o.x, sh, se);
-          Eo[c2] = make_float2(sh, se + (fl[c2] + o.y));
-        }
-      }
-      block_sync<NP>();
-      // R = gamma - X0 + S in double-float (it cancels to ~u32 |gamma|)
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const int row = yp + 16 * k, j = bb * kCB + yc;
-        const float2 x = X0s[row * ld + j];
-        const float2 sr = E[row * (kCB + 1) + yc], si = E[np * (kCB + 1) + row * (kCB + 1) + yc];
-        float re = ghv[k].x, rl = glv[k].x, im = ghv[k].y, il = glv[k].y;
-        df_add(re, rl, -x.x);
-        df_add(re, rl, sr.x);
-        df_add(im, il, -x.y);
-        df_add(im, il, si.x);
-        X0s[row * ld + j] = make_float2(re + (rl + sr.y), im + (il + si.y));   // R replaces X0
-      }
-    };
-    for (int b = 0; b < np / kCB; ++b) {
-      block_sync<NP>();
-      // Y = chi~ o X0 in double-float for rows 2 yp, 2 yp + 1, 2 yp + 32, 2 yp + 33
-      // of column yc; its column exponent e (|Y| < 2^e, -1000 for a zero
-      // column): the thread's max, the warp's two row groups, the 8 warps
-      float y[4][4];
-      float m = 0.f;
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const int l = 2 * yp + (k & 1) + 32 * (k >> 1);
-        const float2 x = X0s[l * ld + b * kCB + yc];
-        y[k][0] = y[k][1] = y[k][2] = y[k][3] = 0.f;
-        cdf_fma(y[k][0], y[k][1], y[k][2], y[k][3], chih[l], chil[l], x, make_float2(0.f, 0.f));
-        m = fmaxf(m, fmaxf(fabsf(y[k][0]), fabsf(y[k][2])));
-      }
-      m *= 1.0001f;
-      int e = m > 0.f ? exp_bound_f32(m) : -1000;
-      e = max(e, __shfl_xor_sync(0xffffffffu, e, 16));
-      if (lane < kCB) cw[warp * kCB + lane] = e;
-      block_sync<NP>();
-      int ecol = cw[yc];
-#pragma unroll
-      for (int w2 = 1; w2 < 8; ++w2) ecol = max(ecol, cw[w2 * kCB + yc]);
-      if (t < kCB) cole2[(b & 1) * kCB + t] = ecol;
-      // digits of the two row pairs, two rows per 32-bit word
-#pragma unroll
-      for (int pr = 0; pr < 2; ++pr) {
-        unsigned w0[kSlices], w1[kSlices], v0[kSlices], v1[kSlices];
-        if (ecol > -1000) {
-          digits_pair_f(y[2 * pr][0], y[2 * pr][1], ecol, w0);
-          digits_pair_f(y[2 * pr][2], y[2 * pr][3], ecol, w1);
-          digits_pair_f(y[2 * pr + 1][0], y[2 * pr + 1][1], ecol, v0);
-          digits_pair_f(y[2 * pr + 1][2], y[2 * pr + 1][3], ecol, v1);
-        } else {
-#pragma unroll
-          for (int s2 = 0; s2 < kSlices; ++s2) w0[s2] = w1[s2] = v0[s2] = v1[s2] = 0u;
-        }
-        const int wo = swz(yc, 2 * yp + 32 * pr) >> 1;
-#pragma unroll
-        for (int s2 = 0; s2 < kSlices; ++s2) {
-          xw[(s2 * 2 + 0) * kCB * 32 + wo] = pack_bf16_hi(w0[s2], v0[s2]);
-          xw[(s2 * 2 + 1) * kCB * 32 + wo] = pack_bf16_hi(w1[s2], v1[s2]);
-        }
-      }
-      fence_async_smem();
-      tc05_fence_before();
-      handoff_arrive();                                 // the producer warp issues block b's MMAs
-      if (b > 0) finish(b - 1);
-      if (!mbar_wait(umma->mbar, umma->phase) && t == 0) atomicOr(flags, kFlagTcTimeout);
-      umma->phase ^= 1;
-      tc05_fence_after();
-    }
-    finish(np / kCB - 1);
-    block_sync<NP>();
-  } else if constexpr (use_tc_residual(NP)) {
+  if constexpr (use_tc_residual(NP)) {
     // ---- residual R = gamma - X0 + gamma Y on the tensor cores, Y = diag(chi~) X0 ----
     // gamma's digits (cut once per input upload: 8 signed base-128 digits
     // relative to per-row powers of two) are in zs / rowe; Y is formed in
@@ -1019,9 +695,9 @@ __device__ __forceinline__ void bse_mixed_system(const Dims& dm, int c, int a, i
     const int nwarp = nthr >> 5;
     const int tiles = (np / 16) * (kCB / 8);
     for (int b = 0; b < np / kCB; ++b) {
-      block_sync<NP>();
+      __syncthreads();
       for (int c2 = t; c2 < kCB; c2 += nthr) cole[c2] = -1000;
-      block_sync<NP>();
+      __syncthreads();
       // lanes take consecutive columns of a row of X0 (no bank conflicts)
       for (int idx = t; idx < kCB * np; idx += nthr) {
         const int l = idx / kCB, c2 = idx - l * kCB;
@@ -1031,7 +707,7 @@ __device__ __forceinline__ void bse_mixed_system(const Dims& dm, int c, int a, i
         const float m = fmaxf(fabsf(yr), fabsf(yi)) * 1.0001f;
         if (m > 0.f) atomicMax(&cole[c2], exp_bound_f32(m));
       }
-      block_sync<NP>();
+      __syncthreads();
       // two consecutive l per thread: one 32-bit word per slice and part
       for (int idx = t; idx < kCB * np / 2; idx += nthr) {
         const int l = 2 * (idx / kCB), c2 = idx - (l / 2) * kCB;
@@ -1059,7 +735,7 @@ __device__ __forceinline__ void bse_mixed_system(const Dims& dm, int c, int a, i
           xw[(s2 * 2 + 1) * kCB * 32 + wo] = w1[s2] | (v1[s2] << 16);
         }
       }
-      block_sync<NP>();
+      __syncthreads();
       for (int tile = warp; tile < tiles; tile += nwarp) {
         const int r16 = (tile / (kCB / 8)) * 16, c8 = (tile % (kCB / 8)) * 8;
         // acc[d][0 / 1][.]: re / im of all digit pairs with sa + sb = d (one
@@ -1131,7 +807,7 @@ __device__ __forceinline__ void bse_mixed_system(const Dims& dm, int c, int a, i
         }
       }
     }
-    block_sync<NP>();
+    __syncthreads();
   } else {
     // Y = chi o X0 as double-float pairs, once per system
     for (int idx = t; idx < np * np; idx += kThr) {
@@ -1165,7 +841,7 @@ __device__ __forceinline__ void bse_mixed_system(const Dims& dm, int c, int a, i
   #pragma unroll
           for (int e = 0; e < 6; ++e) acc[i2][jj][e] = 0.f;
       for (int l0 = 0; l0 < np; l0 += lc) {
-        block_sync<NP>();
+        __syncthreads();
         for (int idx = t; idx < lc * np; idx += kThr) {
           const int r = idx / lc, ll = idx - r * lc;
           const int l = l0 + ll;
@@ -1173,7 +849,7 @@ __device__ __forceinline__ void bse_mixed_system(const Dims& dm, int c, int a, i
           gth[ll * np + r] = in ? Gh[r * n + l] : make_float2(0.f, 0.f);
           gtl[ll * np + r] = in ? Gl[r * n + l] : make_float2(0.f, 0.f);
         }
-        block_sync<NP>();
+        __syncthreads();
         for (int ll = 0; ll < lc; ++ll) {
           const int l = l0 + ll;
           float2 yh[kTile], yl[kTile];
@@ -1219,13 +895,13 @@ __device__ __forceinline__ void bse_mixed_system(const Dims& dm, int c, int a, i
         }
       }
     }
-    block_sync<NP>();
+    __syncthreads();
     // R to shared memory (logical rows, in place of X0)
 #pragma unroll
     for (int ii = 0; ii < kTile; ++ii)
 #pragma unroll
       for (int jj = 0; jj < kTile; ++jj) X0s[(tr + P * ii) * ld + tc + P * jj] = A[ii][kTile + jj];
-    block_sync<NP>();
+    __syncthreads();
   }
 
   // gamma o gamma^T (hi, lo) of this thread's first pass of the Gamma^(2)
@@ -1271,7 +947,7 @@ __device__ __forceinline__ void bse_mixed_system(const Dims& dm, int c, int a, i
     }
     if (tc == 0 && rowpos[ii] >= 0) ediag[j] = make_float2(ex, ey);
   }
-  block_sync<NP>();
+  __syncthreads();
 
   // ---- diag Gamma = diag X0 + diag E (FP64), Gamma^(2), Eq. sd bracket ----
   // Gamma^(2)_jj = sum_x (gamma_jx gamma_xj) chi~_x in double-float; four
@@ -1320,34 +996,7 @@ __device__ __forceinline__ void bse_mixed_system(const Dims& dm, int c, int a, i
     }
     mixed_check_ladder(mc, emax, gmax, fin, ((long)c * nb + a) * N + q, flags);
   }
-  block_sync<NP>();
-}
-
-// The producer warp's side of bse_mixed_system<64> for one system: per
-// column block, wait for the compute warps' handoff, then (lane 0) issue the
-// 32 MMAs (gamma slice sa: A = [Zr; Zi] of slice sa, B = the Y slices 0 .. 7 - sa
-// stacked along N, D at TMEM buffer b & 1, column 32 sa) and commit them.
-__device__ __forceinline__ void mixed_producer(const MixedPtrs& sp, const Tc05* umma) {
-  constexpr int np = 64;
-  const unsigned za = smem_u32(sp.work), xa = smem_u32(sp.work + xs_offset(np));
-  const int lane = threadIdx.x & 31;
-  for (int b = 0; b < np / kCB; ++b) {
-    handoff_wait();
-    if (lane == 0) {
-      tc05_fence_after();
-      const unsigned dt = umma->tmem + (unsigned)(256 * (b & 1));
-#pragma unroll 1
-      for (int sa = 0; sa < kSlices; ++sa) {
-        const unsigned idesc = umma_idesc_bf16(128, 32 * (kSlices - sa));
-#pragma unroll
-        for (int ks = 0; ks < 4; ++ks)
-          umma_bf16(dt + 32 * sa, umma_desc_sw128(za + sa * (2 * np * 128) + 32 * ks), umma_desc_sw128(xa + 32 * ks),
-                    idesc, (sa > 0 || ks > 0) ? 1u : 0u);
-      }
-      umma_commit(umma->mbar);
-    }
-    __syncwarp();
-  }
+  __syncthreads();
 }
 
 }  // namespace df

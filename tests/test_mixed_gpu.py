@@ -257,3 +257,31 @@ def test_tensor_core_sweep_matches_the_cuda_core_sweep(df):
         for a in range(w.n_bos):
             assert nrel(out[0][c, a], out[1][c, a]) < TOL_KERNEL
             assert nrel(out[0][c, a], k64[c, a]) < TOL_KERNEL
+
+
+@pytest.mark.parametrize("n_w", [34, 40, 42, 48, 50, 58, 62, 64])
+@pytest.mark.parametrize("wide", [False, True])
+def test_mixed_two_ladder_blocks(df, n_w, wide):
+    """Orders 33-64 where the kernel's tiles end (8-column panels, 16-row digit blocks, odd ladder
+    counts: three orbits per plane), complex vertices without symmetry, each channel alone and both
+    together; with `wide` the vertex's columns span twelve orders of magnitude and one is zero (the
+    digits are relative to a power of two per column).  Bound: the stated one of the mixed path
+    (each ladder's predicted error <= 1e-9 of its diag Gamma, or the FP64 solve)."""
+    w = I.random_nonsymmetric(n_w, 1, 1, 4, seed=n_w, scale=0.5)
+    if wide:
+        s = 10.0 ** np.random.default_rng(n_w).uniform(-9.0, 3.0, n_w)
+        s[n_w // 3] = 0.0
+        w.gamma_uu = w.gamma_uu * s
+        w.gamma_ud = w.gamma_ud * s
+    _, kref = oracle_first_pass(w)
+    with df.DualFermion.from_workload(w, precision=df.DF_FP32_IR, symmetry=1, eig_mode=0) as d:
+        d.bubble()
+        for mask, chans in ((1, (0,)), (2, (1,)), (3, (0, 1))):
+            d.bse(mask)
+            kern = d.get_kernel()
+            for c in chans:
+                for a in range(w.n_bos):
+                    assert nrel(kern[c, a], kref[c, a]) < TOL_KERNEL, (mask, c, a)
+        # the digit product carries T = S gamma to ~2^-47 of max|S_i| max|gamma_j|: what is left is the
+        # FP32 sweep's error squared, far below the bound on these well-conditioned ladders
+        assert nrel(kern, kref) < 1e-11
