@@ -512,3 +512,33 @@ def test_omega_split_two_handles(df, prec):
         d.sigma()
         e.sigma_finish(e.sigma_partial())
         assert nrel(e.get_sigma(), d.get_sigma()) < 1e-14
+
+
+@pytest.mark.parametrize("n_w", [2, 8, 16, 18, 32, 34, 48, 50, 64, 66, 96, 98, 128])
+@pytest.mark.parametrize("nk", [2, 16, 64])
+def test_leading_eigenvalue_at_tile_edges(df, n_w, nk):
+    """The power iteration at the orders where its column blocks end and at momentum counts on both
+    sides of a block's systems (2, 16 and 64 momenta on a 1D lattice).  Where the second largest
+    modulus is below half of the largest, the FP32 phase settles (0.5^64 < 2e-6) and 24 polish steps
+    reach 1e-12 (0.5^24 < 1e-7 on top of 2e-6), so the flag is 1 and the bound is the stated one of the
+    eigenvalue check, 1e-8."""
+    w = I.random_nonsymmetric(n_w, 0, 1, nk, seed=100 + n_w, scale=0.7)
+    w.gamma_uu[:] += 3.0 * np.linspace(0.5, 1.0, n_w)[:, None]       # a dominant rank-one part
+    w.gamma_ud[:] *= 0.2
+    gd, gm = O.channel_vertices(w.gamma_uu, w.gamma_ud)
+    with df.DualFermion.from_workload(w, eig_mode=2) as d:
+        d.bubble()
+        d.bse(3)
+        chi = d.get_chi()
+        lam, ok = d.get_lambda()
+    seen = 0
+    for c, g in enumerate((gd, gm)):
+        for q in range(w.N):
+            ev = np.linalg.eigvals(g[0] * chi[0, :, q][None, :])
+            ev = ev[np.argsort(-np.abs(ev))]
+            if len(ev) > 1 and abs(ev[1]) > 0.5 * abs(ev[0]):
+                continue
+            seen += 1
+            assert ok[c, 0, q] == 1, (c, q)
+            assert abs(lam[c, 0, q] - ev[0]) < 1e-8 * abs(ev[0]), (c, q)
+    assert seen > 0 or n_w == 2
