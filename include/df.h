@@ -75,9 +75,8 @@ typedef enum df_status {
 typedef enum df_precision {
   DF_FP64 = 0,       /* every step in FP64 (complex128) */
   DF_FP32_IR = 1     /* ladder solves factorised in FP32 (complex64) and refined by
-                        one correction with an extended-precision residual (n_w <= 64:
-                        exact digit products on the tensor cores; 64 < n_w <= 128:
-                        double-float).  Per ladder, rho = max|correction| / max|diag Gamma|
+                        one correction with an extended-precision residual (exact
+                        digit products on the tensor cores; below order 17 double-float).  Per ladder, rho = max|correction| / max|diag Gamma|
                         predicts the error left (~rho^2 of diag Gamma's largest entry);
                         a ladder with rho^2 > ladder_tol is solved again by the FP64 LU
                         (ladder_fallback = 1) or reported (DF_ERR_REFINE_STALL).  Bubble,
@@ -117,9 +116,10 @@ typedef struct df_opts {
   int ladder_fallback;/* DF_FP32_IR: 1 (default) a ladder above ladder_tol is solved again by
                        * the FP64 LU in the same df_bse; 0 its mixed result is kept and the
                        * next df_sigma / df_iterate returns DF_ERR_REFINE_STALL */
-  int mixed_sweep;    /* DF_FP32_IR, orders 64 < n_w <= 128: the FP32 Gauss-Jordan inversion on the
-                       * tensor cores (0, default: tcgen05 panel updates with three-piece BF16
-                       * operands, FP32 accumulation in tensor memory) or on the CUDA cores (1) */
+  int mixed_sweep;    /* DF_FP32_IR, orders 64 < n_w <= 128: 0 (default) FP32 Gauss-Jordan inversion in
+                       * registers and the high-precision product as exact FP16 digits on the
+                       * tensor cores (tcgen05), 1 inversion in shared memory and a double-float
+                       * residual, both on the CUDA cores */
   int w_lo, w_hi;     /* the Omega split (several GPUs, one problem): this handle owns the
                        * bosonic planes a in [w_lo, w_hi) (index a = m + m_max); default 0, 0
                        * = all.  df_bubble and df_bse then cover only those planes and the

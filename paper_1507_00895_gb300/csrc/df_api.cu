@@ -451,7 +451,7 @@ df_status df_init(df_ctx** out, const df_lattice* lat, double beta, double mu, d
     cudaError_t ea = cudaMalloc(&c->bse_ws, c->bse_ws_bytes);
     if (ea != cudaSuccess) { st = fail(c, DF_ERR_OOM, "cudaMalloc bse workspace", ea); goto bad; }
     if (opts->precision == DF_FP32_IR) {
-      c->tcr_off = mixed_tcr_offset(dm);
+      c->dig128_off = mixed_digits128_offset(dm);
       ea = cudaMalloc(&c->mixed_ws, mixed_workspace_bytes(dm));
       if (ea != cudaSuccess) { st = fail(c, DF_ERR_OOM, "cudaMalloc mixed workspace", ea); goto bad; }
     }

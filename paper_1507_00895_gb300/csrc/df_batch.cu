@@ -19,9 +19,9 @@
 
 #include "df_bse_dev.cuh"
 #include "df_fft_dev.cuh"
+#include "df_mixed128_dev.cuh"
 #include "df_mixed64_dev.cuh"
 #include "df_mixed_dev.cuh"
-#include "df_mixed_large_dev.cuh"
 
 namespace df {
 
@@ -50,8 +50,8 @@ struct PointDev {
   int active;    // 1 until converged
   double mix, tol, resid;
   double2 *g, *delta, *gam, *gg, *g0, *gk, *gr, *chi, *kc, *prod, *sigma;
-  float2 *gam_hi, *gam_lo, *gg_hi, *gg_lo;   // mixed: FP32 (hi, lo) of gam and gg (orders > 64: of gam^T)
-  unsigned char* gdig;                         // mixed, n_pad 32 / 64: gamma's digits
+  float2 *gam_hi, *gam_lo, *gg_hi, *gg_lo;   // mixed: FP32 (hi, lo) of gam and gg
+  unsigned char* gdig;                         // mixed, orders > 16: gamma's digits
   double* red;   // [2 n_w + 4]
   int* flags;    // [4]
 };
@@ -148,14 +148,15 @@ __global__ void batch_setup_elem_kernel(const PointDev* __restrict__ pts, int p)
       float hx = (float)v.x, hy = (float)v.y;
       P.gam_hi[idx] = make_float2(hx, hy);
       P.gam_lo[idx] = make_float2((float)(v.x - (double)hx), (float)(v.y - (double)hy));
-      // orders > 64 keep gamma^T's words in these slots (the large-order kernel's residual)
-      const double2 t = mixed_pad(n) > 64 ? G[j * n + i] : w;
-      hx = (float)t.x; hy = (float)t.y;
+      hx = (float)w.x; hy = (float)w.y;
       P.gg_hi[idx] = make_float2(hx, hy);
-      P.gg_lo[idx] = make_float2((float)(t.x - (double)hx), (float)(t.y - (double)hy));
+      P.gg_lo[idx] = make_float2((float)(w.x - (double)hx), (float)(w.y - (double)hy));
     }
   }
-  if (P.gdig && mixed_pad(n) == 64)
+  if (P.gdig && mixed_pad(n) == 128)
+    gamma_digits_cols128(n, 2 * P.dm.nb, P.gam, P.gdig, (blockIdx.x * blockDim.x + threadIdx.x) >> 5,
+                         (gridDim.x * blockDim.x) >> 5, threadIdx.x & 31);
+  else if (P.gdig && mixed_pad(n) == 64)
     gamma_digits_cols(n, 2 * P.dm.nb, P.gam, P.gdig, (blockIdx.x * blockDim.x + threadIdx.x) >> 5,
                       (gridDim.x * blockDim.x) >> 5, threadIdx.x & 31);
   else if (P.gdig)
@@ -350,36 +351,52 @@ batch_bse_mixed64_kernel(const PointDev* __restrict__ pts, const int* __restrict
   m64_teardown(blk);
 }
 
-// mixed ladders of order 64 < n <= 128 (the shared-memory Gauss-Jordan body),
-// 256 threads, the same chunked queue over the class's cost-sorted points
-__global__ void __launch_bounds__(256, 1)
-batch_bse_gj_kernel(const PointDev* __restrict__ pts, const int* __restrict__ order, const long* __restrict__ start,
-                    int nseg, int chunk, unsigned long long* __restrict__ counter, int* __restrict__ redo) {
-  extern __shared__ __align__(16) unsigned char smraw[];
-  __shared__ GjShared sh;
+// orders 65-128: one ladder at a time per block (df_mixed128_dev.cuh); nmax: the class's largest
+// order, whose shared-memory layout serves every order
+__global__ void __launch_bounds__(kM128Threads, 1)
+batch_bse_mixed128_kernel(const PointDev* __restrict__ pts, const int* __restrict__ order,
+                          const long* __restrict__ start, int nseg, int chunk,
+                          unsigned long long* __restrict__ counter, int* __restrict__ redo, int nmax) {
+  extern __shared__ __align__(1024) unsigned char sm128[];
+  __shared__ uint64_t bars_s[1 + 2 * kM128MaxRing];
+  __shared__ unsigned tslot_s;
+  __shared__ int fail_s;
   __shared__ unsigned long long item_s;
+  if (smem_u32(sm128) & 1023u) {                 // the swizzled operand tiles need 1024-byte alignment
+    if (threadIdx.x == 0) atomicOr(pts[0].flags, kFlagTcLayout);
+    return;
+  }
+  M128State st;
+  m128_setup(st, sm128, bars_s, &tslot_s, &fail_s);
+  M128Layout L = m128_layout(nmax);
   const long total = start[nseg];
-  for (;;) {
+  bool ok = true;
+  while (ok) {
+    __syncthreads();
     if (threadIdx.x == 0) item_s = atomicAdd(counter, (unsigned long long)chunk);
     __syncthreads();
     const long item = (long)item_s;
-    __syncthreads();
     if (item >= total) break;
-    const long end = min(item + (long)chunk, total);
-    for (long s = item; s < end; ++s) {
+    const long last = min(item + (long)chunk, total);
+    for (long s = item; s < last && ok; ++s) {
       const int k = find_segment(start, nseg, s);
       const PointDev& P = pts[order[k]];
       if (!P.active) continue;
       const Dims& dm = P.ldm;
-      const long local = s - start[k];
-      const long per_ch = (long)dm.na * dm.N;      // the view's planes a0 .. a0 + na - 1
-      const int c = (int)(local / per_ch);
-      const int rem = (int)(local - (long)c * per_ch);
-      const int a = dm.a0 + rem / dm.N, q = rem - (a - dm.a0) * dm.N;
-      gj_ir_system(dm, c, a, q, P.gam_hi, P.gam_lo, P.gg_hi, P.gg_lo, P.gg, P.lchi, P.lkc, P.flags, smraw, sh,
-                   batch_check(redo, order[k]));
+      const long local = s - start[k], plane = local / dm.N;
+      const int c = (int)(plane / dm.na), a = dm.a0 + (int)(plane % dm.na), key = c * dm.nb + a;
+      const size_t mat = (size_t)key * dm.n_w * dm.n_w;
+      L.ld = (dm.n_w + 31) / 32 * 32;
+      ok = m128_system(dm, c, a, (int)(local - plane * dm.N), P.gam_hi + mat, P.gam_lo + mat, P.gg_hi + mat,
+                       P.gg_lo + mat, P.gdig + (size_t)key * kM128DigBytes, P.lchi, P.lkc, P.flags, L, st,
+                       batch_check(redo, order[k]));
+      if (!ok) {
+        m128_drain(st, L);
+        if (threadIdx.x == 0) atomicOr(P.flags, kFlagTcTimeout);
+      }
     }
   }
+  m128_teardown(st);
 }
 
 }  // namespace df
@@ -393,6 +410,7 @@ using namespace df;
 namespace {
 
 int mixed_np_of(int n) { return mixed_pad(n); }
+size_t batch_digit_bytes(int n) { return n > 64 ? (size_t)kM128DigBytes : mixed_digit_bytes(mixed_pad(n)); }
 
 using MixedKernel = void (*)(const PointDev*, const int*, const long*, int, int, unsigned long long*, int*);
 
@@ -408,7 +426,8 @@ MixedKernel mixed_kernel_of(int np) {
 
 struct LadderGroup {          // one persistent ladder launch
   bool mixed = false;
-  int np = 0;                 // mixed: padded order (block = (np/4)^2 threads)
+  int np = 0;                 // mixed: padded order class
+  int nmax = 0;               // mixed: the class's largest order
   std::vector<int> order;     // points, cost-sorted
   long* d_start = nullptr;    // [nseg + 1]
   int* d_order = nullptr;
@@ -501,8 +520,8 @@ df_status record_pass(df_batch* b) {
       batch_bse_f64_kernel<<<g.grid, kBseThreads, g.smem, s>>>(b->d_pts, g.d_order, g.d_start, g.nseg, b->chunk,
                                                                b->d_counters + g.counter_slot, b->ws, b->ws_stride);
     } else if (g.np > 64) {
-      batch_bse_gj_kernel<<<g.grid, g.threads, g.smem, s>>>(b->d_pts, g.d_order, g.d_start, g.nseg, b->chunk,
-                                                            b->d_counters + g.counter_slot, b->d_redo);
+      batch_bse_mixed128_kernel<<<g.grid, g.threads, g.smem, s>>>(b->d_pts, g.d_order, g.d_start, g.nseg, b->chunk,
+                                                                  b->d_counters + g.counter_slot, b->d_redo, g.nmax);
     } else {
       mixed_kernel_of(g.np)<<<g.grid, g.threads, g.smem, s>>>(b->d_pts, g.d_order, g.d_start, g.nseg, b->chunk,
                                                               b->d_counters + g.counter_slot, b->d_redo);
@@ -556,14 +575,14 @@ df_status configure_groups(df_batch* b) {
   // the largest class
   for (auto& g : b->groups) {
     if (g.mixed && g.np > 64) {
-      g.threads = 256;
-      g.smem = (size_t)gj_layout(kGjMaxN).total;       // the largest order's layout serves every order
-      B_CUDA(b, cudaFuncSetAttribute((const void*)batch_bse_gj_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)g.smem),
+      g.threads = kM128Threads;
+      g.nmax = 0;
+      for (int p : g.order) g.nmax = std::max(g.nmax, b->host_pts[p].dm.n_w);
+      g.smem = (size_t)m128_layout(g.nmax).total;
+      B_CUDA(b, cudaFuncSetAttribute((const void*)batch_bse_mixed128_kernel,
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.smem),
              "large-order mixed smem attribute");
-      int per = 0;
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, batch_bse_gj_kernel, g.threads, g.smem);
-      g.grid = b->sms * std::max(1, per);
+      g.grid = b->sms;                                  // 512 columns of tensor memory: one block per SM
     } else if (g.mixed) {
       g.threads = g.np == 64 ? kM64Threads : mixed_block_threads(g.np);
       g.smem = g.np == 64 ? (size_t)kM64Smem : sizeof(float2) * (size_t)mixed_layout(g.np).total;
@@ -702,7 +721,7 @@ df_status df_batch_init(df_batch** out, int npts, const df_point* pts, int preci
     dm.mu = q.mu;
     dm.t = q.t;
     dm.tp = q.tp;
-    P.mixed = (precision == DF_FP32_IR && mixed_np_of(q.n_w) <= kGjMaxN) ? 1 : 0;
+    P.mixed = (precision == DF_FP32_IR && mixed_np_of(q.n_w) <= 128) ? 1 : 0;
     P.sym = q.symmetry ? 1 : 0;
     P.refl = q.symmetry == 2 ? 1 : 0;
     P.n_orb = P.sym ? build_wedge(q.dim, q.nk, qmaps[i], qreps[i]) : dm.N;
@@ -730,7 +749,7 @@ df_status df_batch_init(df_batch** out, int npts, const df_point* pts, int preci
     total += align_up(sizeof(double) * (2 * dm.n_w + 4));
     total += align_up(sizeof(int) * 4);
     if (P.mixed) total += align_up(sizeof(float2) * nv) * 4;      // gam hi, lo; gg hi, lo
-    if (P.mixed) total += align_up((size_t)2 * dm.nb * mixed_digit_bytes(mixed_pad(dm.n_w)));   // gamma's digits
+    if (P.mixed) total += align_up((size_t)2 * dm.nb * batch_digit_bytes(dm.n_w));   // gamma's digits
     if (P.sym) {
       const size_t nw = (size_t)dm.nb * dm.n_w * P.n_orb;
       total += align_up(sizeof(double2) * nw) * 3;                // compact chi, kc (2)
@@ -772,7 +791,7 @@ df_status df_batch_init(df_batch** out, int npts, const df_point* pts, int preci
       P.gam_lo = (float2*)take(sizeof(float2) * nv);
       P.gg_hi = (float2*)take(sizeof(float2) * nv);
       P.gg_lo = (float2*)take(sizeof(float2) * nv);
-      if (const size_t db = mixed_digit_bytes(mixed_pad(dm.n_w))) P.gdig = (unsigned char*)take((size_t)2 * dm.nb * db);
+      if (const size_t db = batch_digit_bytes(dm.n_w)) P.gdig = (unsigned char*)take((size_t)2 * dm.nb * db);
     }
     if (P.sym) {
       const size_t nw = (size_t)dm.nb * dm.n_w * P.n_orb;

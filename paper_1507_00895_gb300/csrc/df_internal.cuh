@@ -278,7 +278,7 @@ struct df_ctx {
   double* h_red = nullptr;     // pinned host mirror of the final residual
   void* bse_ws = nullptr;      // global scratch of the BSE kernel (large n)
   void* mixed_ws = nullptr;    // DF_FP32_IR: gamma as FP32 (hi, lo) pairs
-  size_t tcr_off = 0;          // byte offset of the tensor-core residual's digits in mixed_ws (fixed at
+  size_t dig128_off = 0;       // byte offset of gamma's digits (orders > 64) in mixed_ws (fixed at
                                // df_init: the hand-back list before it is sized for the full grid)
   int mixed_grid = 0;
   size_t bse_ws_bytes = 0;
@@ -332,11 +332,11 @@ cudaError_t launch_bse_mixed(df_ctx* c, int channel_mask, int* flags);
 // orders 64 < n_w <= 128 (df_mixed_large.cu)
 cudaError_t launch_bse_mixed_large(df_ctx* c, int channel_mask, int* flags);
 MixedCheck mixed_check(df_ctx* c);
-size_t mixed_tcr_offset(const Dims& dm);      // byte offset of the tensor-core residual's gamma digits
-size_t tcr_workspace_bytes(const Dims& dm);
+size_t mixed_digits128_offset(const Dims& dm);
+size_t digits128_bytes(const Dims& dm);
 unsigned* mixed_check_words(df_ctx* c);   // [0] worst rho^2, [2] hand-back count, [3 ..] list
 cudaError_t launch_bse_f64_list(df_ctx* c, const int* list);
-cudaError_t launch_split_gamma_t(df_ctx* c);
+cudaError_t launch_gamma_large(df_ctx* c);
 // point-group reduction (df_sym.cu)
 int build_wedge(int dim, int nk, std::vector<int>& qmap, std::vector<int>& qrep);
 cudaError_t launch_wedge_gather(df_ctx* c, const Dims& ladder_dims);

@@ -136,10 +136,10 @@ static size_t mixed_check_offset(const Dims& dm) {
   const size_t digits = (size_t)2 * dm.nb * mixed_digit_bytes(np);
   return ((size_t)4 * 2 * dm.nb * dm.n_w * dm.n_w * sizeof(float2) + digits + 15) & ~(size_t)15;
 }
-size_t mixed_tcr_offset(const Dims& dm) {
+size_t mixed_digits128_offset(const Dims& dm) {
   return (mixed_check_offset(dm) + sizeof(int) * (4 + (size_t)2 * dm.nb * dm.N) + 1023) & ~(size_t)1023;
 }
-size_t mixed_workspace_bytes(const Dims& dm) { return mixed_tcr_offset(dm) + tcr_workspace_bytes(dm); }
+size_t mixed_workspace_bytes(const Dims& dm) { return mixed_digits128_offset(dm) + digits128_bytes(dm); }
 // [0] worst rho^2 (float bits), [1] unused, [2] hand-back count, [3 ..] list
 unsigned* mixed_check_words(df_ctx* c) { return (unsigned*)((char*)c->mixed_ws + mixed_check_offset(c->dm)); }
 
@@ -166,7 +166,7 @@ cudaError_t launch_split_gamma(df_ctx* c, const double2* gg) {
   split_gamma_kernel<<<256, 256, 0, c->stream>>>(count, c->gam, gg, hi, hi + count, hi + 2 * count, hi + 3 * count);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  if (mixed_np(dm.n_w) > 64) return launch_split_gamma_t(c);   // slots 2, 3: gamma^T's words
+  if (mixed_np(dm.n_w) > 64) return launch_gamma_large(c);
   if (unsigned char* gd = gdig_ptr(c)) {
     const int np = mixed_np(dm.n_w), rows = 2 * dm.nb * np;
     if (np == 64)

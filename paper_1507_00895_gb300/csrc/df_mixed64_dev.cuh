@@ -55,7 +55,7 @@ constexpr int kM64TsLd = 65;                              // row stride of T (fl
 constexpr int kM64ELd = 66;                               // row stride of the exchange (float2)
 constexpr int kM64Acc = 32 * kDig;                        // TMEM columns of one 16-row block's accumulators
 
-// gamma's digits of one matrix in global memory, by padded order (0: none kept)
+// gamma's digits of one matrix in global memory, by padded order (0: none kept; orders > 64: df_mixed128_dev.cuh)
 __host__ __device__ constexpr size_t mixed_digit_bytes(int np) {
   return np == 64 ? kM64DigBytes : (use_tc_residual(np) ? gdig_bytes(np) : 0);
 }
@@ -177,19 +177,22 @@ __device__ __forceinline__ float rcp_approx(float x) {
   return r;
 }
 
-// The eight in-place Gauss-Jordan steps of a panel of 64 rows on two warps, one
-// row per lane (this lane's row r, its panel columns pv).  Per step each warp's
+// The eight in-place Gauss-Jordan steps of a panel of 32 WARPS rows, one row per
+// lane (this lane's row r, its panel columns pv; warp `half` of the team).  Per step each warp's
 // unused row with the largest key (|re| + |im| bits with 127 - row in the low
 // 7: largest to 2^-16, ties to the lowest row) goes to its slot of cand, its
-// key to ckey (two sets of slots in turn), a 64-thread barrier, and both warps
-// take the better row (u); then every row adds f u, f = -m / pivot with m its
+// key to ckey (two sets of slots in turn), the team's barrier, and all its warps
+// take the best row (u); then every row adds f u, f = -m / pivot with m its
 // entry of the pivot column (the pivot row, taken as zero: 1 / pivot).  The
 // next column and its search come before the rest of the update, so that the
 // search's latency is covered.  This chain of n steps is the ladder's critical
 // path: ~80 instructions a step and no branches.  W = P' - unit columns at the
 // pivot rows goes to wk [step][row].
-__device__ __forceinline__ void m64_panel(float2 (&pv)[kPanel], int r, int half, int lane, int k0, float2* wk,
-                                          float4* cand, uint2* ckey, int* piv_s, int* rowstep, int* flags, int bar) {
+template <int WARPS>
+__device__ __forceinline__ void gj_panel_team(float2 (&pv)[kPanel], int r, int half, int lane, int k0, float2* wk,
+                                              float4* cand, unsigned* ckey, int* piv_s, int* rowstep, int* flags,
+                                              int bar) {
+  constexpr int kRows = 32 * WARPS;
   const bool taken = rowstep[r] >= 0;
   unsigned km = taken ? 0u : ~0x7Fu, kr = taken ? 0u : (unsigned)(127 - r);   // 0 once the row is a pivot
   int step = -1;
@@ -199,15 +202,25 @@ __device__ __forceinline__ void m64_panel(float2 (&pv)[kPanel], int r, int half,
   for (int i = 0; i < kPanel; ++i) {
     const int par = i & 1;
     const unsigned kw = __reduce_max_sync(0xffffffffu, key);
-    const unsigned ca = smem_u32(cand + (par * 2 + half) * (kPanel / 2));
+    const unsigned ca = smem_u32(cand + (par * WARPS + half) * (kPanel / 2));
     const bool best = key == kw;
 #pragma unroll
     for (int c = 0; c < kPanel; c += 2) st_shared_if(best, ca + 8 * c, pv[c], pv[c + 1]);
-    if (lane == 0) reinterpret_cast<unsigned*>(ckey + par)[half] = kw;
-    asm volatile("bar.sync %0, 64;" ::"r"(bar) : "memory");
-    const uint2 ks = ckey[par];
-    const unsigned kb = max(ks.x, ks.y);
-    const float4* cb = cand + (par * 2 + (ks.y > ks.x ? 1 : 0)) * (kPanel / 2);
+    if (lane == 0) ckey[par * WARPS + half] = kw;
+    asm volatile("bar.sync %0, %1;" ::"r"(bar), "n"(kRows) : "memory");
+    unsigned kb;
+    int wb;
+    if constexpr (WARPS == 2) {
+      const uint2 ks = *reinterpret_cast<const uint2*>(ckey + par * 2);
+      kb = max(ks.x, ks.y);
+      wb = ks.y > ks.x ? 1 : 0;
+    } else {
+      const uint4 ks = *reinterpret_cast<const uint4*>(ckey + par * 4);
+      const unsigned k01 = max(ks.x, ks.y), k23 = max(ks.z, ks.w);
+      kb = max(k01, k23);
+      wb = k23 > k01 ? (ks.w > ks.z ? 3 : 2) : (ks.y > ks.x ? 1 : 0);
+    }
+    const float4* cb = cand + (par * WARPS + wb) * (kPanel / 2);
     const float2 z = reinterpret_cast<const float2*>(cb)[i];
     float2 u[kPanel];
 #pragma unroll
@@ -238,7 +251,7 @@ __device__ __forceinline__ void m64_panel(float2 (&pv)[kPanel], int r, int half,
       if (c != i && c != i + 1) pv[c] = cfmaf2(f, u[c], pv[c]);
   }
 #pragma unroll
-  for (int c = 0; c < kPanel; ++c) wk[c * 64 + r] = make_float2(step == c ? pv[c].x - 1.f : pv[c].x, pv[c].y);
+  for (int c = 0; c < kPanel; ++c) wk[c * kRows + r] = make_float2(step == c ? pv[c].x - 1.f : pv[c].x, pv[c].y);
   if (step >= 0) {
     rowstep[r] = k0 + step;
     piv_s[k0 + step] = r;
@@ -322,7 +335,7 @@ __device__ __forceinline__ void m64_system(const Dims& dm, int c, int a, int q, 
     float4* prs = reinterpret_cast<float4*>(sm + kM64Work) + warp * 32;   // [step][4]: this warp's columns of the pivot rows
     float2* swap = reinterpret_cast<float2*>(sm + kM64Work + 8 * 512);    // [column][32]: half a panel on its way
     float4* cand = reinterpret_cast<float4*>(swap + kPanel * 32);         // [2][2][kPanel / 2]
-    uint2* ckey = reinterpret_cast<uint2*>(cand + 2 * kPanel);            // [2]
+    unsigned* ckey = reinterpret_cast<unsigned*>(cand + 2 * kPanel);      // [2][2]
 #pragma unroll 1
     for (int kp = 0; kp < npan; ++kp) {
       if (warp == kp || warp == (kp ^ 1)) {
@@ -336,7 +349,7 @@ __device__ __forceinline__ void m64_system(const Dims& dm, int c, int a, int q, 
         float2 pv[kPanel];
 #pragma unroll
         for (int c = 0; c < kPanel; ++c) pv[c] = half ? swap[c * 32 + lane] : A[0][c];
-        m64_panel(pv, r, half, lane, kPanel * kp, wbuf + kp * 512, cand, ckey, piv_s, rowstep, flags, 3 + gr.g);
+        gj_panel_team<2>(pv, r, half, lane, kPanel * kp, wbuf + kp * 512, cand, ckey, piv_s, rowstep, flags, 3 + gr.g);
         if (half == 1) {
 #pragma unroll
           for (int c = 0; c < kPanel; ++c) swap[c * 32 + lane] = pv[c];

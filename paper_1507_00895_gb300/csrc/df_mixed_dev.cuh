@@ -235,6 +235,18 @@ __device__ __forceinline__ void tmem_ld16(unsigned taddr, float* v) {
 #pragma unroll
   for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[j]);
 }
+// TMEM allocation of a fixed power-of-two column count (warp 0 calls alloc/dealloc)
+template <int COLS>
+__device__ __forceinline__ void tmem_alloc_cols(unsigned* slot) {
+  asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(slot)), "n"(COLS)
+               : "memory");
+  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+}
+template <int COLS>
+__device__ __forceinline__ void tmem_dealloc_cols(unsigned taddr) {
+  asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "n"(COLS) : "memory");
+}
+
 __device__ __forceinline__ void dd_add(float& hi, float& lo, float v) {
   float s, e;
   two_sum(hi, v, s, e);

@@ -17,8 +17,7 @@
 
 #include <cuda_bf16.h>
 
-#include "df_tcgj_dev.cuh"
-#include "df_tcr_dev.cuh"
+#include "df_mixed_dev.cuh"
 
 namespace df {
 

@@ -285,3 +285,21 @@ def test_mixed_two_ladder_blocks(df, n_w, wide):
         # the digit product carries T = S gamma to ~2^-47 of max|S_i| max|gamma_j|: what is left is the
         # FP32 sweep's error squared, far below the bound on these well-conditioned ladders
         assert nrel(kern, kref) < 1e-11
+
+
+@pytest.mark.parametrize("n_w", [66, 72, 80, 94, 96, 98, 112, 126, 128])
+@pytest.mark.parametrize("wide", [False, True])
+def test_mixed_streamed_digits(df, n_w, wide):
+    """Orders 65-128 where the kernel's tiles end (8-column panels, 16-row blocks, 64-column tiles,
+    pieces of 32 K of the streamed digits), the same inputs and bound as for the orders below."""
+    test_mixed_two_ladder_blocks(df, n_w, wide)
+
+
+def test_mixed_orders_share_a_batch_class(df):
+    """A batch's large-order class runs every order on the largest one's shared-memory layout."""
+    ws = [I.half_filled_atom(f"b{n}", 1, 8, U=3.0 + 0.01 * n, beta=2.0, n_w=n, m_max=1) for n in (128, 66, 96, 80)]
+    with df.DualFermionBatch(ws, precision=df.DF_FP32_IR) as b:
+        b.iterate(1)
+        for i, w in enumerate(ws):
+            st, _ = oracle_first_pass(w)
+            assert nrel(b.get_sigma(i), st.sigma) < TOL_SIGMA, w.n_w
