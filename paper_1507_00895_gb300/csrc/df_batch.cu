@@ -20,8 +20,8 @@
 #include "df_bse_dev.cuh"
 #include "df_fft_dev.cuh"
 #include "df_mixed128_dev.cuh"
+#include "df_mixed32_dev.cuh"
 #include "df_mixed64_dev.cuh"
-#include "df_mixed_dev.cuh"
 
 namespace df {
 
@@ -51,7 +51,7 @@ struct PointDev {
   double mix, tol, resid;
   double2 *g, *delta, *gam, *gg, *g0, *gk, *gr, *chi, *kc, *prod, *sigma;
   float2 *gam_hi, *gam_lo, *gg_hi, *gg_lo;   // mixed: FP32 (hi, lo) of gam and gg
-  unsigned char* gdig;                         // mixed, orders > 16: gamma's digits
+  unsigned char* gdig;                         // mixed: gamma's digits
   double* red;   // [2 n_w + 4]
   int* flags;    // [4]
 };
@@ -159,9 +159,12 @@ __global__ void batch_setup_elem_kernel(const PointDev* __restrict__ pts, int p)
   else if (P.gdig && mixed_pad(n) == 64)
     gamma_digits_cols(n, 2 * P.dm.nb, P.gam, P.gdig, (blockIdx.x * blockDim.x + threadIdx.x) >> 5,
                       (gridDim.x * blockDim.x) >> 5, threadIdx.x & 31);
+  else if (P.gdig && mixed_pad(n) == 32)
+    gamma_digits_frag<32>(n, 2 * P.dm.nb, P.gam, P.gdig, (blockIdx.x * blockDim.x + threadIdx.x) >> 5,
+                          (gridDim.x * blockDim.x) >> 5, threadIdx.x & 31);
   else if (P.gdig)
-    gamma_digits_rows(n, mixed_pad(n), 2 * P.dm.nb, P.gam, P.gdig, (blockIdx.x * blockDim.x + threadIdx.x) >> 5,
-                      (gridDim.x * blockDim.x) >> 5, threadIdx.x & 31);
+    gamma_digits_frag<16>(n, 2 * P.dm.nb, P.gam, P.gdig, (blockIdx.x * blockDim.x + threadIdx.x) >> 5,
+                          (gridDim.x * blockDim.x) >> 5, threadIdx.x & 31);
 }
 
 __global__ void __launch_bounds__(kFftThreads)
@@ -265,38 +268,43 @@ __global__ void batch_wedge_scatter_kernel(const PointDev* __restrict__ pts) {
   }
 }
 
+// orders up to 32: one ladder of one (point, channel, W) at a time per warp; a block takes
+// kBatch32Take chunks of systems at once, several ladders per warp
+constexpr int kBatch32Take = 8;
 template <int NP>
-__global__ void __launch_bounds__(mixed_block_threads(NP))
-batch_bse_mixed_kernel(const PointDev* __restrict__ pts, const int* __restrict__ order, const long* __restrict__ start,
-                       int nseg, int chunk, unsigned long long* __restrict__ counter, int* __restrict__ redo) {
-  extern __shared__ __align__(1024) float2 smf[];
-  __shared__ int piv_s[128];
-  __shared__ unsigned long long item_s;
-  const MixedPtrs sp = mixed_ptrs(smf, NP, piv_s);
+__global__ void __launch_bounds__(M32<NP>::kThreads, 1)
+batch_bse_mixed32_kernel(const PointDev* __restrict__ pts, const int* __restrict__ order,
+                         const long* __restrict__ start, int nseg, int chunk,
+                         unsigned long long* __restrict__ counter, int* __restrict__ redo) {
+  using M = M32<NP>;
+  extern __shared__ __align__(16) unsigned char sm32[];
+  unsigned long long& item_s = *reinterpret_cast<unsigned long long*>(sm32 + M::kItem);
+  unsigned char* ws = sm32 + M::kBytes + (threadIdx.x >> 5) * M::kWarp;
   const long total = start[nseg];
   long cur = -1;                       // (point, channel, W) whose gamma digits are in shared memory
   for (;;) {
-    if (threadIdx.x == 0) item_s = atomicAdd(counter, (unsigned long long)chunk);
     __syncthreads();
-    const long item = (long)item_s;
+    if (threadIdx.x == 0) item_s = atomicAdd(counter, (unsigned long long)(kBatch32Take * chunk));
     __syncthreads();
-    if (item >= total) break;
-    const long end = min(item + (long)chunk, total);
-    for (long s = item; s < end; ++s) {
+    long s = (long)item_s;
+    if (s >= total) break;
+    const long last = min(s + (long)(kBatch32Take * chunk), total);
+    while (s < last) {
       const int k = find_segment(start, nseg, s);
       const PointDev& P = pts[order[k]];
-      if (!P.active) continue;
       const Dims& dm = P.ldm;
-      const long local = s - start[k];
-      const long per_ch = (long)dm.na * dm.N;      // the view's planes a0 .. a0 + na - 1
-      const int c = (int)(local / per_ch);
-      const int rem = (int)(local - (long)c * per_ch);
-      const int a = dm.a0 + rem / dm.N, q = rem - (a - dm.a0) * dm.N;
-      const long key = (long)k * 256 + c * dm.nb + a;
-      bse_mixed_system<NP>(dm, c, a, q, P.gam, P.gam_hi, P.gam_lo, P.gg_hi, P.gg_lo, P.lchi, P.lkc, P.flags, sp,
-                           P.gdig ? P.gdig + (size_t)(c * dm.nb + a) * gdig_bytes(NP) : nullptr, key != cur,
-                           batch_check(redo, order[k]));
-      cur = key;
+      const long plane = (s - start[k]) / dm.N;    // (channel, view plane) of the point
+      const long base = start[k] + plane * dm.N, end = min(last, base + dm.N);
+      if (P.active) {
+        const int c = (int)(plane / dm.na), a = dm.a0 + (int)(plane % dm.na), key = c * dm.nb + a;
+        const long id = (long)k * 256 + key;
+        if (id != cur) m32_load_gamma<NP>(sm32, P.gdig + (size_t)key * M::kBytes);
+        cur = id;
+        const size_t mat = (size_t)key * dm.n_w * dm.n_w;
+        for (long x = s + (threadIdx.x >> 5); x < end; x += M::kWarps)
+          m32_system<NP>(dm, c, a, (int)(x - base), sm32, P.gg_hi + mat, P.gg_lo + mat, P.lchi, P.lkc, P.flags, ws, batch_check(redo, order[k]));
+      }
+      s = end;
     }
   }
 }
@@ -414,15 +422,16 @@ size_t batch_digit_bytes(int n) { return n > 64 ? (size_t)kM128DigBytes : mixed_
 
 using MixedKernel = void (*)(const PointDev*, const int*, const long*, int, int, unsigned long long*, int*);
 
-// the ladder kernel instance of a padded order (8, 16, 32 or 64)
+// the ladder kernel, its block and its shared memory at a padded order (16, 32 or 64)
 MixedKernel mixed_kernel_of(int np) {
   switch (np) {
-    case 8: return batch_bse_mixed_kernel<8>;
-    case 16: return batch_bse_mixed_kernel<16>;
-    case 32: return batch_bse_mixed_kernel<32>;
+    case 16: return batch_bse_mixed32_kernel<16>;
+    case 32: return batch_bse_mixed32_kernel<32>;
     default: return batch_bse_mixed64_kernel;
   }
 }
+int mixed_threads_of(int np) { return np == 16 ? M32<16>::kThreads : np == 32 ? M32<32>::kThreads : kM64Threads; }
+int mixed_smem_of(int np) { return np == 16 ? M32<16>::kSmem : np == 32 ? M32<32>::kSmem : kM64Smem; }
 
 struct LadderGroup {          // one persistent ladder launch
   bool mixed = false;
@@ -584,8 +593,8 @@ df_status configure_groups(df_batch* b) {
              "large-order mixed smem attribute");
       g.grid = b->sms;                                  // 512 columns of tensor memory: one block per SM
     } else if (g.mixed) {
-      g.threads = g.np == 64 ? kM64Threads : mixed_block_threads(g.np);
-      g.smem = g.np == 64 ? (size_t)kM64Smem : sizeof(float2) * (size_t)mixed_layout(g.np).total;
+      g.threads = mixed_threads_of(g.np);
+      g.smem = (size_t)mixed_smem_of(g.np);
       B_CUDA(b, cudaFuncSetAttribute((const void*)mixed_kernel_of(g.np), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)g.smem),
              "mixed smem attribute");
@@ -791,7 +800,7 @@ df_status df_batch_init(df_batch** out, int npts, const df_point* pts, int preci
       P.gam_lo = (float2*)take(sizeof(float2) * nv);
       P.gg_hi = (float2*)take(sizeof(float2) * nv);
       P.gg_lo = (float2*)take(sizeof(float2) * nv);
-      if (const size_t db = batch_digit_bytes(dm.n_w)) P.gdig = (unsigned char*)take((size_t)2 * dm.nb * db);
+      P.gdig = (unsigned char*)take((size_t)2 * dm.nb * batch_digit_bytes(dm.n_w));
     }
     if (P.sym) {
       const size_t nw = (size_t)dm.nb * dm.n_w * P.n_orb;
@@ -891,22 +900,22 @@ df_status df_batch_init(df_batch** out, int npts, const df_point* pts, int preci
       return b->host_pts[x].dm.n_w > b->host_pts[y].dm.n_w;   // largest ladders first
     });
     LadderGroup f64;
-    std::vector<LadderGroup> mixed_groups(6);   // padded orders 4 .. 128
-    for (int k = 0; k < 6; ++k) {
+    std::vector<LadderGroup> mixed_groups(4);   // padded orders 16 .. 128
+    for (int k = 0; k < 4; ++k) {
       mixed_groups[k].mixed = true;
-      mixed_groups[k].np = 4 << k;
+      mixed_groups[k].np = 16 << k;
     }
     for (int i : idx) {
       if (b->host_pts[i].mixed) {
         int k = 0;
-        while ((4 << k) < mixed_np_of(b->host_pts[i].dm.n_w)) ++k;
+        while ((16 << k) < mixed_np_of(b->host_pts[i].dm.n_w)) ++k;
         mixed_groups[k].order.push_back(i);
       } else {
         f64.order.push_back(i);
       }
     }
     if (!f64.order.empty()) b->groups.push_back(f64);
-    for (int k = 5; k >= 0; --k)
+    for (int k = 3; k >= 0; --k)
       if (!mixed_groups[k].order.empty()) b->groups.push_back(mixed_groups[k]);
     for (size_t gi = 0; gi < b->groups.size(); ++gi) {
       LadderGroup& g = b->groups[gi];

@@ -280,7 +280,6 @@ struct df_ctx {
   void* mixed_ws = nullptr;    // DF_FP32_IR: gamma as FP32 (hi, lo) pairs
   size_t dig128_off = 0;       // byte offset of gamma's digits (orders > 64) in mixed_ws (fixed at
                                // df_init: the hand-back list before it is sized for the full grid)
-  int mixed_grid = 0;
   size_t bse_ws_bytes = 0;
   int bse_grid = 0;
   int iter_done = 0;

@@ -1,7 +1,8 @@
 // Mixed-precision ladder solves (DF_FP32_IR) of one problem: the kernels around
 // the per-ladder bodies of df_mixed64_dev.cuh (orders 33-64, two ladders of
-// one (channel, W) at a time per block) and df_mixed_dev.cuh (orders up to 32),
-// gamma's words and digits, and the launchers.
+// one (channel, W) at a time per block) and df_mixed32_dev.cuh (orders up to 32,
+// one ladder per warp), gamma's words and digits, and the launchers.
+#include "df_mixed32_dev.cuh"
 #include "df_mixed64_dev.cuh"
 
 namespace df {
@@ -22,11 +23,12 @@ __global__ void split_gamma_kernel(size_t count, const double2* __restrict__ g, 
   }
 }
 
-// gamma's digits for the tensor-core residual (once per input upload)
-__global__ void gamma_digits_kernel(int n, int np, int count, const double2* __restrict__ gam,
-                                    unsigned char* __restrict__ out) {
-  gamma_digits_rows(n, np, count, gam, out, (blockIdx.x * blockDim.x + threadIdx.x) >> 5,
-                    (gridDim.x * blockDim.x) >> 5, threadIdx.x & 31);
+// gamma's digits (once per input upload)
+template <int NP>
+__global__ void gamma_digits32_kernel(int n, int count, const double2* __restrict__ gam,
+                                      unsigned char* __restrict__ out) {
+  gamma_digits_frag<NP>(n, count, gam, out, (blockIdx.x * blockDim.x + threadIdx.x) >> 5,
+                        (gridDim.x * blockDim.x) >> 5, threadIdx.x & 31);
 }
 
 __global__ void gamma_digits64_kernel(int n, int count, const double2* __restrict__ gam,
@@ -35,31 +37,28 @@ __global__ void gamma_digits64_kernel(int n, int count, const double2* __restric
                     threadIdx.x & 31);
 }
 
-// One contiguous range of systems per block (so that consecutive systems
-// share (channel, W) and gamma's digits stay in shared memory).
+// Orders up to 32: one contiguous range of systems per block, split where
+// (channel, W) changes; the warps of a block take its systems in turn.
 template <int NP>
-__global__ void __launch_bounds__(mixed_block_threads(NP))
-bse_mixed_kernel(Dims dm, int ch0, int nch, const double2* __restrict__ gam,
-                 const float2* __restrict__ gam_hi, const float2* __restrict__ gam_lo,
-                 const float2* __restrict__ gg_hi, const float2* __restrict__ gg_lo,
-                 const double2* __restrict__ chi, double2* __restrict__ kc,
-                 const unsigned char* __restrict__ gdig, int* __restrict__ flags, MixedCheck mc) {
-  extern __shared__ __align__(1024) float2 smf[];
-  __shared__ int piv_s[128];
-  const MixedPtrs sp = mixed_ptrs(smf, NP, piv_s);
+__global__ void __launch_bounds__(M32<NP>::kThreads, 1)
+bse_mixed32_kernel(Dims dm, int ch0, int nch, const float2* __restrict__ gg_hi, const float2* __restrict__ gg_lo,
+                   const double2* __restrict__ chi, double2* __restrict__ kc, const unsigned char* __restrict__ gdig,
+                   int* __restrict__ flags, MixedCheck mc) {
+  using M = M32<NP>;
+  extern __shared__ __align__(16) unsigned char sm32[];
+  unsigned char* ws = sm32 + M::kBytes + (threadIdx.x >> 5) * M::kWarp;
   const int N = dm.N, nb = dm.nb, na = dm.na;
   const long systems = (long)nch * na * N;
-  const long per = (systems + gridDim.x - 1) / gridDim.x;
-  const long s0 = (long)blockIdx.x * per, s1 = s0 + per < systems ? s0 + per : systems;
-  int cur = -1;
-  for (long sys = s0; sys < s1; ++sys) {
-    const int c = ch0 + (int)(sys / ((long)na * N));
-    const int rem = (int)(sys - (long)(c - ch0) * na * N);
-    const int a = dm.a0 + rem / N, q = rem - (a - dm.a0) * N;
-    const int key = c * nb + a;
-    bse_mixed_system<NP>(dm, c, a, q, gam, gam_hi, gam_lo, gg_hi, gg_lo, chi, kc, flags, sp,
-                         gdig ? gdig + (size_t)key * gdig_bytes(NP) : nullptr, key != cur, mc);
-    cur = key;
+  const long s1 = systems * (blockIdx.x + 1) / gridDim.x;
+  long s = systems * blockIdx.x / gridDim.x;
+  while (s < s1) {
+    const long plane = s / N, end = min(s1, (plane + 1) * N);
+    const int c = ch0 + (int)(plane / na), a = dm.a0 + (int)(plane % na), key = c * nb + a;
+    m32_load_gamma<NP>(sm32, gdig + (size_t)key * M::kBytes);
+    const size_t mat = (size_t)key * dm.n_w * dm.n_w;
+    for (long x = s + (threadIdx.x >> 5); x < end; x += M::kWarps)
+      m32_system<NP>(dm, c, a, (int)(x - plane * N), sm32, gg_hi + mat, gg_lo + mat, chi, kc, flags, ws, mc);
+    s = end;
   }
 }
 
@@ -124,8 +123,6 @@ cudaError_t launch_wait_selftest(int arrive, unsigned spins, int* flags, cudaStr
 
 static int mixed_np(int n) { return mixed_pad(n); }
 
-// the register-resident [D | RHS] tile limits this kernel to n_w <= 64; orders
-// up to 128 take the shared-memory Gauss-Jordan kernel of df_mixed_large.cu
 bool mixed_supported(int n_w) { return mixed_np(n_w) <= 128; }
 
 // gamma hi, lo; gamma o gamma^T hi, lo (orders > 64: gamma^T hi, lo); gamma's
@@ -155,7 +152,7 @@ MixedCheck mixed_check(df_ctx* c) {
 
 static unsigned char* gdig_ptr(df_ctx* c) {
   const int np = mixed_np(c->dm.n_w);
-  if (!mixed_digit_bytes(np)) return nullptr;
+  if (np > 64) return nullptr;
   return (unsigned char*)c->mixed_ws + (size_t)4 * 2 * c->dm.nb * c->dm.n_w * c->dm.n_w * sizeof(float2);
 }
 
@@ -172,45 +169,30 @@ cudaError_t launch_split_gamma(df_ctx* c, const double2* gg) {
     if (np == 64)
       gamma_digits64_kernel<<<(rows + 7) / 8, 256, 0, c->stream>>>(dm.n_w, 2 * dm.nb, c->gam, gd);
     else
-      gamma_digits_kernel<<<(rows + 7) / 8, 256, 0, c->stream>>>(dm.n_w, np, 2 * dm.nb, c->gam, gd);
+      (np == 32 ? gamma_digits32_kernel<32> : gamma_digits32_kernel<16>)<<<(rows + 7) / 8, 256, 0, c->stream>>>(
+          dm.n_w, 2 * dm.nb, c->gam, gd);
     e = cudaGetLastError();
   }
   return e;
 }
 
+// orders up to 32: one block per SM, one ladder per warp
 template <int NP>
-static cudaError_t launch_bse_mixed_np(df_ctx* c, int channel_mask, int* flags) {
+static cudaError_t launch_bse_mixed32(df_ctx* c, int channel_mask, int* flags) {
+  using M = M32<NP>;
   const Dims& dm = c->dm;
-  constexpr int threads = mixed_block_threads(NP);
-  const size_t smem = sizeof(float2) * (size_t)mixed_layout(NP).total;
-  cudaError_t e = cudaFuncSetAttribute((const void*)bse_mixed_kernel<NP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
+  cudaError_t e = cudaFuncSetAttribute((const void*)bse_mixed32_kernel<NP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       M::kSmem);
   if (e != cudaSuccess) return e;
-  if (c->mixed_grid == 0) {
-    int per_sm = 0, sms = 0;
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, bse_mixed_kernel<NP>, threads, smem);
-    c->mixed_grid = sms * (per_sm < 1 ? 1 : per_sm);
-  }
+  int sms = 0;
+  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device)) != cudaSuccess) return e;
   const size_t count = (size_t)2 * dm.nb * dm.n_w * dm.n_w;
-  const float2* hi = (const float2*)c->mixed_ws;
-  const MixedCheck mc = mixed_check(c);
-  // one launch per channel; both channels in one launch when a channel is only a
-  // few waves of the grid (the reduced grids), where the last partial wave of
-  // each launch would otherwise idle most blocks
-  const long per_channel = (long)dm.na * dm.N;
-  const bool both = (channel_mask & 3) == 3 && per_channel < 16L * c->mixed_grid;
-  for (int ch = 0; ch < 2; ++ch) {
-    if (!(channel_mask & (1 << ch))) continue;
-    const int nch = both ? 2 : 1;
-    const long systems = nch * per_channel;
-    const int grid = (int)(systems < c->mixed_grid ? systems : c->mixed_grid);
-    bse_mixed_kernel<NP><<<grid, threads, smem, c->stream>>>(dm, ch, nch, c->gam, hi, hi + count, hi + 2 * count,
-                                                             hi + 3 * count, c->chi, c->kc, gdig_ptr(c), flags, mc);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if (both) break;
-  }
-  return cudaSuccess;
+  const float2* gg = (const float2*)c->mixed_ws + 2 * count;
+  const int nch = (channel_mask & 1) + ((channel_mask >> 1) & 1), ch0 = (channel_mask & 1) ? 0 : 1;
+  const long systems = (long)nch * dm.na * dm.N;
+  bse_mixed32_kernel<NP><<<(int)(systems < sms ? systems : sms), M::kThreads, M::kSmem, c->stream>>>(
+      dm, ch0, nch, gg, gg + count, c->chi, c->kc, gdig_ptr(c), flags, mixed_check(c));
+  return cudaGetLastError();
 }
 
 // orders 33-64: one block of two ladder groups per SM
@@ -237,9 +219,8 @@ static cudaError_t launch_bse_mixed64(df_ctx* c, int channel_mask, int* flags) {
 cudaError_t launch_bse_mixed(df_ctx* c, int channel_mask, int* flags) {
   cudaError_t e;
   switch (mixed_np(c->dm.n_w)) {
-    case 8: e = launch_bse_mixed_np<8>(c, channel_mask, flags); break;
-    case 16: e = launch_bse_mixed_np<16>(c, channel_mask, flags); break;
-    case 32: e = launch_bse_mixed_np<32>(c, channel_mask, flags); break;
+    case 16: e = launch_bse_mixed32<16>(c, channel_mask, flags); break;
+    case 32: e = launch_bse_mixed32<32>(c, channel_mask, flags); break;
     case 64: e = launch_bse_mixed64(c, channel_mask, flags); break;
     case 128: e = launch_bse_mixed_large(c, channel_mask, flags); break;   // df_mixed_large.cu
     default: return cudaErrorInvalidValue;

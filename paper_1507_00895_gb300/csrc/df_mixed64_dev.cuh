@@ -55,11 +55,6 @@ constexpr int kM64TsLd = 65;                              // row stride of T (fl
 constexpr int kM64ELd = 66;                               // row stride of the exchange (float2)
 constexpr int kM64Acc = 32 * kDig;                        // TMEM columns of one 16-row block's accumulators
 
-// gamma's digits of one matrix in global memory, by padded order (0: none kept; orders > 64: df_mixed128_dev.cuh)
-__host__ __device__ constexpr size_t mixed_digit_bytes(int np) {
-  return np == 64 ? kM64DigBytes : (use_tc_residual(np) ? gdig_bytes(np) : 0);
-}
-
 // shared memory of a group, byte offsets
 constexpr int kM64Work = 0;          // S digits [kDig][32][64] fp16 | exchange | the sweep's rows
 constexpr int kM64WorkBytes = kDig * 32 * 128;

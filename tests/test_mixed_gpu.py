@@ -303,3 +303,23 @@ def test_mixed_orders_share_a_batch_class(df):
         for i, w in enumerate(ws):
             st, _ = oracle_first_pass(w)
             assert nrel(b.get_sigma(i), st.sigma) < TOL_SIGMA, w.n_w
+
+
+@pytest.mark.parametrize("n_w", [2, 6, 8, 10, 14, 16, 18, 24, 26, 30, 32])
+@pytest.mark.parametrize("wide", [False, True])
+def test_mixed_ladder_per_warp(df, n_w, wide):
+    """Orders up to 32 where the kernel's tiles end (padded orders 16 and 32, 8-column and 16-row
+    product tiles, one or two lanes per row), the same inputs and bound as for the orders above."""
+    test_mixed_two_ladder_blocks(df, n_w, wide)
+
+
+def test_mixed_small_orders_share_a_batch_class(df):
+    """Orders of one padded order in one queue; the points end inside a block's take, and a plane has
+    more ladders than a block has warps."""
+    ws = [I.half_filled_atom(f"b{n}", 1, 32, U=3.0 + 0.01 * n, beta=2.0, n_w=n, m_max=1)
+          for n in (2, 32, 16, 18, 10, 30, 24)]
+    with df.DualFermionBatch(ws, precision=df.DF_FP32_IR) as b:
+        b.iterate(1)
+        for i, w in enumerate(ws):
+            st, _ = oracle_first_pass(w)
+            assert nrel(b.get_sigma(i), st.sigma) < TOL_SIGMA, w.n_w
