@@ -152,322 +152,6 @@ chi_ladder_kernel(Dims dm, const double2* __restrict__ gam, const double2* __res
 }
 
 // ---------------------------------------------------------------------------
-// The same ladder term under DF_FP32_IR (n_w <= 64): x = D^-1 gamma L by
-// mixed-precision iterative refinement.  D = 1 - gamma_W diag(chi~_W(q)) is
-// factorised once in FP32 (complex64 in shared memory, row stride n + 1,
-// partial pivoting on |re| + |im|); then, from x = 0 and r = gamma L,
-//     D d = r / |r|   (the FP32 factors),   x += |r| d,   r = gamma L - D x
-// with x, r and the products gamma v in FP64 (D x = x - gamma (chi~ o x)).
-// Each step shrinks the error by about cond(D) 2^-24.  A system stops when
-// its correction d is below ir_tol |x| (max norms of |re| + |im|), or when
-// d times its ratio to the previous correction is (the error left after a
-// contracting step); it is handed back to the FP64 LU kernel (appended to
-// `redo`, count in redo[0], output not written here) on an exactly zero FP32
-// pivot, a non-finite value, a correction that did not halve, or after
-// max_steps solves.  128 threads: all of them run the rank-1 updates (one
-// column each, rows split in 128 / n groups; the owners of the next column
-// leave per-group pivot candidates, so that a column step takes two
-// barriers) and the FP64 row products (128 / n rounded down to a power of
-// two lanes per row; those of gamma L interleaved with the column steps);
-// warp 0 runs the FP32 triangular solves (two rows per lane in registers).
-// ---------------------------------------------------------------------------
-constexpr int kChiIrThreads = 128;
-constexpr int kChiIrMaxN = 64;
-
-struct ChiIrShared {
-  int perm[kChiIrMaxN];
-  double2 xs[kChiIrMaxN], lv[kChiIrMaxN], b[kChiIrMaxN], x[kChiIrMaxN], v[kChiIrMaxN], r[kChiIrMaxN];
-  float2 invd[kChiIrMaxN];
-  // per row group: the largest |re| + |im| of the next pivot column among the
-  // group's rows, its row (n when the group has none) and its value
-  float pabs[kChiIrThreads];
-  int prow[kChiIrThreads];
-  float2 pval[kChiIrThreads];
-  int bad, state;
-};
-
-// sum_j gamma_ij v_j for row i by `tpr` adjacent lanes (lane part of them
-// takes j = part mod tpr); every lane of the warp must call it, rows i >= n
-// contribute nothing.  The sum is complete in every lane of the group.
-__device__ __forceinline__ double2 chi_ir_rowdot(const double2* __restrict__ G, const double2* v, int n, int i,
-                                                 int part, int tpr) {
-  double2 s0 = mk(0.0, 0.0), s1 = mk(0.0, 0.0);
-  if (i < n) {
-    const double2* g = G + (size_t)i * n;
-    int j = part;
-    for (; j + tpr < n; j += 2 * tpr) {
-      s0 = cfma(__ldg(g + j), v[j], s0);
-      s1 = cfma(__ldg(g + j + tpr), v[j + tpr], s1);
-    }
-    if (j < n) s0 = cfma(__ldg(g + j), v[j], s0);
-  }
-  s0 = s0 + s1;
-  for (int o = tpr >> 1; o > 0; o >>= 1) {
-    s0.x += __shfl_xor_sync(0xffffffffu, s0.x, o);
-    s0.y += __shfl_xor_sync(0xffffffffu, s0.y, o);
-  }
-  return s0;
-}
-
-// 1/z in FP32 for the FP32 factorisation (a reciprocal of |z|^2: outside
-// ~1e-19 < |z| < 1e19 it gives 0 or non-finite values, and the system is
-// handed back by the refinement's checks)
-__device__ __forceinline__ float2 cinv_f32(float2 z) {
-  const float d = __frcp_rn(z.x * z.x + z.y * z.y);
-  return make_float2(z.x * d, -z.y * d);
-}
-
-__device__ __forceinline__ double warp_max(double v) {
-  for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;
-}
-
-__global__ void __launch_bounds__(kChiIrThreads, 5)
-chi_ladder_ir_kernel(Dims dm, const double2* __restrict__ gam, const float2* __restrict__ gam32,
-                     const double2* __restrict__ chi, const double2* __restrict__ Lb,
-                     const double2* __restrict__ chi0, double2* __restrict__ out, int* __restrict__ redo,
-                     int max_steps, double tol) {
-  extern __shared__ float2 A[];        // [n][n + 1]
-  __shared__ ChiIrShared sh;
-  const int n = dm.n_w, N = dm.N, nb = dm.nb, ld = n + 1;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  // rank-1 update / build map: column j, row group i0 of rpp
-  const int rpp = kChiIrThreads / n, j = tid % n, i0 = tid / n;
-  // row-product map: tpr lanes per row
-  int tpr = 1;
-  while (tpr < 32 && 2 * tpr * n <= kChiIrThreads) tpr *= 2;
-  const int ri = tid / tpr, rpart = tid % tpr;
-  const long systems = 2L * nb * N;
-  for (long sys = blockIdx.x; sys < systems; sys += gridDim.x) {
-    const int c = (int)(sys / ((long)nb * N));
-    const int rem = (int)(sys - (long)c * nb * N);
-    const int a = rem / N, q = rem - a * N;
-    const double2* G = gam + ((size_t)c * nb + a) * n * n;
-    const float2* G32 = gam32 + ((size_t)c * nb + a) * n * n;
-    for (int i = tid; i < n; i += kChiIrThreads) {
-      sh.xs[i] = chi[((size_t)a * n + i) * N + q];
-      sh.lv[i] = Lb[((size_t)a * n + i) * N + q];
-      sh.perm[i] = i;
-    }
-    if (tid == 0) sh.bad = 0;
-    __syncthreads();
-    // D in FP32 from gamma's leading FP32 words and FP32-rounded chi~ (only
-    // the factorisation uses it; the residuals take D from FP64 gamma); the
-    // threads of column 0 leave their row group's pivot candidate
-    if (i0 < rpp) {
-      const float2 xj = make_float2((float)sh.xs[j].x, (float)sh.xs[j].y);
-      float best = -1.f;
-      int brow = n;
-      float2 bval = make_float2(0.f, 0.f);
-      for (int i = i0; i < n; i += rpp) {
-        float2 t = cmul(__ldg(G32 + (size_t)i * n + j), xj);
-        t = make_float2((i == j ? 1.f : 0.f) - t.x, -t.y);
-        A[i * ld + j] = t;
-        if (j == 0 && cabs1(t) > best) { best = cabs1(t); brow = i; bval = t; }
-      }
-      if (j == 0) { sh.pabs[i0] = best; sh.prow[i0] = brow; sh.pval[i0] = bval; }
-    }
-    __syncthreads();
-    // ---- FP32 LU with partial pivoting, two barriers per column; the FP64
-    // row products b = gamma L run alongside, one term per column step, their
-    // loads issued a step ahead ----
-    double2 bacc = mk(0.0, 0.0), gnext = mk(0.0, 0.0);
-    if (ri < n && rpart < n) gnext = __ldg(G + (size_t)ri * n + rpart);
-    int npart = rpp < n ? rpp : n;         // row groups holding pivot candidates
-    for (int k = 0; k < n; ++k) {
-      // the pivot of column k from the row groups' candidates (every thread
-      // takes the same one: largest, then lowest row)
-      float best = -1.f;
-      int p = n;
-      float2 pv = make_float2(0.f, 0.f);
-      for (int g = 0; g < npart; ++g) {
-        const float v = sh.pabs[g];
-        const int rr = sh.prow[g];
-        if (v > best || (v == best && rr < p)) { best = v; p = rr; pv = sh.pval[g]; }
-      }
-      if (p >= n) { p = k; pv = make_float2(0.f, 0.f); }   // no candidate (NaN column): a zero pivot
-      const bool zero = (pv.x == 0.f && pv.y == 0.f);
-      const float2 inv = zero ? make_float2(0.f, 0.f) : cinv_f32(pv);
-      if (tid == 0) {
-        if (zero) sh.bad = 1;
-        sh.invd[k] = inv;
-        if (p != k) { const int t = sh.perm[k]; sh.perm[k] = sh.perm[p]; sh.perm[p] = t; }
-      }
-      // rows k and p exchanged (column k: the pivot on the diagonal, the old
-      // A_kk scaled into row p), the other multipliers of column k scaled
-      if (p != k && tid < n) {
-        if (tid == k) {
-          const float2 okk = A[k * ld + k];
-          A[k * ld + k] = pv;
-          A[p * ld + k] = cmul(okk, inv);
-        } else {
-          const float2 t = A[k * ld + tid];
-          A[k * ld + tid] = A[p * ld + tid];
-          A[p * ld + tid] = t;
-        }
-      }
-      if (tid > k && tid < n && tid != p) A[tid * ld + k] = cmul(A[tid * ld + k], inv);
-      __syncthreads();
-      // rank-1 update of the trailing m x m block, spread over all threads:
-      // thread = g m + jc takes column k + 1 + jc, rows k + 1 + g + ng t with
-      // ng = floor(128 / m) groups (the quotients in FP32: exact here, every
-      // true quotient is at least 0.5 / m from an integer); the threads of
-      // column k + 1 leave the next pivot candidates
-      const int m = n - k - 1;
-      if (m > 0) {
-        const float rcp = __frcp_rn((float)m);
-        const int ng = __float2int_rz(128.f * rcp + 0.5f * rcp);
-        const int g = __float2int_rz(((float)tid + 0.5f) * rcp);
-        npart = ng < m ? ng : m;
-        if (g < ng) {
-          const int jcol = k + 1 + (tid - g * m);
-          const bool cand = (jcol == k + 1);
-          const float2 u = A[k * ld + jcol];
-          float bb = -1.f;
-          int br = n;
-          float2 bv = make_float2(0.f, 0.f);
-          int r = k + 1 + g;
-          // rows in batches of four, all loads of a batch before its stores
-          // (the compiler cannot order them otherwise: columns k and jcol share A)
-          for (; r + 3 * ng < n; r += 4 * ng) {
-            float2 l[4], t[4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              l[e] = A[(r + e * ng) * ld + k];
-              t[e] = A[(r + e * ng) * ld + jcol];
-            }
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              t[e] = cfms(l[e], u, t[e]);
-              A[(r + e * ng) * ld + jcol] = t[e];
-            }
-            if (cand) {
-#pragma unroll
-              for (int e = 0; e < 4; ++e)
-                if (cabs1(t[e]) > bb) { bb = cabs1(t[e]); br = r + e * ng; bv = t[e]; }
-            }
-          }
-          for (; r < n; r += ng) {
-            const float2 t = cfms(A[r * ld + k], u, A[r * ld + jcol]);
-            A[r * ld + jcol] = t;
-            if (cand && cabs1(t) > bb) { bb = cabs1(t); br = r; bv = t; }
-          }
-          if (cand && g < m) {
-            sh.pabs[g] = bb;
-            sh.prow[g] = br;
-            sh.pval[g] = bv;
-          }
-        }
-      }
-      {
-        const int jj = rpart + tpr * k;
-        if (ri < n && jj < n) {
-          const double2 gv = gnext;
-          if (jj + tpr < n) gnext = __ldg(G + (size_t)ri * n + jj + tpr);
-          bacc = cfma(gv, sh.lv[jj], bacc);
-        }
-      }
-      __syncthreads();
-    }
-    for (int o = tpr >> 1; o > 0; o >>= 1) {
-      bacc.x += __shfl_xor_sync(0xffffffffu, bacc.x, o);
-      bacc.y += __shfl_xor_sync(0xffffffffu, bacc.y, o);
-    }
-    if (rpart == 0 && ri < n) {
-      sh.b[ri] = bacc;
-      sh.r[ri] = bacc;
-      sh.x[ri] = mk(0.0, 0.0);
-    }
-    __syncthreads();
-    // ---- refinement: state 0 going on, 1 converged, 2 handed back; every
-    // thread reads the state right after the barrier that follows its write,
-    // and warp 0 writes it again only after the next barrier ----
-    int state = sh.bad ? 2 : 0;
-    double dprev = 0.0;
-    for (int it = 0; state == 0; ++it) {
-      if (warp == 0) {
-        const bool h0 = lane < n, h1 = lane + 32 < n;
-        double rm = fmax(h0 ? cabs1(sh.r[sh.perm[lane]]) : 0.0, h1 ? cabs1(sh.r[sh.perm[lane + 32]]) : 0.0);
-        rm = warp_max(rm);
-        const double sc = rm > 0.0 ? 1.0 / rm : 0.0;
-        float2 y0 = make_float2(0.f, 0.f), y1 = y0;
-        if (h0) { const double2 t = sh.r[sh.perm[lane]]; y0 = make_float2((float)(t.x * sc), (float)(t.y * sc)); }
-        if (h1) { const double2 t = sh.r[sh.perm[lane + 32]]; y1 = make_float2((float)(t.x * sc), (float)(t.y * sc)); }
-        for (int k = 0; k < n - 1; ++k) {          // unit-lower forward substitution
-          const float2 src = k < 32 ? y0 : y1;
-          const float2 yk = make_float2(__shfl_sync(0xffffffffu, src.x, k & 31), __shfl_sync(0xffffffffu, src.y, k & 31));
-          if (lane > k && h0) y0 = cfms(A[lane * ld + k], yk, y0);
-          if (lane + 32 > k && h1) y1 = cfms(A[(lane + 32) * ld + k], yk, y1);
-        }
-        for (int k = n - 1; k >= 0; --k) {         // upper back substitution
-          const float2 src = k < 32 ? y0 : y1;
-          const float2 yk = make_float2(__shfl_sync(0xffffffffu, src.x, k & 31), __shfl_sync(0xffffffffu, src.y, k & 31));
-          const float2 xk = cmul(yk, sh.invd[k]);
-          if (lane == k) y0 = xk;
-          if (lane + 32 == k) y1 = xk;
-          if (lane < k) y0 = cfms(A[lane * ld + k], xk, y0);
-          if (lane + 32 < k) y1 = cfms(A[(lane + 32) * ld + k], xk, y1);
-        }
-        double dn = 0.0, xn = 0.0;
-        if (h0) {
-          const double2 d = mk((double)y0.x * rm, (double)y0.y * rm);
-          const double2 xv = sh.x[lane] + d;
-          sh.x[lane] = xv;
-          sh.v[lane] = cmul(sh.xs[lane], xv);
-          dn = cabs1(d);
-          xn = cabs1(xv);
-        }
-        if (h1) {
-          const double2 d = mk((double)y1.x * rm, (double)y1.y * rm);
-          const double2 xv = sh.x[lane + 32] + d;
-          sh.x[lane + 32] = xv;
-          sh.v[lane + 32] = cmul(sh.xs[lane + 32], xv);
-          dn = fmax(dn, cabs1(d));
-          xn = fmax(xn, cabs1(xv));
-        }
-        // NaN compares false: a non-finite value hands the system back
-        dn = warp_max(isfinite(dn) ? dn : INFINITY);
-        xn = warp_max(isfinite(xn) ? xn : INFINITY);
-        int st = 0;
-        if (!(dn < INFINITY) || !(xn < INFINITY)) st = 2;
-        else if (dn <= tol * xn) st = 1;
-        else if (it > 0 && dn > 0.5 * dprev) st = 2;
-        else if (it > 0 && dn * dn <= 0.5 * tol * xn * dprev) st = 1;
-        else if (it + 1 >= max_steps) st = 2;
-        dprev = dn;
-        if (st == 1) {                              // out = chi0 + L . x
-          double2 s2 = mk(0.0, 0.0);
-          if (h0) s2 = cfma(sh.lv[lane], sh.x[lane], s2);
-          if (h1) s2 = cfma(sh.lv[lane + 32], sh.x[lane + 32], s2);
-          for (int o = 16; o > 0; o >>= 1) {
-            s2.x += __shfl_xor_sync(0xffffffffu, s2.x, o);
-            s2.y += __shfl_xor_sync(0xffffffffu, s2.y, o);
-          }
-          if (lane == 0) {
-            const double2 c0 = chi0[(size_t)a * N + q];
-            out[((size_t)c * nb + a) * N + q] = mk(c0.x + s2.x, c0.y + s2.y);
-          }
-        }
-        if (lane == 0) sh.state = st;
-      }
-      __syncthreads();
-      state = sh.state;
-      if (state != 0) break;
-      {   // r = gamma L - x + gamma (chi~ o x)
-        const double2 s = chi_ir_rowdot(G, sh.v, n, ri, rpart, tpr);
-        if (rpart == 0 && ri < n) sh.r[ri] = sh.b[ri] - sh.x[ri] + s;
-      }
-      __syncthreads();
-    }
-    if (tid == 0 && state == 2) {
-      const int slot = atomicAdd(redo, 1);
-      redo[1 + slot] = (int)sys;
-    }
-    __syncthreads();
-  }
-}
-
-// ---------------------------------------------------------------------------
 // host launchers
 // ---------------------------------------------------------------------------
 
@@ -568,9 +252,8 @@ cudaError_t launch_bse_f64_list(df_ctx* c, const int* list) {
 
 // the ladder term of the susceptibilities for both channels: FP64 LU on the
 // persistent grid and LU scratch of the FP64 ladder kernel, or under
-// DF_FP32_IR the refinement kernel first (D from gamma's FP32 leading words,
-// the first array of the mixed-precision workspace) and the FP64 LU only for
-// the systems it hands back (redo: 1 + 2 nb N ints)
+// DF_FP32_IR (n_w <= 64) the refinement kernel of df_chi.cu first and the FP64 LU
+// only for the systems it hands back (redo: 1 + 2 nb N ints)
 cudaError_t launch_chi_ladder(df_ctx* c, const double2* Lb, const double2* chi0, double2* out, int* redo) {
   const Dims& dm = c->dm;
   const int n = dm.n_w;
@@ -581,23 +264,9 @@ cudaError_t launch_chi_ladder(df_ctx* c, const double2* Lb, const double2* chi0,
   if (e != cudaSuccess) return e;
   const long systems = 2L * dm.nb * dm.N;
   const int* list = nullptr;
-  if (c->opts.precision == DF_FP32_IR && n <= kChiIrMaxN && c->mixed_ws) {
-    const size_t ism = sizeof(float2) * (size_t)n * (n + 1);
-    e = cudaFuncSetAttribute((const void*)chi_ladder_ir_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ism);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute((const void*)chi_ladder_ir_kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
-                             (int)cudaSharedmemCarveoutMaxShared);
-    if (e != cudaSuccess) return e;
-    int sms = 0, per_sm = 0;
-    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device)) != cudaSuccess) return e;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void*)chi_ladder_ir_kernel, kChiIrThreads, ism);
-    if (e != cudaSuccess) return e;
-    if (per_sm < 1) per_sm = 1;
-    const long ig = (long)sms * per_sm;
+  if (c->opts.precision == DF_FP32_IR && n <= 64 && c->mixed_ws) {
     if ((e = cudaMemsetAsync(redo, 0, sizeof(int), c->stream)) != cudaSuccess) return e;
-    chi_ladder_ir_kernel<<<(int)(systems < ig ? systems : ig), kChiIrThreads, ism, c->stream>>>(
-        dm, c->gam, (const float2*)c->mixed_ws, c->chi, Lb, chi0, out, redo, c->opts.ir_max_steps, c->opts.ir_tol);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if ((e = launch_chi_ladder_ir(c, Lb, chi0, out, redo)) != cudaSuccess) return e;
     list = redo;
   }
   const int grid = (int)(systems < c->bse_grid ? systems : c->bse_grid);

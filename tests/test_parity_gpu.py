@@ -388,6 +388,22 @@ def test_susceptibility_refined(df, name, kw):
         assert np.array_equal(d.susceptibility(), chi64)
 
 
+@pytest.mark.parametrize("n_w", [2, 6, 8, 14, 30, 32, 34, 46, 58, 62, 64])
+def test_susceptibility_refined_orders(df, n_w):
+    # the refinement kernel's padded orders (32, 64) and column groups (4, 8 with a remainder), complex
+    # vertices without symmetry, more systems per (channel, W) than ladders per block; the refinement
+    # stops at 1e-13 of the solution, so 1e-11 of the largest chi leaves it two digits for L . x
+    w = I.random_nonsymmetric(n_w, 1, 1, 16, seed=n_w, scale=0.5)
+    with df.DualFermion.from_workload(w, eig_mode=0) as d:
+        d.iterate(1)
+        sigma = d.get_sigma()
+        chi64 = d.susceptibility()
+    with df.DualFermion.from_workload(w, precision=df.DF_FP32_IR, eig_mode=0) as d:
+        d.set_sigma(sigma)
+        chi = d.susceptibility()
+    assert 0 < np.max(np.abs(chi - chi64)) < 1e-11 * np.max(np.abs(chi64))
+
+
 @pytest.mark.parametrize("K", [1, 3])
 def test_radius_extension(df, K):
     # outside the ladder radius (|lambda| up to 25): flagged systems take the
