@@ -167,11 +167,18 @@ __global__ void batch_setup_elem_kernel(const PointDev* __restrict__ pts, int p)
                           (gridDim.x * blockDim.x) >> 5, threadIdx.x & 31);
 }
 
+// Sigma~ = 0 and G~ of it, one block per plane of the points' extended boxes (start: their first blocks)
 __global__ void __launch_bounds__(kFftThreads)
-batch_setup_dyson_kernel(const PointDev* __restrict__ pts, int p) {
+batch_setup_dyson_kernel(const PointDev* __restrict__ pts, const long* __restrict__ start, int npts) {
   extern __shared__ double2 sm[];
+  const int p = find_segment(start, npts, blockIdx.x);
   const PointDev& P = pts[p];
-  dyson_ifft_plane(P.dm, blockIdx.x, P.g0, P.sigma, P.gk, P.gr, sm, sm + P.dm.nk / 2);
+  const int e = (int)(blockIdx.x - start[p]), i = e - P.dm.m_max;
+  if (i >= 0 && i < P.dm.n_w)
+    for (int r = threadIdx.x; r < P.dm.N; r += blockDim.x) P.sigma[(size_t)i * P.dm.N + r] = mk(0.0, 0.0);
+  if (e == 0 && threadIdx.x < 4) P.flags[threadIdx.x] = 0;
+  __syncthreads();
+  dyson_ifft_plane(P.dm, e, P.g0, P.sigma, P.gk, P.gr, sm, sm + P.dm.nk / 2);
 }
 
 // ---- ladder stages ---------------------------------------------------------
@@ -463,7 +470,8 @@ struct df_batch {
   size_t arena_bytes = 0;
   // FFT-stage tables
   long *d_plane_start = nullptr, *d_box_start = nullptr;
-  long total_planes = 0, total_box = 0;
+  long* d_ext_start = nullptr;                 // first planes of the points' extended boxes
+  long total_planes = 0, total_box = 0, total_ext = 0;
   size_t fft_smem1 = 0, fft_smem2 = 0;
   std::vector<LadderGroup> groups;
   unsigned long long* d_counters = nullptr;   // one per ladder group
@@ -858,32 +866,36 @@ df_status df_batch_init(df_batch** out, int npts, const df_point* pts, int preci
     goto bad;
   }
   {
-    size_t fs = 0;
-    for (int i = 0; i < npts; ++i)
-      fs = std::max(fs, fft_smem_bytes(b->host_pts[i].dm.nk, b->host_pts[i].dm.N, 1));
-    cudaFuncSetAttribute((const void*)batch_setup_dyson_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fs);
+    std::vector<long> es(npts + 1, 0);
     for (int i = 0; i < npts; ++i) {
       const Dims& dm = b->host_pts[i].dm;
+      es[i + 1] = es[i] + dm.ne;
+      b->fft_smem1 = std::max(b->fft_smem1, fft_smem_bytes(dm.nk, dm.N, 1));
       batch_setup_elem_kernel<<<64, 256, 0, b->stream>>>(b->d_pts, i);
-      batch_setup_dyson_kernel<<<dm.ne, kFftThreads, fft_smem_bytes(dm.nk, dm.N, 1), b->stream>>>(b->d_pts, i);
     }
+    b->total_ext = es[npts];
+    BALLOC(b->d_ext_start, sizeof(long) * (npts + 1), "extended-box table");
+    cudaMemcpy(b->d_ext_start, es.data(), sizeof(long) * (npts + 1), cudaMemcpyHostToDevice);
+    cudaFuncSetAttribute((const void*)batch_setup_dyson_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)b->fft_smem1);
+    batch_setup_dyson_kernel<<<(unsigned)b->total_ext, kFftThreads, b->fft_smem1, b->stream>>>(b->d_pts, b->d_ext_start,
+                                                                                             npts);
     if ((e = cudaGetLastError()) != cudaSuccess) { st = bfail(b, DF_ERR_CUDA, "batch set-up", e); goto bad; }
   }
 
   // ---- work tables ----
   {
     std::vector<long> ps(npts + 1, 0), bs(npts + 1, 0);
-    size_t f1 = 0, f2 = 0;
+    size_t f2 = 0;
     for (int i = 0; i < npts; ++i) {
       const Dims& dm = b->host_pts[i].dm;
       ps[i + 1] = ps[i] + (long)dm.nb * dm.n_w;
       bs[i + 1] = bs[i] + dm.n_w;
-      f1 = std::max(f1, fft_smem_bytes(dm.nk, dm.N, 1));
       f2 = std::max(f2, fft_smem_bytes(dm.nk, dm.N, 2));
     }
     b->total_planes = ps[npts];
     b->total_box = bs[npts];
-    b->fft_smem1 = f1;
+    const size_t f1 = b->fft_smem1;
     b->fft_smem2 = f2;
     BALLOC(b->d_plane_start, sizeof(long) * (npts + 1), "plane table");
     BALLOC(b->d_box_start, sizeof(long) * (npts + 1), "box table");
@@ -987,6 +999,7 @@ void df_batch_destroy(df_batch* b) {
   cudaFree(b->d_pts);
   cudaFree(b->d_out);
   cudaFree(b->d_plane_start);
+  cudaFree(b->d_ext_start);
   cudaFree(b->d_box_start);
   cudaFree(b->d_counters);
   cudaFree(b->ws);
@@ -1037,15 +1050,11 @@ df_status df_batch_reset(df_batch* b) {
     PointDev& P = b->host_pts[i];
     P.active = 1;
     P.resid = -1.0;
-    B_CUDA(b, cudaMemsetAsync(P.sigma, 0, sizeof(double2) * P.dm.n_w * P.dm.N, b->stream), "reset");
-    B_CUDA(b, cudaMemsetAsync(P.flags, 0, sizeof(int) * 4, b->stream), "reset");
   }
   B_CUDA(b, cudaMemcpyAsync(b->d_pts, b->host_pts.data(), sizeof(PointDev) * b->npts, cudaMemcpyHostToDevice,
                             b->stream), "reset");
-  for (int i = 0; i < b->npts; ++i) {
-    const Dims& dm = b->host_pts[i].dm;
-    batch_setup_dyson_kernel<<<dm.ne, kFftThreads, fft_smem_bytes(dm.nk, dm.N, 1), b->stream>>>(b->d_pts, i);
-  }
+  batch_setup_dyson_kernel<<<(unsigned)b->total_ext, kFftThreads, b->fft_smem1, b->stream>>>(b->d_pts, b->d_ext_start,
+                                                                                           b->npts);
   B_CUDA(b, cudaGetLastError(), "reset");
   B_CUDA(b, cudaStreamSynchronize(b->stream), "reset");
   b->passes = 0;
