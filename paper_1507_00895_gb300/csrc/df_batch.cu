@@ -224,18 +224,23 @@ batch_bse_f64_list_kernel(const PointDev* __restrict__ pts, const int* __restric
   extern __shared__ double2 sm[];
   __shared__ BseF64Shared sh;
   const int count = redo[0];
-  for (int s = blockIdx.x; s < count; s += gridDim.x) {
-    const int code = redo[1 + s];
+  // a short list is spread over the grid as ranges of right-hand sides (bse_f64_kernel)
+  const int parts = count > 0 && (int)gridDim.x > count ? min((int)gridDim.x / count, 8) : 1;
+  for (int s = blockIdx.x; s < count * parts; s += gridDim.x) {
+    const int code = redo[1 + s / parts], part = s % parts;
     const PointDev& P = pts[code >> 24];
     const Dims& dm = P.ldm;
+    const int nc = min(dm.n_w, kListChunk), chunks = (dm.n_w + nc - 1) / nc, cpp = (chunks + parts - 1) / parts;
+    const int jb = part * cpp * nc, je = min(jb + cpp * nc, dm.n_w);
+    if (jb >= je) continue;
     const int sys = code & 0xFFFFFF;
     const int c = sys / (dm.nb * dm.N), rem = sys - c * dm.nb * dm.N;
     const int a = rem / dm.N, q = rem - a * dm.N;
-    const int nc = default_nc_dev(dm.n_w);
-    const bool lu_smem = dm.n_w <= kLuSmemOrder;
+    const bool lu_smem = dm.n_w <= kListSmemOrder;
     const BseSmem L = bse_layout(dm.n_w, nc, lu_smem);
     double2* LU = lu_smem ? sm + L.lu : ws + blockIdx.x * ws_stride;
-    bse_f64_system(dm, c, a, q, nc, P.gam, P.gg, P.lchi, P.lkc, LU, sm + L.y, sm + L.xs, sm + L.invu, sh, P.flags);
+    bse_f64_system(dm, c, a, q, nc, P.gam, P.gg, P.lchi, P.lkc, LU, sm + L.y, sm + L.xs, sm + L.invu, sh, P.flags, 0,
+                   nullptr, jb, je);
   }
 }
 
@@ -966,12 +971,15 @@ df_status df_batch_init(df_batch** out, int npts, const df_point* pts, int preci
         if (g.mixed)
           for (int p : g.order) {
             const int n = b->host_pts[p].dm.n_w;
-            sm_max = std::max(sm_max, sizeof(double2) * (size_t)bse_layout(n, default_nc(n), n <= kLuSmemOrder).total);
+            sm_max = std::max(sm_max, sizeof(double2) * (size_t)bse_layout(n, std::min(n, kListChunk), n <= kListSmemOrder).total);
           }
       b->redo_smem = sm_max;
-      b->redo_grid = b->sms * kLuScratchPerSm;   // blocks beyond the list's count exit at once
       e = cudaFuncSetAttribute((const void*)batch_bse_f64_list_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                (int)sm_max);
+      int per = 0;
+      if (e == cudaSuccess)
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, batch_bse_f64_list_kernel, kBseThreads, sm_max);
+      b->redo_grid = b->sms * std::min(std::max(per, 1), kLuScratchPerSm);   // the scratch has that many slices
       if (e != cudaSuccess) { st = bfail(b, DF_ERR_CUDA, "hand-back kernel", e); goto bad; }
     }
   }

@@ -231,22 +231,23 @@ cudaError_t launch_bse(df_ctx* c, int channel_mask) {
 cudaError_t launch_bse_f64_list(df_ctx* c, const int* list) {
   const Dims& dm = c->dm;
   const int n = dm.n_w;
-  const int nc = bse_chunk(n) < 16 ? bse_chunk(n) : 16;   // 16-column ranges to spread (fits the default layout)
-  const size_t smem = bse_smem_bytes(n);
+  const int nc = n < kListChunk ? n : kListChunk;
+  const bool in_smem = n <= kListSmemOrder;
+  const size_t smem = sizeof(double2) * (size_t)bse_layout(n, nc, in_smem).total;
   int sms = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
-  cudaError_t e = cudaFuncSetAttribute(bse_lu_in_smem(n) ? (const void*)bse_f64_kernel<true>
-                                                         : (const void*)bse_f64_kernel<false>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const void* fn = in_smem ? (const void*)bse_f64_kernel<true> : (const void*)bse_f64_kernel<false>;
+  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  if (bse_lu_in_smem(n))
-    bse_f64_kernel<true><<<c->bse_grid, kBseThreads, smem, c->stream>>>(dm, 0, 2, nc, c->gam, gg_ptr(c), c->chi,
-                                                                        c->kc, nullptr, flag_ptr(c), 0, nullptr, list,
-                                                                        sms);
+  int per_sm = 0;
+  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kBseThreads, smem)) != cudaSuccess) return e;
+  const int grid = in_smem ? sms * (per_sm < 1 ? 1 : per_sm) : c->bse_grid;   // (the scratch has bse_grid slices)
+  if (in_smem)
+    bse_f64_kernel<true><<<grid, kBseThreads, smem, c->stream>>>(dm, 0, 2, nc, c->gam, gg_ptr(c), c->chi, c->kc, nullptr,
+                                                                 flag_ptr(c), 0, nullptr, list, grid);
   else
-    bse_f64_kernel<false><<<c->bse_grid, kBseThreads, smem, c->stream>>>(dm, 0, 2, nc, c->gam, gg_ptr(c), c->chi,
-                                                                         c->kc, lu_ws_ptr(c), flag_ptr(c), 0, nullptr,
-                                                                         list, sms);
+    bse_f64_kernel<false><<<grid, kBseThreads, smem, c->stream>>>(dm, 0, 2, nc, c->gam, gg_ptr(c), c->chi, c->kc,
+                                                                  lu_ws_ptr(c), flag_ptr(c), 0, nullptr, list, grid);
   return cudaGetLastError();
 }
 

@@ -323,3 +323,27 @@ def test_mixed_small_orders_share_a_batch_class(df):
         for i, w in enumerate(ws):
             st, _ = oracle_first_pass(w)
             assert nrel(b.get_sigma(i), st.sigma) < TOL_SIGMA, w.n_w
+
+
+@pytest.mark.parametrize("n_w", [12, 40, 48, 80, 96, 98, 128])
+def test_single_hand_back_is_split(df, n_w):
+    """One nearly singular ladder (as above): a list this short is split into ranges of 16 right-hand sides
+    (remainders at 40, 48 and 98), in shared memory up to order 96.  In a batch and on a handle the
+    result is the FP64 path's for that ladder, so Sigma~ is within the mixed path's bound of it although the
+    ladder's FP32 factorisation has no digit left."""
+    w = I.workload("paper_u20", nk=4, n_w=n_w, m_max=0)
+    st, _ = oracle_first_pass(w)
+    gd, gm = O.channel_vertices(w.gamma_uu, w.gamma_ud)
+    ev = np.linalg.eigvals(gm[0] * st.chi[0, :, 5][None, :])
+    gm = gm * ((1.0 - 1e-9) / ev[np.argmax(np.abs(ev))])
+    w.gamma_uu, w.gamma_ud = (gd + gm) / 2, (gd - gm) / 2
+    with df.DualFermion.from_workload(w) as d64, df.DualFermion.from_workload(w, precision=df.DF_FP32_IR) as d:
+        for h in (d64, d):
+            h.bubble()
+            h.bse(3)
+        assert d.ladder_stats()[1] >= 1
+        assert np.array_equal(d.get_kernel()[1, 0, :, 5], d64.get_kernel()[1, 0, :, 5])
+    with df.DualFermionBatch([w]) as b64, df.DualFermionBatch([w], precision=df.DF_FP32_IR) as b:
+        b64.iterate(1)
+        b.iterate(1)
+        assert nrel(b.get_sigma(0), b64.get_sigma(0)) < TOL_SIGMA
