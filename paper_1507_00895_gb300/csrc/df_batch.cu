@@ -80,7 +80,7 @@ batch_bubble_kernel(const PointDev* __restrict__ pts, const long* __restrict__ s
   const int local = (int)(blockIdx.x - start[p]);
   const int a = local / P.dm.n_w, i = local - a * P.dm.n_w;
   if (P.refl && a < P.dm.m_max) return;             // W < 0: not needed under the reflection
-  bubble_plane(P.dm, a, i, P.gr, P.chi, sm, sm + P.dm.nk / 2);
+  bubble_plane<false>(P.dm, a, i, P.gr, P.chi, sm, sm + P.dm.nk / 2);
 }
 
 __global__ void __launch_bounds__(kFftThreads)
@@ -92,7 +92,7 @@ batch_sigma_prod_kernel(const PointDev* __restrict__ pts, const long* __restrict
   const int local = (int)(blockIdx.x - start[p]);
   const int a = local / P.dm.n_w, i = local - a * P.dm.n_w;
   if (P.refl && a < P.dm.m_max) return;             // W < 0: summed by the reflection
-  sigma_prod_plane(P.dm, a, i, P.kc, P.gr, P.prod, sm, sm + P.dm.nk / 2);
+  sigma_prod_plane<false>(P.dm, a, i, P.kc, P.gr, P.prod, sm, sm + P.dm.nk / 2);
 }
 
 __global__ void __launch_bounds__(kFftThreads)
@@ -103,7 +103,7 @@ batch_sigma_dyson_kernel(const PointDev* __restrict__ pts, const long* __restric
   const PointDev& P = pts[p];
   if (!P.active) return;
   const int i = (int)(blockIdx.x - start[p]);
-  sigma_dyson_plane(P.dm, i, P.mix, P.prod, P.g0, P.sigma, P.gk, P.gr, P.red, sm, sm + P.dm.nk / 2,
+  sigma_dyson_plane<false>(P.dm, i, P.mix, P.prod, P.g0, P.sigma, P.gk, P.gr, P.red, sm, sm + P.dm.nk / 2,
                     sm + P.dm.nk / 2 + P.dm.N, red_sm, P.refl);
 }
 
@@ -178,7 +178,7 @@ batch_setup_dyson_kernel(const PointDev* __restrict__ pts, const long* __restric
     for (int r = threadIdx.x; r < P.dm.N; r += blockDim.x) P.sigma[(size_t)i * P.dm.N + r] = mk(0.0, 0.0);
   if (e == 0 && threadIdx.x < 4) P.flags[threadIdx.x] = 0;
   __syncthreads();
-  dyson_ifft_plane(P.dm, e, P.g0, P.sigma, P.gk, P.gr, sm, sm + P.dm.nk / 2);
+  dyson_ifft_plane<false>(P.dm, e, P.g0, P.sigma, P.gk, P.gr, sm, sm + P.dm.nk / 2);
 }
 
 // ---- ladder stages ---------------------------------------------------------

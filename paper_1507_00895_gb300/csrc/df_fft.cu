@@ -19,52 +19,58 @@ __global__ void init_g0_kernel(Dims dm, const double2* __restrict__ g, const dou
     init_g0_elem(dm, idx, g, delta, g0, gk);
 }
 
+template <bool R8>
 __global__ void __launch_bounds__(kFftThreads)
 dyson_ifft_kernel(Dims dm, int first, const double2* __restrict__ g0, const double2* __restrict__ sigma,
                   double2* __restrict__ gk, double2* __restrict__ gr) {
   extern __shared__ double2 sm[];
-  dyson_ifft_plane(dm, first + blockIdx.x, g0, sigma, gk, gr, sm, sm + dm.nk / 2);
+  dyson_ifft_plane<R8>(dm, first + blockIdx.x, g0, sigma, gk, gr, sm, sm + dm.nk / 2);
 }
 
+template <bool R8>
 __global__ void __launch_bounds__(kFftThreads)
 bubble_kernel(Dims dm, const double2* __restrict__ gr, double2* __restrict__ chi) {
   extern __shared__ double2 sm[];
   const int b = blockIdx.x / dm.n_w, i = blockIdx.x - b * dm.n_w, a = dm.a0 + b;
-  bubble_plane(dm, a, i, gr, chi, sm, sm + dm.nk / 2);
+  bubble_plane<R8>(dm, a, i, gr, chi, sm, sm + dm.nk / 2);
 }
 
+template <bool R8>
 __global__ void __launch_bounds__(kFftThreads)
 sigma_prod_kernel(Dims dm, const double2* __restrict__ kc, const double2* __restrict__ gr,
                   double2* __restrict__ prod) {
   extern __shared__ double2 sm[];
   const int b = blockIdx.x / dm.n_w, i = blockIdx.x - b * dm.n_w, a = dm.a0 + b;
-  sigma_prod_plane(dm, a, i, kc, gr, prod, sm, sm + dm.nk / 2);
+  sigma_prod_plane<R8>(dm, a, i, kc, gr, prod, sm, sm + dm.nk / 2);
 }
 
+template <bool R8>
 __global__ void __launch_bounds__(kFftThreads)
 sigma_dyson_kernel(Dims dm, double mix, const double2* __restrict__ prod, const double2* __restrict__ g0,
                    double2* __restrict__ sigma, double2* __restrict__ gk, double2* __restrict__ gr,
                    double* __restrict__ red, int refl) {
   extern __shared__ double2 sm[];
   __shared__ double red_sm[32];
-  sigma_dyson_plane(dm, blockIdx.x, mix, prod, g0, sigma, gk, gr, red, sm, sm + dm.nk / 2,
+  sigma_dyson_plane<R8>(dm, blockIdx.x, mix, prod, g0, sigma, gk, gr, red, sm, sm + dm.nk / 2,
                     sm + dm.nk / 2 + dm.N, red_sm, refl);
 }
 
 // The Omega split: this problem's share of Eq. sd, out[i][k] = (T/2) FFT[sum over
 // its bosonic planes of prod[W][i]](k), before mixing and Dyson
+template <bool R8>
 __global__ void __launch_bounds__(kFftThreads)
 sigma_partial_kernel(Dims dm, const double2* __restrict__ prod, double2* __restrict__ out, int refl) {
   extern __shared__ double2 sm[];
   const int i = blockIdx.x;
   double2* s = sm + dm.nk / 2;
-  sigma_sum_plane(dm, i, prod, sm, s, refl);
+  sigma_sum_plane<R8>(dm, i, prod, sm, s, refl);
   const double pref = 0.5 * dm.T;
-  for (int k = threadIdx.x; k < dm.N; k += blockDim.x) out[(size_t)i * dm.N + k] = cscale(s[k], pref);
+  for (int k = threadIdx.x; k < dm.N; k += blockDim.x) out[(size_t)i * dm.N + k] = cscale(s[fft_out<R8>(dm, k)], pref);
 }
 
 // ... and the rest of the pass from the sum of every share: mixing, residual
 // partials, Eq. dyson, G~(r)
+template <bool R8>
 __global__ void __launch_bounds__(kFftThreads)
 sigma_finish_kernel(Dims dm, double mix, const double2* __restrict__ total, const double2* __restrict__ g0,
                     double2* __restrict__ sigma, double2* __restrict__ gk, double2* __restrict__ gr,
@@ -74,9 +80,9 @@ sigma_finish_kernel(Dims dm, double mix, const double2* __restrict__ total, cons
   const int i = blockIdx.x;
   double2* s = sm + dm.nk / 2;
   load_twiddles(sm, dm.nk);
-  for (int k = threadIdx.x; k < dm.N; k += blockDim.x) s[k] = total[(size_t)i * dm.N + k];
+  for (int k = threadIdx.x; k < dm.N; k += blockDim.x) s[fft_out<R8>(dm, k)] = total[(size_t)i * dm.N + k];
   __syncthreads();
-  sigma_finish_plane(dm, i, mix, 1.0, s, g0, sigma, gk, gr, red, sm, s + dm.N, red_sm);
+  sigma_finish_plane<R8>(dm, i, mix, 1.0, s, g0, sigma, gk, gr, red, sm, s + dm.N, red_sm);
 }
 
 // Section "Resulting observables", per box element (w, k): Eq. sigma_lat
@@ -153,6 +159,9 @@ static size_t fft_smem(const Dims& dm, int planes) { return fft_smem_bytes(dm.nk
 static cudaError_t set_smem(const void* fn, size_t bytes) {
   return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
+// a plane kernel's instance for the lattice (fft_radix8)
+#define FFT_KERNEL(dm, name) (fft_radix8(dm) ? name<true> : name<false>)
+#define FFT_SMEM(dm, name, bytes) set_smem(fft_radix8(dm) ? (const void*)name<true> : (const void*)name<false>, bytes)
 
 cudaError_t launch_init_g0(df_ctx* c) {
   const Dims& dm = c->dm;
@@ -165,9 +174,10 @@ cudaError_t launch_init_g0(df_ctx* c) {
 cudaError_t launch_dyson_ifft(df_ctx* c, int first_plane, int n_planes) {
   const Dims& dm = c->dm;
   const size_t sm = fft_smem(dm, 1);
-  cudaError_t e = set_smem((const void*)dyson_ifft_kernel, sm);
+  cudaError_t e = FFT_SMEM(dm, dyson_ifft_kernel, sm);
   if (e != cudaSuccess) return e;
-  dyson_ifft_kernel<<<n_planes, kFftThreads, sm, c->stream>>>(dm, first_plane, c->g0, c->sigma, c->gk, c->gr);
+  FFT_KERNEL(dm, dyson_ifft_kernel)<<<n_planes, kFftThreads, sm, c->stream>>>(dm, first_plane, c->g0, c->sigma, c->gk,
+                                                                         c->gr);
   return cudaGetLastError();
 }
 
@@ -185,9 +195,9 @@ static Dims pass_planes(const df_ctx* c) {
 cudaError_t launch_bubble(df_ctx* c, int all_planes) {
   const Dims dm = all_planes ? c->dm : pass_planes(c);
   const size_t sm = fft_smem(dm, 1);
-  cudaError_t e = set_smem((const void*)bubble_kernel, sm);
+  cudaError_t e = FFT_SMEM(dm, bubble_kernel, sm);
   if (e != cudaSuccess) return e;
-  bubble_kernel<<<dm.na * dm.n_w, kFftThreads, sm, c->stream>>>(dm, c->gr, c->chi);
+  FFT_KERNEL(dm, bubble_kernel)<<<dm.na * dm.n_w, kFftThreads, sm, c->stream>>>(dm, c->gr, c->chi);
   return cudaGetLastError();
 }
 
@@ -213,12 +223,12 @@ cudaError_t launch_obs_bubbles(df_ctx* c, double2* planes, double2* P, double2* 
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   size_t sm = fft_smem(dm, 1);
-  if ((e = set_smem((const void*)dyson_ifft_kernel, sm)) != cudaSuccess) return e;
-  if ((e = set_smem((const void*)bubble_kernel, sm)) != cudaSuccess) return e;
-  dyson_ifft_kernel<<<dm.ne, kFftThreads, sm, c->stream>>>(dm, 0, Gp, nullptr, nullptr, Gr);
-  dyson_ifft_kernel<<<dm.ne, kFftThreads, sm, c->stream>>>(dm, 0, Fp, nullptr, nullptr, Fr);
-  bubble_kernel<<<dm.nb * dm.n_w, kFftThreads, sm, c->stream>>>(dm, Gr, P);
-  bubble_kernel<<<dm.nb * dm.n_w, kFftThreads, sm, c->stream>>>(dm, Fr, L);
+  if ((e = FFT_SMEM(dm, dyson_ifft_kernel, sm)) != cudaSuccess) return e;
+  if ((e = FFT_SMEM(dm, bubble_kernel, sm)) != cudaSuccess) return e;
+  FFT_KERNEL(dm, dyson_ifft_kernel)<<<dm.ne, kFftThreads, sm, c->stream>>>(dm, 0, Gp, nullptr, nullptr, Gr);
+  FFT_KERNEL(dm, dyson_ifft_kernel)<<<dm.ne, kFftThreads, sm, c->stream>>>(dm, 0, Fp, nullptr, nullptr, Fr);
+  FFT_KERNEL(dm, bubble_kernel)<<<dm.nb * dm.n_w, kFftThreads, sm, c->stream>>>(dm, Gr, P);
+  FFT_KERNEL(dm, bubble_kernel)<<<dm.nb * dm.n_w, kFftThreads, sm, c->stream>>>(dm, Fr, L);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   const int nq = dm.nb * dm.N;
   sum_w_kernel<<<(nq + 255) / 256, 256, 0, c->stream>>>(dm, P, chi0);
@@ -230,12 +240,12 @@ cudaError_t launch_sigma_partial(df_ctx* c, double2* out) {
   const Dims& dm = c->dm;
   const Dims pp = pass_planes(c);
   size_t sm = fft_smem(dm, 1);
-  cudaError_t e = set_smem((const void*)sigma_prod_kernel, sm);
+  cudaError_t e = FFT_SMEM(dm, sigma_prod_kernel, sm);
   if (e != cudaSuccess) return e;
-  sigma_prod_kernel<<<pp.na * pp.n_w, kFftThreads, sm, c->stream>>>(pp, c->kc, c->gr, c->prod);
+  FFT_KERNEL(dm, sigma_prod_kernel)<<<pp.na * pp.n_w, kFftThreads, sm, c->stream>>>(pp, c->kc, c->gr, c->prod);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  if ((e = set_smem((const void*)sigma_partial_kernel, sm)) != cudaSuccess) return e;
-  sigma_partial_kernel<<<dm.n_w, kFftThreads, sm, c->stream>>>(dm, c->prod, out, c->opts.symmetry == 2);
+  if ((e = FFT_SMEM(dm, sigma_partial_kernel, sm)) != cudaSuccess) return e;
+  FFT_KERNEL(dm, sigma_partial_kernel)<<<dm.n_w, kFftThreads, sm, c->stream>>>(dm, c->prod, out, c->opts.symmetry == 2);
   return cudaGetLastError();
 }
 
@@ -243,9 +253,10 @@ cudaError_t launch_sigma_partial(df_ctx* c, double2* out) {
 cudaError_t launch_sigma_finish(df_ctx* c, const double2* total, double mix) {
   const Dims& dm = c->dm;
   const size_t sm = fft_smem(dm, 2);
-  cudaError_t e = set_smem((const void*)sigma_finish_kernel, sm);
+  cudaError_t e = FFT_SMEM(dm, sigma_finish_kernel, sm);
   if (e != cudaSuccess) return e;
-  sigma_finish_kernel<<<dm.n_w, kFftThreads, sm, c->stream>>>(dm, mix, total, c->g0, c->sigma, c->gk, c->gr, c->red);
+  FFT_KERNEL(dm, sigma_finish_kernel)<<<dm.n_w, kFftThreads, sm, c->stream>>>(dm, mix, total, c->g0, c->sigma, c->gk, c->gr,
+                                                                         c->red);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   residual_reduce_kernel<<<1, kFftThreads, 0, c->stream>>>(dm.n_w, c->red);
   return cudaGetLastError();
@@ -255,13 +266,13 @@ cudaError_t launch_sigma(df_ctx* c, double mix) {
   const Dims& dm = c->dm;
   const Dims pp = pass_planes(c);
   size_t sm = fft_smem(dm, 1);
-  cudaError_t e = set_smem((const void*)sigma_prod_kernel, sm);
+  cudaError_t e = FFT_SMEM(dm, sigma_prod_kernel, sm);
   if (e != cudaSuccess) return e;
-  sigma_prod_kernel<<<pp.na * pp.n_w, kFftThreads, sm, c->stream>>>(pp, c->kc, c->gr, c->prod);
+  FFT_KERNEL(dm, sigma_prod_kernel)<<<pp.na * pp.n_w, kFftThreads, sm, c->stream>>>(pp, c->kc, c->gr, c->prod);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   sm = fft_smem(dm, 2);
-  if ((e = set_smem((const void*)sigma_dyson_kernel, sm)) != cudaSuccess) return e;
-  sigma_dyson_kernel<<<dm.n_w, kFftThreads, sm, c->stream>>>(dm, mix, c->prod, c->g0, c->sigma, c->gk,
+  if ((e = FFT_SMEM(dm, sigma_dyson_kernel, sm)) != cudaSuccess) return e;
+  FFT_KERNEL(dm, sigma_dyson_kernel)<<<dm.n_w, kFftThreads, sm, c->stream>>>(dm, mix, c->prod, c->g0, c->sigma, c->gk,
                                                              c->gr, c->red, c->opts.symmetry == 2);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   residual_reduce_kernel<<<1, kFftThreads, 0, c->stream>>>(dm.n_w, c->red);
