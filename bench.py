@@ -44,10 +44,10 @@ PEAKS_PATH = os.path.join(ROOT, "MEASURED_PEAKS.json")
 FLUSH_BYTES = 256 << 20
 # DRAM bytes (read + write) per launch of the ladder kernel from one ncu capture
 # of that kernel on this workload (None once the kernel changes)
-NCU_TRAFFIC = {"bse_f64_kernel": None, "bse_mixed_kernel": 19867904}
+NCU_TRAFFIC = {"bse_f64_kernel": None, "bse_mixed64_kernel": None}
 # tensor-pipe share of the mixed ladder kernel's cycles (ncu sm__pipe_tensor_cycles_active,
 # the committed profile of the same kernel; None once the kernel changes)
-NCU_TENSOR_PIPE = {"bse_mixed_kernel": 0.082}
+NCU_TENSOR_PIPE = {"bse_mixed64_kernel": None}
 
 
 def measured_alu_peaks(df):
@@ -547,7 +547,7 @@ def large_order_bench(df, I, passes: int = 2):
         out[name] = {"s_per_pass": wall, "ladder_ms_per_pass": bse_ms,
                      "fp64_equivalent_TFLOP_per_s": fp64_eq / (bse_ms * 1e-3) / 1e12,
                      "kernel": "bse_f64_kernel" if prec == df.DF_FP64 else
-                               "bse_tcr_kernel (tcgen05 Gauss-Jordan sweep and digit residual)"}
+                               "bse_mixed128_kernel (Gauss-Jordan sweep in registers, digit product on tcgen05)"}
     out["err_fp32ir_vs_fp64_first_pass"] = float(np.max(np.abs(sig["fp32ir"] - sig["fp64"]))
                                                  / np.max(np.abs(sig["fp64"])))
     with df.DualFermion.from_workload(w, precision=df.DF_FP32_IR, mixed_sweep=1) as d:
@@ -889,15 +889,15 @@ def run_ours(args):
                     "issued_flop_per_launch": systems_per_launch * algo_flop, "launch_ms": bse_avg_s * 1e3}
         else:
             pk = peaks["fp32_gflops"]
-            # issued: the FP32 Gauss-Jordan sweep of [D | gamma] (2 n^3 complex MACs) plus the
-            # residual product gamma Y (n^3 complex MACs, as exact bf16 digit products on tcgen05)
-            issued = 8.0 * 3.0 * n ** 3
+            # issued: the FP32 Gauss-Jordan sweep of D (n^3 complex MACs) plus the product
+            # T = S gamma (n^3 complex MACs, as exact FP16 digit products on tcgen05)
+            issued = 8.0 * 2.0 * n ** 3
             roof = {"bound": "alu", "achieved": achieved, "peak": pk, "unit": "GFLOP/s", "frac": achieved / pk,
-                    "traffic": NCU_TRAFFIC.get("bse_mixed_kernel"), "kernel": "bse_mixed_kernel",
+                    "traffic": NCU_TRAFFIC.get("bse_mixed64_kernel"), "kernel": "bse_mixed64_kernel",
                     "peak_source": "FP32 pipe, " + peaks["source"], "flop_model": flop_model,
                     "flop_per_launch": systems_per_launch * algo_flop,
                     "issued_flop_per_launch": systems_per_launch * issued, "launch_ms": bse_avg_s * 1e3,
-                    "tensor_pipe_frac": NCU_TENSOR_PIPE.get("bse_mixed_kernel")}
+                    "tensor_pipe_frac": NCU_TENSOR_PIPE.get("bse_mixed64_kernel")}
         if prec != df.DF_FP64:
             worst, back = d.ladder_stats()
             roof["ladder_error_control"] = {"worst_rho2_last_step": worst, "handed_back_to_fp64": back,

@@ -263,7 +263,7 @@ df_status df_lattice_observables(df_ctx* c, double* sigma_lat, double* g_lat, in
  *   L_{W,w}(q) = -(T/N) sum_k frakG_{w,k} frakG_{w+W,k+q},
  *   frakG = G~ (G0~ + g) / G0~,
  * G from Eq. glat, Gamma = (1 - gamma chi~)^-1 gamma (Eq. lin_alg_inv, FP64
- * LU with partial pivoting; under DF_FP32_IR an FP32 LU refined in FP64
+ * LU with partial pivoting; under DF_FP32_IR an FP32 inverse refined in FP64
  * until ir_tol, each system that does not get there within ir_max_steps
  * solves taken again by the FP64 LU) with chi~ the dual bubble of the current G~
  * (recomputed here; df_get_chi returns it afterwards), w over the box.  The
@@ -333,9 +333,8 @@ typedef struct df_point {
 
 typedef struct df_batch df_batch;
 
-/* precision: DF_FP64 for every point, or DF_FP32_IR for every point (n_w <= 64
- * by the register-tile kernel, larger orders by the shared-memory Gauss-Jordan
- * one), with the per-ladder error control of DF_FP32_IR at ladder_tol = 1e-9:
+/* precision: DF_FP64 for every point, or DF_FP32_IR for every point, with the
+ * per-ladder error control of DF_FP32_IR at ladder_tol = 1e-9:
  * ladders above it are solved again by the FP64 LU in the same pass.
  * npts in [1, 4096] (DF_FP32_IR: [1, 127]).  tol > 0: a point stops once its
  * residual r <= tol.  stream may be NULL (the batch then creates its own). */

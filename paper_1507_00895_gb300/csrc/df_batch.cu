@@ -56,9 +56,6 @@ struct PointDev {
   int* flags;    // [4]
 };
 
-// the FP64 right-hand-side chunk of an order (as default_nc on the host)
-__device__ __forceinline__ int default_nc_dev(int n) { return n <= 32 ? n : (n <= 64 ? 32 : 16); }
-
 __device__ __forceinline__ int find_segment(const long* start, int nseg, long x) {
   // largest k with start[k] <= x (start[0] = 0, start[nseg] = total)
   int lo = 0, hi = nseg - 1;

@@ -531,8 +531,7 @@ def warmstart_sigma(d: "DualFermion", y, mean, sd, kmap):
 
 
 def mixed_supported(n_w: int) -> bool:
-    """DF_FP32_IR covers every ladder order a handle or a batch takes: n_w <= 64 with
-    [D | RHS] in registers, up to 128 by the shared-memory Gauss-Jordan kernel."""
+    """DF_FP32_IR covers every ladder order a handle or a batch takes."""
     return 2 <= n_w <= 128
 
 

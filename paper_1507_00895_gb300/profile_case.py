@@ -4,11 +4,11 @@
 
 Cases (inputs from paper_1507_00895_gb300.inputs; every stage runs in libdf):
   mixed64  2D 16x16, n_w = 64, N_W = 15, DF_FP32_IR: bubble + both ladder
-           channels (7,680 ladders of order 64, bse_mixed_kernel)
+           channels (7,680 ladders of order 64, bse_mixed64_kernel)
   bench64  the benchmark's workload itself (2D 32x32, n_w = 64, N_W = 15),
            DF_FP32_IR: bubble + both ladder channels (30,720 ladders)
   tc96     3D 8^3, n_w = 96, N_W = 5, DF_FP32_IR: bubble + both ladder channels
-           (5,120 ladders of order 96, the tensor-core Gauss-Jordan kernel)
+           (5,120 ladders of order 96, bse_mixed128_kernel)
   simt96   the same with the CUDA-core Gauss-Jordan (mixed_sweep = 1)
   fft3d    3D 16^3, n_w = 96, N_W = 21 (the 3D workload at its stated size), FP64:
            Eq. dual_bubble and Eq. sd + Dyson only (the lattice-FFT kernels;
