@@ -354,12 +354,13 @@ batch_bse_mixed64_kernel(const PointDev* __restrict__ pts, const int* __restrict
       if (P.active) {
         const int c = (int)(plane / dm.na), a = dm.a0 + (int)(plane % dm.na), key = c * dm.nb + a;
         const long id = (long)k * 256 + key;
-        if (id != cur) m64_load_digits(blk, P.gdig + (size_t)key * kM64DigBytes);
+        const unsigned char* gd = P.gdig + (size_t)key * kM64DigBytes;
+        if (id != cur) m64_load_digits(blk, gd);
         cur = id;
         const size_t mat = (size_t)key * dm.n_w * dm.n_w;
         for (long x = s + blk.gr.g; x < end; x += kM64Groups)
-          m64_system(dm, c, a, (int)(x - base), P.gam_hi + mat, P.gam_lo + mat, P.gg_hi + mat, P.gg_lo + mat, P.lchi,
-                     P.lkc, P.flags, blk.gr, smem_u32(sm64), reinterpret_cast<const float*>(sm64 + kM64Gexp),
+          m64_system(dm, c, a, (int)(x - base), reinterpret_cast<const float4*>(gd + kM64Shared), P.gg_hi + mat,
+                     P.gg_lo + mat, P.lchi, P.lkc, P.flags, blk.gr, smem_u32(sm64), reinterpret_cast<const float*>(sm64 + kM64Gexp),
                      batch_check(redo, order[k]));
       }
       s = end;
@@ -404,7 +405,7 @@ batch_bse_mixed128_kernel(const PointDev* __restrict__ pts, const int* __restric
       const int c = (int)(plane / dm.na), a = dm.a0 + (int)(plane % dm.na), key = c * dm.nb + a;
       const size_t mat = (size_t)key * dm.n_w * dm.n_w;
       L.ld = (dm.n_w + 31) / 32 * 32;
-      ok = m128_system(dm, c, a, (int)(local - plane * dm.N), P.gam_hi + mat, P.gam_lo + mat, P.gg_hi + mat,
+      ok = m128_system(dm, c, a, (int)(local - plane * dm.N), P.gg_hi + mat,
                        P.gg_lo + mat, P.gdig + (size_t)key * kM128DigBytes, P.lchi, P.lkc, P.flags, L, st,
                        batch_check(redo, order[k]));
       if (!ok) {

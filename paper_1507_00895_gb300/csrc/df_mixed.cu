@@ -65,8 +65,7 @@ bse_mixed32_kernel(Dims dm, int ch0, int nch, const float2* __restrict__ gg_hi, 
 // Orders 33-64: one contiguous range of systems per block, split where
 // (channel, W) changes; the two groups of a block take its systems in turn.
 __global__ void __launch_bounds__(kM64Threads, 1)
-bse_mixed64_kernel(Dims dm, int ch0, int nch, const float2* __restrict__ gam_hi, const float2* __restrict__ gam_lo,
-                   const float2* __restrict__ gg_hi, const float2* __restrict__ gg_lo,
+bse_mixed64_kernel(Dims dm, int ch0, int nch, const float2* __restrict__ gg_hi, const float2* __restrict__ gg_lo,
                    const double2* __restrict__ chi, double2* __restrict__ kc, const unsigned char* __restrict__ gdig,
                    int* __restrict__ flags, MixedCheck mc) {
   extern __shared__ __align__(1024) unsigned char sm64[];
@@ -85,11 +84,12 @@ bse_mixed64_kernel(Dims dm, int ch0, int nch, const float2* __restrict__ gam_hi,
   while (s < s1) {
     const long plane = s / N, end = min(s1, (plane + 1) * N);
     const int c = ch0 + (int)(plane / na), a = dm.a0 + (int)(plane % na), key = c * nb + a;
-    m64_load_digits(blk, gdig + (size_t)key * kM64DigBytes);
+    const unsigned char* gd = gdig + (size_t)key * kM64DigBytes;
+    m64_load_digits(blk, gd);
     const size_t mat = (size_t)key * dm.n_w * dm.n_w;
     for (long x = s + blk.gr.g; x < end; x += kM64Groups)
-      m64_system(dm, c, a, (int)(x - plane * N), gam_hi + mat, gam_lo + mat, gg_hi + mat, gg_lo + mat, chi, kc, flags,
-                 blk.gr, smem_u32(sm64), reinterpret_cast<const float*>(sm64 + kM64Gexp), mc);
+      m64_system(dm, c, a, (int)(x - plane * N), reinterpret_cast<const float4*>(gd + kM64Shared), gg_hi + mat,
+                 gg_lo + mat, chi, kc, flags, blk.gr, smem_u32(sm64), reinterpret_cast<const float*>(sm64 + kM64Gexp), mc);
     s = end;
   }
   m64_teardown(blk);
@@ -209,7 +209,7 @@ static cudaError_t launch_bse_mixed64(df_ctx* c, int channel_mask, int* flags) {
   const int nch = (channel_mask & 1) + ((channel_mask >> 1) & 1), ch0 = (channel_mask & 1) ? 0 : 1;
   const long pairs = ((long)nch * dm.na * dm.N + kM64Groups - 1) / kM64Groups;
   bse_mixed64_kernel<<<(int)(pairs < sms ? pairs : sms), kM64Threads, kM64Smem, c->stream>>>(
-      dm, ch0, nch, hi, hi + count, hi + 2 * count, hi + 3 * count, c->chi, c->kc, gdig_ptr(c), flags, mc);
+      dm, ch0, nch, hi + 2 * count, hi + 3 * count, c->chi, c->kc, gdig_ptr(c), flags, mc);
   return cudaGetLastError();
 }
 

@@ -16,12 +16,13 @@
 // Tile t's finishing lanes 64 t .. 64 t + 63 are the columns j themselves: the
 // digit rows are [gamma_re; gamma_im] in tile 0 and [gamma_im; gamma_re] in tile 1.
 //
-// Cycles per ladder (instrumented copy, n = 96 / 128): D 21k / 28k, sweep 118k / 182k
+// Cycles per ladder (instrumented copy, n = 96 / 128): D 21k / 28k (with n-strided reads of gamma; its
+// words by column since: 4.00 -> 3.89 and 30.1 -> 29.1 ms below), sweep 118k / 182k
 // (the updates run near the FMA rate), digits 12k / 16k, products with their
 // stream 128k / 211k (92k / 150k of it the stream alone: 1.8 / 3.1 MB per ladder, ~6 TB/s from
-// L2 over all SMs), fold, exchange and R 33k / 44k.  Measured: 3,630 ladders of order 96 4.1 ms (9.3 with
+// L2 over all SMs), fold, exchange and R 33k / 44k.  Measured: 3,630 ladders of order 96 3.9 ms (9.3 with
 // the sweep of [D | gamma] on the tensor cores and a base-128 digit residual streamed in
-// 8-column blocks), 17,952 of order 128 32 ms (96.8 with the sweep on the tensor cores and a
+// 8-column blocks), 17,952 of order 128 29 ms (96.8 with the sweep on the tensor cores and a
 // double-float residual on the CUDA cores).  The CUDA-core sweep also leaves a
 // smaller residual than three-piece BF16 products: worst rho^2 on the 3D workload
 // 1.5e-12 (4.6e-10).
@@ -33,7 +34,8 @@ namespace df {
 constexpr int kM128Threads = 512;
 constexpr int kM128Issuer = 0, kM128Streamer = 32;        // the threads that issue the MMAs and stream the digits
 constexpr int kM128Piece = 128 * 64;                      // 128 digit rows x 32 K, 64-byte swizzled
-constexpr int kM128DigBytes = 2 * kDig * 4 * kM128Piece + 128 * 4;   // a matrix's digits and column weights
+constexpr int kM128Words = 2 * kDig * 4 * kM128Piece + 128 * 4;      // a matrix's digits and column weights,
+constexpr int kM128DigBytes = kM128Words + 128 * 128 * 16;           // then its words [column][row] (hi, lo)
 constexpr int kM128MaxRing = 10;
 constexpr int kM128Atom = kDig * 32 * 128;                // S digits of one 64-wide K block: [kDig][32][64] fp16
 constexpr int kM128TmemT = 256;                           // TMEM columns: accumulators [0, 192), T re [256, 384), im [384, 512)
@@ -98,7 +100,9 @@ __device__ __forceinline__ void gamma_digits_cols128(int n, int count, const dou
     if (m > 0.0) frexp(m, &e);                            // m < 2^e
     if (lane == 0) colw[j] = e > -1000 ? (e - 8 > 127 ? __int_as_float(0x7f800000) : pow2f(e - 8)) : 0.f;
     const int tile = j >> 6;
+    float4* words = reinterpret_cast<float4*>(O + kM128Words) + j * 128;
     for (int l = lane; l < 128; l += 32) {
+      words[l] = split_words(l < n && j < n ? G[(size_t)l * n + j] : mk(0.0, 0.0));
       double re = 0.0, im = 0.0;
       if (l < n && j < n && e > -1000) {
         re = ldexp(G[(size_t)l * n + j].x, 8 - e);
@@ -167,8 +171,7 @@ __device__ __forceinline__ bool m128_stream(int count, int& at, int nkat, const 
 // One ladder.  Gh, Gl, GGh, GGl: the (hi, lo) words of gamma and gamma o gamma^T of this
 // (channel, W), gdig gamma's digits and column weights.  Returns false when a bounded wait gave
 // up (the same in every thread).
-__device__ __forceinline__ bool m128_system(const Dims& dm, int c, int a, int q, const float2* __restrict__ Gh,
-                                            const float2* __restrict__ Gl, const float2* __restrict__ GGh,
+__device__ __forceinline__ bool m128_system(const Dims& dm, int c, int a, int q, const float2* __restrict__ GGh,
                                             const float2* __restrict__ GGl,
                                             const unsigned char* __restrict__ gdig,
                                             const double2* __restrict__ chi, double2* __restrict__ kc,
@@ -203,25 +206,21 @@ __device__ __forceinline__ bool m128_system(const Dims& dm, int c, int a, int q,
   m128_sync();
   {
     // ---- D into registers ----
+    const float4* words = reinterpret_cast<const float4*>(gdig + kM128Words);
     float2 A[4][kPanel];
     const int c0 = kPanel * warp;
 #pragma unroll
     for (int ii = 0; ii < 4; ++ii) {
       const int r = lane + 32 * ii;
+      float4 g[kPanel];
 #pragma unroll
-      for (int p = 0; p < 4; ++p) {
-        const bool in = r < n && c0 + 2 * p < n;            // n is even: pairs of columns are 16-byte aligned
-        const float4 hv = in ? __ldg(reinterpret_cast<const float4*>(Gh + r * n + c0 + 2 * p)) : make_float4(0.f, 0.f, 0.f, 0.f);
-        const float4 lv = in ? __ldg(reinterpret_cast<const float4*>(Gl + r * n + c0 + 2 * p)) : make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int c2 = 0; c2 < kPanel; ++c2) g[c2] = __ldg(words + (c0 + c2) * 128 + r);   // rows across the lanes
 #pragma unroll
-        for (int e = 0; e < 2; ++e) {
-          const int col = c0 + 2 * p + e;
-          const float2 gh = e ? make_float2(hv.z, hv.w) : make_float2(hv.x, hv.y);
-          const float2 gl = e ? make_float2(lv.z, lv.w) : make_float2(lv.x, lv.y);
-          float sr = (r == col) ? 1.f : 0.f, lr = 0.f, si = 0.f, li = 0.f;
-          cdf_fma(sr, lr, si, li, make_float2(-gh.x, -gh.y), make_float2(-gl.x, -gl.y), chih[col], chil[col]);
-          A[ii][2 * p + e] = make_float2(sr + lr, si + li);
-        }
+      for (int c2 = 0; c2 < kPanel; ++c2) {
+        const int col = c0 + c2;
+        float sr = (r == col) ? 1.f : 0.f, lr = 0.f, si = 0.f, li = 0.f;
+        cdf_fma(sr, lr, si, li, make_float2(-g[c2].x, -g[c2].y), make_float2(-g[c2].z, -g[c2].w), chih[col], chil[col]);
+        A[ii][c2] = make_float2(sr + lr, si + li);
       }
     }
     // ---- in-place Gauss-Jordan sweep (the factors in S's place, the rows on their way in the digits') ----

@@ -32,7 +32,7 @@
 // overlap the other's arithmetic.  Bound by latency: the pivot chain (~60k of a
 // group's 119k cycles per ladder at n = 64) with four warps per scheduler,
 // issue slots 45% busy, 108k warp instructions per ladder.  Measured, 30,720
-// ladders of order 64: 6.45 ms (11.2 ms with one ladder per block, [D | gamma]
+// ladders of order 64: 6.12 ms (6.45 with rows of gamma read across n-strided lanes, 11.2 ms with one ladder per block, [D | gamma]
 // swept and the residual gamma - D X0 formed after it); 1,536 of order 48, whose
 // padding is no longer swept: 0.25 ms (0.57).  Tried: packed f32x2 multiply-adds in the
 // update (40k cycles against 34k), a panel on one warp (1000 cycles a step
@@ -50,7 +50,8 @@ constexpr int kM64Group = 256;                            // threads per ladder
 constexpr int kM64Groups = 2;
 constexpr int kM64Threads = kM64Group * kM64Groups;
 constexpr int kM64Slice = 128 * 128;                      // one gamma digit slice: [gamma_re; gamma_im] columns j, K = l
-constexpr int kM64DigBytes = kDig * kM64Slice + 64 * 4;   // a matrix's digits and column weights in global memory
+constexpr int kM64Shared = kDig * kM64Slice + 64 * 4;     // a matrix's digits and column weights: kept in shared memory
+constexpr int kM64DigBytes = kM64Shared + 64 * 64 * 16;   // then its words [column][row] (hi, lo), in global memory
 constexpr int kM64TsLd = 65;                              // row stride of T (float2)
 constexpr int kM64ELd = 66;                               // row stride of the exchange (float2)
 constexpr int kM64Acc = 32 * kDig;                        // TMEM columns of one 16-row block's accumulators
@@ -96,6 +97,12 @@ __device__ __forceinline__ unsigned dig_pair(unsigned m0, unsigned m1) {
   return *reinterpret_cast<const unsigned*>(&h);
 }
 
+// v's FP32 (hi, lo) words
+__device__ __forceinline__ float4 split_words(double2 v) {
+  const float hx = (float)v.x, hy = (float)v.y;
+  return make_float4(hx, hy, (float)(v.x - (double)hx), (float)(v.y - (double)hy));
+}
+
 // gamma's digits, `count` n x n matrices (FP64, n <= 64) -> out[count][kM64DigBytes]:
 // per column j with the exponent bound e_j over both parts (|gamma_lj| < 2^e_j) the
 // weight 2^(e_j - 8) (0 for a zero column), digits at [slice][j (re) or 64 + j (im)][l], 128-byte
@@ -114,7 +121,9 @@ __device__ __forceinline__ void gamma_digits_cols(int n, int count, const double
     int e = -1000;
     if (m > 0.0) frexp(m, &e);                            // m < 2^e
     if (lane == 0) colw[j] = e > -1000 ? (e - 8 > 127 ? __int_as_float(0x7f800000) : pow2f(e - 8)) : 0.f;
+    float4* words = reinterpret_cast<float4*>(out + (size_t)mtx * kM64DigBytes + kM64Shared) + j * 64;
     for (int l = lane; l < 64; l += 32) {
+      words[l] = split_words(l < n && j < n ? G[(size_t)l * n + j] : mk(0.0, 0.0));
       double re = 0.0, im = 0.0;
       if (l < n && j < n && e > -1000) {
         re = ldexp(G[(size_t)l * n + j].x, 8 - e);
@@ -265,9 +274,9 @@ struct M64Group {
 // One ladder by the kM64Group threads of group gr.  gdig: the block's gamma
 // digits in shared memory (their address), gwt the columns' weights 2^(e_j - 8).
 // Writes kc[c][a][:][q].
-__device__ __forceinline__ void m64_system(const Dims& dm, int c, int a, int q, const float2* __restrict__ Gh,
-                                           const float2* __restrict__ Gl, const float2* __restrict__ GGh,
-                                           const float2* __restrict__ GGl, const double2* __restrict__ chi,
+__device__ __forceinline__ void m64_system(const Dims& dm, int c, int a, int q, const float4* __restrict__ words,
+                                           const float2* __restrict__ GGh, const float2* __restrict__ GGl,
+                                           const double2* __restrict__ chi,
                                            double2* __restrict__ kc, int* __restrict__ flags, M64Group& gr,
                                            unsigned gdig, const float* gwt, const MixedCheck& mc) {
   const int n = dm.n_w, N = dm.N, nb = dm.nb;
@@ -297,29 +306,21 @@ __device__ __forceinline__ void m64_system(const Dims& dm, int c, int a, int q, 
     if (i == 0) *badw = 0;
   }
   {
-    // ---- D into registers (gamma's words loaded ahead of chi~; n is even, so pairs of columns are 16-byte aligned) ----
+    // ---- D into registers (gamma's words loaded ahead of chi~, rows across the lanes) ----
     float2 A[2][kPanel];
     {
       const int c0 = kPanel * warp;
-      float4 h[2][4], l[2][4];
+      float4 g[2][kPanel];
 #pragma unroll
-      for (int ii = 0; ii < 2; ++ii) {
-        const int r = lane + 32 * ii;
+      for (int ii = 0; ii < 2; ++ii)
 #pragma unroll
-        for (int p = 0; p < 4; ++p) {
-          const bool in = r < n && c0 + 2 * p < n;
-          h[ii][p] = in ? __ldg(reinterpret_cast<const float4*>(Gh + r * n + c0 + 2 * p)) : make_float4(0.f, 0.f, 0.f, 0.f);
-          l[ii][p] = in ? __ldg(reinterpret_cast<const float4*>(Gl + r * n + c0 + 2 * p)) : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-      }
+        for (int jj = 0; jj < kPanel; ++jj) g[ii][jj] = __ldg(words + (c0 + jj) * 64 + lane + 32 * ii);
       m64_sync(gr.g);
 #pragma unroll
       for (int ii = 0; ii < 2; ++ii)
 #pragma unroll
         for (int jj = 0; jj < kPanel; ++jj) {
-          const float4 hv = h[ii][jj >> 1], lv = l[ii][jj >> 1];
-          const float2 gh = (jj & 1) ? make_float2(hv.z, hv.w) : make_float2(hv.x, hv.y);
-          const float2 gl = (jj & 1) ? make_float2(lv.z, lv.w) : make_float2(lv.x, lv.y);
+          const float2 gh = make_float2(g[ii][jj].x, g[ii][jj].y), gl = make_float2(g[ii][jj].z, g[ii][jj].w);
           float sr = (lane + 32 * ii == c0 + jj) ? 1.f : 0.f, lr = 0.f, si = 0.f, li = 0.f;
           cdf_fma(sr, lr, si, li, make_float2(-gh.x, -gh.y), make_float2(-gl.x, -gl.y), chih[c0 + jj], chil[c0 + jj]);
           A[ii][jj] = make_float2(sr + lr, si + li);
@@ -703,7 +704,7 @@ __device__ __forceinline__ void m64_load_digits(const M64Block& b, const unsigne
   __syncthreads();
   const uint4* src = reinterpret_cast<const uint4*>(gdig);
   uint4* dst = reinterpret_cast<uint4*>(b.sm);
-  for (int i = threadIdx.x; i < kM64DigBytes / 16; i += kM64Threads) dst[i] = __ldg(src + i);
+  for (int i = threadIdx.x; i < kM64Shared / 16; i += kM64Threads) dst[i] = __ldg(src + i);
   fence_async_smem();
   __syncthreads();
 }

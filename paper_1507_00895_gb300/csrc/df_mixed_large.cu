@@ -49,8 +49,7 @@ __global__ void gamma_digits128_kernel(int n, int count, const double2* __restri
 }
 
 __global__ void __launch_bounds__(kM128Threads, 1)
-bse_mixed128_kernel(Dims dm, int ch0, int nch, const float2* __restrict__ gam_hi, const float2* __restrict__ gam_lo,
-                    const float2* __restrict__ gg_hi, const float2* __restrict__ gg_lo,
+bse_mixed128_kernel(Dims dm, int ch0, int nch, const float2* __restrict__ gg_hi, const float2* __restrict__ gg_lo,
                     const double2* __restrict__ chi, double2* __restrict__ kc, const unsigned char* __restrict__ gdig,
                     int* __restrict__ flags, MixedCheck mc) {
   extern __shared__ __align__(1024) unsigned char sm128[];
@@ -71,7 +70,7 @@ bse_mixed128_kernel(Dims dm, int ch0, int nch, const float2* __restrict__ gam_hi
     const long plane = s / N;
     const int c = ch0 + (int)(plane / na), a = dm.a0 + (int)(plane % na), key = c * nb + a;
     const size_t mat = (size_t)key * n * n;
-    if (!m128_system(dm, c, a, (int)(s - plane * N), gam_hi + mat, gam_lo + mat, gg_hi + mat, gg_lo + mat,
+    if (!m128_system(dm, c, a, (int)(s - plane * N), gg_hi + mat, gg_lo + mat,
                      gdig + (size_t)key * kM128DigBytes, chi, kc, flags, L, st, mc)) {
       m128_drain(st, L);
       if (threadIdx.x == 0) atomicOr(flags, kFlagTcTimeout);
@@ -120,7 +119,7 @@ static cudaError_t launch_bse_mixed128(df_ctx* c, int channel_mask, int* flags) 
   const int nch = (channel_mask & 1) + ((channel_mask >> 1) & 1), ch0 = (channel_mask & 1) ? 0 : 1;
   const long systems = (long)nch * dm.na * dm.N;
   bse_mixed128_kernel<<<(int)(systems < sms ? systems : sms), kM128Threads, smem, c->stream>>>(
-      dm, ch0, nch, hi, hi + count, hi + 2 * count, hi + 3 * count, c->chi, c->kc, digits128_ptr(c), flags,
+      dm, ch0, nch, hi + 2 * count, hi + 3 * count, c->chi, c->kc, digits128_ptr(c), flags,
       mixed_check(c));
   return cudaGetLastError();
 }
