@@ -66,6 +66,35 @@ SMALL = [
 ]
 
 
+@pytest.mark.parametrize("dim,nk", [(2, 32), (2, 64), (3, 16), (4, 8)])
+def test_large_plane_transforms(df, dim, nk):
+    """The lattices whose transforms run in radix-8/4 passes (from 1024 points on), every axis length they
+    take, inputs without symmetry.  Each transform is ~20 roundings deep, 1e-12 of the largest value leaves
+    two digits over that; Sigma~ has the ladders behind it (TOL64)."""
+    w = I.random_nonsymmetric(4, 1, dim, nk, seed=nk + dim, scale=0.3)
+    st, _, _ = oracle_first_pass(w)
+    with df.DualFermion.from_workload(w, eig_mode=0) as d, df.DualFermion.from_workload(w, eig_mode=0) as e:
+        d.bubble()
+        assert nrel(d.get_chi(), st.chi) < 1e-12
+        d.bse(3)
+        d.sigma()
+        sig = d.get_sigma()
+        assert nrel(sig, st.sigma) < TOL64
+        g = st.g0_ext.copy()
+        box = slice(w.m_max, w.m_max + w.n_w)
+        g[box] = 1.0 / (1.0 / g[box] - sig)
+        assert nrel(d.get_gtilde(), g) < 1e-12
+        e.bubble()                                          # the split's kernels
+        e.bse(3)
+        e.sigma_finish(e.sigma_partial())
+        assert nrel(e.get_sigma(), sig) < 1e-12
+        assert nrel(e.get_gtilde(), g) < 1e-12
+        e.set_sigma(2.0 * sig)                              # Dyson from a given Sigma~
+        e.bubble()
+        g[box] = 1.0 / (1.0 / st.g0_ext[box] - 2.0 * sig)
+        assert nrel(e.get_gtilde(), g) < 1e-12
+
+
 @pytest.mark.parametrize("name,kw", SMALL)
 def test_first_pass_all_stages(df, name, kw):
     w = I.workload(name, **kw)
