@@ -17,7 +17,7 @@ constexpr int kBseThreads = 256;
 constexpr int kLuSmemOrder = 40;
 // The hand-back lists are short, so that a ladder's own latency counts, not the blocks per
 // SM: shared memory as far as it reaches, and ranges of kListChunk right-hand sides
-// spread over the idle blocks.  Measured, order 64: 208 ladders 831 -> 587 us, about 30 390 -> 370 us
+// spread over the idle blocks.  Measured, order 64: about 150 ladders 831 -> 587 us, about 30 390 -> 370 us
 // (the FP64 pipe of one SM needs 175 us for one range: the factorisation is repeated per range);
 // a 24-point batch's list 657 -> 366 us (it was not split before).
 constexpr int kListSmemOrder = 96;
