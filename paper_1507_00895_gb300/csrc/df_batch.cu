@@ -784,6 +784,13 @@ df_status df_batch_init(df_batch** out, int npts, const df_point* pts, int preci
     e = cudaMalloc((void**)&(ptr), (bytes));                                        \
     if (e != cudaSuccess) { st = bfail(b, DF_ERR_OOM, what, e); goto bad; }         \
   } while (0)
+// host tables go up on the batch's own stream: a copy on the legacy stream may still be on its way when it
+// returns (pageable source), and nothing orders a non-blocking stream after it
+#define BTRY(call, what)                                                            \
+  do {                                                                              \
+    if ((e = (call)) != cudaSuccess) { st = bfail(b, DF_ERR_CUDA, what, e); goto bad; } \
+  } while (0)
+#define BCOPY(dst, src, bytes, what) BTRY(cudaMemcpyAsync((dst), (src), (bytes), cudaMemcpyHostToDevice, b->stream), what)
   BALLOC(b->arena, total, "batch arena");
   for (int i = 0; i < npts; ++i) {
     PointDev& P = b->host_pts[i];
@@ -878,9 +885,9 @@ df_status df_batch_init(df_batch** out, int npts, const df_point* pts, int preci
     }
     b->total_ext = es[npts];
     BALLOC(b->d_ext_start, sizeof(long) * (npts + 1), "extended-box table");
-    cudaMemcpy(b->d_ext_start, es.data(), sizeof(long) * (npts + 1), cudaMemcpyHostToDevice);
-    cudaFuncSetAttribute((const void*)batch_setup_dyson_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)b->fft_smem1);
+    BCOPY(b->d_ext_start, es.data(), sizeof(long) * (npts + 1), "extended-box table");
+    BTRY(cudaFuncSetAttribute((const void*)batch_setup_dyson_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)b->fft_smem1), "set-up smem attribute");
     batch_setup_dyson_kernel<<<(unsigned)b->total_ext, kFftThreads, b->fft_smem1, b->stream>>>(b->d_pts, b->d_ext_start,
                                                                                              npts);
     if ((e = cudaGetLastError()) != cudaSuccess) { st = bfail(b, DF_ERR_CUDA, "batch set-up", e); goto bad; }
@@ -902,11 +909,14 @@ df_status df_batch_init(df_batch** out, int npts, const df_point* pts, int preci
     b->fft_smem2 = f2;
     BALLOC(b->d_plane_start, sizeof(long) * (npts + 1), "plane table");
     BALLOC(b->d_box_start, sizeof(long) * (npts + 1), "box table");
-    cudaMemcpy(b->d_plane_start, ps.data(), sizeof(long) * (npts + 1), cudaMemcpyHostToDevice);
-    cudaMemcpy(b->d_box_start, bs.data(), sizeof(long) * (npts + 1), cudaMemcpyHostToDevice);
-    cudaFuncSetAttribute((const void*)batch_bubble_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)f1);
-    cudaFuncSetAttribute((const void*)batch_sigma_prod_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)f1);
-    cudaFuncSetAttribute((const void*)batch_sigma_dyson_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)f2);
+    BCOPY(b->d_plane_start, ps.data(), sizeof(long) * (npts + 1), "plane table");
+    BCOPY(b->d_box_start, bs.data(), sizeof(long) * (npts + 1), "box table");
+    BTRY(cudaFuncSetAttribute((const void*)batch_bubble_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)f1),
+         "bubble smem attribute");
+    BTRY(cudaFuncSetAttribute((const void*)batch_sigma_prod_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)f1),
+         "product smem attribute");
+    BTRY(cudaFuncSetAttribute((const void*)batch_sigma_dyson_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)f2),
+         "Dyson smem attribute");
 
     // ladder groups: FP64 (all non-mixed points) + one per mixed padded order
     std::vector<int> idx(npts);
@@ -944,8 +954,8 @@ df_status df_batch_init(df_batch** out, int npts, const df_point* pts, int preci
       g.total = st_[g.nseg];
       BALLOC(g.d_start, sizeof(long) * (g.nseg + 1), "ladder table");
       BALLOC(g.d_order, sizeof(int) * g.nseg, "ladder order");
-      cudaMemcpy(g.d_start, st_.data(), sizeof(long) * (g.nseg + 1), cudaMemcpyHostToDevice);
-      cudaMemcpy(g.d_order, g.order.data(), sizeof(int) * g.nseg, cudaMemcpyHostToDevice);
+      BCOPY(g.d_start, st_.data(), sizeof(long) * (g.nseg + 1), "ladder table");
+      BCOPY(g.d_order, g.order.data(), sizeof(int) * g.nseg, "ladder order");
     }
     BALLOC(b->d_counters, sizeof(unsigned long long) * std::max<size_t>(1, b->groups.size()), "counters");
     // global LU scratch for FP64 ladders of order > kLuSmemOrder
@@ -981,6 +991,8 @@ df_status df_batch_init(df_batch** out, int npts, const df_point* pts, int preci
       if (e != cudaSuccess) { st = bfail(b, DF_ERR_CUDA, "hand-back kernel", e); goto bad; }
     }
   }
+#undef BCOPY
+#undef BTRY
 #undef BALLOC
   if ((st = configure_groups(b)) != DF_OK) goto bad;
   if ((st = build_graph(b)) != DF_OK) goto bad;
