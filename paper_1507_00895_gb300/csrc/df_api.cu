@@ -435,8 +435,8 @@ df_status df_init(df_ctx** out, const df_lattice* lat, double beta, double mu, d
     ALLOC(c->lam_ok_w, (size_t)2 * dm.nb * nw);
     ALLOC(c->sym_chk, 2);
     cudaError_t ea;
-    if ((ea = cudaMemcpy(c->qmap, qmap.data(), sizeof(int) * dm.N, cudaMemcpyHostToDevice)) != cudaSuccess ||
-        (ea = cudaMemcpy(c->qrep, qrep.data(), sizeof(int) * nw, cudaMemcpyHostToDevice)) != cudaSuccess ||
+    if ((ea = cudaMemcpyAsync(c->qmap, qmap.data(), sizeof(int) * dm.N, cudaMemcpyHostToDevice, c->stream)) != cudaSuccess ||
+        (ea = cudaMemcpyAsync(c->qrep, qrep.data(), sizeof(int) * nw, cudaMemcpyHostToDevice, c->stream)) != cudaSuccess ||
         (ea = cudaMemsetAsync(c->chi_w, 0, sizeof(double2) * dm.nb * dm.n_w * nw, c->stream)) != cudaSuccess ||
         (ea = cudaMemsetAsync(c->kc_w, 0, sizeof(double2) * 2 * dm.nb * dm.n_w * nw, c->stream)) != cudaSuccess ||
         (ea = cudaMemsetAsync(c->lam_w, 0, sizeof(double2) * 2 * dm.nb * nw, c->stream)) != cudaSuccess ||

@@ -622,14 +622,16 @@ df_status df_mlp_create(df_mlp** out, int n_in, int width, int n_out, int max_ba
       (e = cudaMalloc(&m->m1, sizeof(float) * o)) != cudaSuccess ||
       (e = cudaMalloc(&m->m2, sizeof(float) * o)) != cudaSuccess ||
       (e = cudaMalloc(&m->d_timeout, sizeof(int))) != cudaSuccess ||
-      (e = cudaMemset(m->d_timeout, 0, sizeof(int))) != cudaSuccess) {
+      (e = cudaMemsetAsync(m->d_timeout, 0, sizeof(int), m->stream)) != cudaSuccess) {
     st = mfail(m, DF_ERR_OOM, "cudaMalloc", e);
   }
   const long pb = pad128(max_batch);
   m->loss_blocks = pb / 128 * ((n_out + 63) / 64);
-  auto zalloc = [&](void** p, size_t bytes) {    // the atoms' padding stays zero
+  // the atoms' padding stays zero; every fill and copy on the network's stream, whose kernels nothing else
+  // orders after the legacy stream's work
+  auto zalloc = [&](void** p, size_t bytes) {
     if (st != DF_OK) return;
-    if ((e = cudaMalloc(p, bytes)) != cudaSuccess || (e = cudaMemset(*p, 0, bytes)) != cudaSuccess)
+    if ((e = cudaMalloc(p, bytes)) != cudaSuccess || (e = cudaMemsetAsync(*p, 0, bytes, m->stream)) != cudaSuccess)
       st = mfail(m, DF_ERR_OOM, "cudaMalloc activations", e);
   };
   for (int l = 0; l < 4; ++l) {
@@ -643,10 +645,11 @@ df_status df_mlp_create(df_mlp** out, int n_in, int width, int n_out, int max_ba
   }
   zalloc((void**)&m->part_loss, sizeof(float) * m->loss_blocks);
   if (st == DF_OK &&
-      ((e = cudaMemcpy(m->params, h.data(), sizeof(float) * o, cudaMemcpyHostToDevice)) != cudaSuccess ||
-       (e = cudaMemset(m->m1, 0, sizeof(float) * o)) != cudaSuccess ||
-       (e = cudaMemset(m->m2, 0, sizeof(float) * o)) != cudaSuccess ||
-       (e = cudaMemset(m->grads, 0, sizeof(float) * o)) != cudaSuccess))
+      ((e = cudaMemcpyAsync(m->params, h.data(), sizeof(float) * o, cudaMemcpyHostToDevice, m->stream)) != cudaSuccess ||
+       (e = cudaMemsetAsync(m->m1, 0, sizeof(float) * o, m->stream)) != cudaSuccess ||
+       (e = cudaMemsetAsync(m->m2, 0, sizeof(float) * o, m->stream)) != cudaSuccess ||
+       (e = cudaMemsetAsync(m->grads, 0, sizeof(float) * o, m->stream)) != cudaSuccess ||
+       (e = cudaStreamSynchronize(m->stream)) != cudaSuccess))
     st = mfail(m, DF_ERR_CUDA, "initialise parameters", e);
   if (st != DF_OK) {
     fprintf(stderr, "libdf: df_mlp_create: %s\n", m->err.c_str());

@@ -16,3 +16,10 @@ def legacy_stream_calls(name):
 
 def test_batch_tables_go_up_on_the_batch_stream():
     assert legacy_stream_calls("df_batch.cu") == []
+
+
+def test_network_and_handle_set_up_on_their_own_streams():
+    assert legacy_stream_calls("df_mlp.cu") == []
+    # (df_selftest_wait launches on the legacy stream itself)
+    calls = [c for c in legacy_stream_calls("df_api.cu") if not re.match(r"cudaMem(set|cpy)\((d, 0|&h, d),", c)]
+    assert calls == []
