@@ -169,7 +169,7 @@ __device__ __forceinline__ void bse_f64_system(const Dims& dm, int c, int a, int
   bool series = false;
   if (radius_K > 0) {
     const double2 l = lam[((size_t)c * nb + a) * N + q];
-    series = (l.x * l.x + l.y * l.y >= 1.0);
+    series = !(l.x * l.x + l.y * l.y < 1.0);            // as the kernel's own flag: not finite counts as outside
   }
   if (series) {
     for (int i = tid; i < n; i += blockDim.x) xs[i] = chi[((size_t)a * n + i) * N + q];

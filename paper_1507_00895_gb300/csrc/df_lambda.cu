@@ -26,10 +26,19 @@
 // from the growth two steps earlier, so |v| stays near 1 without waiting for
 // this step's norm.
 //
+// Range: chi~ of a system is scaled by the power of two that brings max|gamma|
+// max|chi~| to [1/4, 1) (exact; lambda is scaled back in FP64), so that the first two steps, which
+// have no growth to go by, and the squared norms stay within FP32 whatever lambda's size.
+// A growth that changes by many orders of magnitude within two steps (a start vector
+// that A nearly annihilates) can still carry |v| out of [2^-40, 2^40]: the
+// bookkeeping warp sees it, and the block runs the phase again in `exact` mode, which
+// waits for each step's own norm (two more barriers a step).  The polish starts from a settled vector,
+// with the growth of its last step.  Costs 0.2-1.2 us a launch (128 systems of order 16: 38.0 -> 39.2 us).
+//
 // Bound by the steps' latency (64 + 24 dependent products) with few systems,
 // by FP32 issue with many.  Q = 4 systems share each register of gamma; with
 // fewer blocks than SMs Q = 2 spreads them (see launch_lambda).
-#include "df_internal.cuh"
+#include "df_mixed_dev.cuh"
 
 namespace df {
 
@@ -81,17 +90,22 @@ __device__ __forceinline__ void eig_fold(float2 (&y)[Q], int jb, float2 (&out)[Q
   }
 }
 
-// S of step j + 2 from |v_j|^2 = vv, |y_j|^2 = yy, S_j and S_{j+1}: with the growth
-// g^2 = yy / vv kept, |v_{j+2}|^2 = yy S_j^2 S_{j+1}^2 g^2, and S^2 = 1 / (g^2 |v_{j+2}|^2) rounded
-// to a power of four brings |v_{j+3}| into [1/2, 2] (within 2^+-40; 1 for a zero or non-finite norm)
-__device__ __forceinline__ float eig_scale(float yy, float vv, float sj, float sj1) {
-  const float g2 = vv > 0.f ? __fdividef(yy, vv) : 0.f;
-  const float a = g2 * (sj * sj1), w = (yy * a) * a;          // g^2 |v_{j+2}|^2
+// the power of two next to 1 / sqrt(w), within 2^+-40 (1 for a zero or non-finite w)
+__device__ __forceinline__ float eig_pow2(float w) {
   if (!(w > 0.f) || !(w < 3e38f)) return 1.f;
   int e = (int)((__float_as_uint(w) >> 23) & 0xFFu) - 127;
   e = e < -80 ? -80 : (e > 80 ? 80 : e);
   return __int_as_float((127 - (e >> 1)) << 23);
 }
+// S of step j + 2 from |y_j|^2 = yy, S_j and S_{j+1}: with the growth
+// g^2 = |y_j|^2 / |v_j|^2 kept, |v_{j+2}|^2 = yy S_j^2 S_{j+1}^2 g^2, and S^2 = 1 / (g^2 |v_{j+2}|^2) rounded
+// to a power of four brings |v_{j+3}| into [1/2, 2]
+__device__ __forceinline__ float eig_scale(float yy, float g2, float sj, float sj1) {
+  const float a = g2 * (sj * sj1);
+  return eig_pow2((yy * a) * a);                               // g^2 |v_{j+2}|^2
+}
+// the squared norms the steps can work with: 2^-80 .. 2^80
+constexpr float kEigMin = 8.3e-25f, kEigMax = 1.2e24f;
 
 template <int CPL, int Q>
 __global__ void __launch_bounds__(EigShape<CPL, Q>::T + 32, CPL <= 8 ? 3 : (CPL <= 16 ? 2 : 1))
@@ -108,7 +122,7 @@ lambda_kernel(Dims dm, int ch0, int a0, int na, double tol, const double2* __res
   __shared__ float part[2][NW][Q][8];                // per warp: FP32 phase: v^H y, |y|^2, vprev^H y; polish: pairs of
                                                      // v^H y (re, im), |y|^2, |v|^2
   __shared__ float scal[2][Q];                       // S of a step
-  __shared__ int stop_s[2], conv_s[Q];
+  __shared__ int stop_s[2], conv_s[Q], lost_s;
   const int n = dm.n_w, N = dm.N, nb = dm.nb;
   const int qtiles = (N + Q - 1) / Q;
   const int tile = blockIdx.x % qtiles;
@@ -140,20 +154,56 @@ lambda_kernel(Dims dm, int ch0, int a0, int na, double tol, const double2* __res
       const double2 x = (i < n && t0 + k < nq) ? chi[((size_t)a * n + i) * N + q0 + t0 + k] : mk(0.0, 0.0);
       xh[k] = make_float2((float)x.x, (float)x.y);
       xl[k] = make_float2((float)(x.x - (double)xh[k].x), (float)(x.y - (double)xh[k].y));
-      v[k] = make_float2(i < n ? rsqrtf((float)n) : 0.f, 0.f);
-      vp[k] = make_float2(0.f, 0.f);
     }
-  } else if (lane < Q) {
-    scal[0][lane] = scal[1][lane] = 1.f;
-    if (lane < 2) stop_s[lane] = 0;
+    // the largest |gamma| of the warp's rows, the largest |chi~| of its systems' entries
+    unsigned gm = 0u;
+#pragma unroll
+    for (int k = 0; k < CPL; ++k) gm = max(gm, __float_as_uint(fmaxf(fabsf(gh[k].x), fabsf(gh[k].y))));
+    gm = __reduce_max_sync(0xffffffffu, gm);
+    if (lane == 0) part[0][warp][0][7] = __uint_as_float(gm);
+#pragma unroll
+    for (int k = 0; k < QL; ++k) {
+      float m = fmaxf(fabsf(xh[k].x), fabsf(xh[k].y));
+#pragma unroll
+      for (int o = 4; o < 32; o <<= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+      if (lane < 4 && owner) part[0][warp][t0 + k][6] = m;
+    }
+  }
+  __syncthreads();
+  // chi~ of system t by 2^-e: lambda of the scaled problem is 2^-e lambda (e of an infinite or NaN
+  // product: 0); false for A = 0
+  auto range_exp = [&](int t, int& e) {
+    float g = 0.f, x = 0.f;
+#pragma unroll
+    for (int w = 0; w < NW; ++w) {
+      g = fmaxf(g, part[0][w][0][7]);
+      x = fmaxf(x, part[0][w][t][6]);
+    }
+    e = g < INFINITY && x < INFINITY ? exp_bound_f32(g) + exp_bound_f32(x) : 0;
+    return g > 0.f && x > 0.f;
+  };
+  int lexp = 0;                                      // e of the bookkeeping lane's system
+  bool alive = false;
+  if (book) {
+    if (lane < nq && !(alive = range_exp(lane, lexp))) lexp = 0;
+  } else {
+#pragma unroll
+    for (int k = 0; k < QL; ++k) {
+      int e;
+      if (!range_exp(t0 + k, e)) e = 0;
+      const float s1 = pow2f(-(e >> 1)), s2 = pow2f((e >> 1) - e);   // (2^-e itself may leave FP32's range)
+      xh[k] = cscale(cscale(xh[k], s1), s2);
+      xl[k] = cscale(cscale(xl[k], s1), s2);
+    }
   }
 
   // ---- FP32 phase ----
   // bookkeeping state of system `lane` (step j's data is handled during step j + 1): the iterate's
   // norm, S of the next step, the last quotient.  Kept short: it is on the steps' critical path
-  float vv = 1.f, s1 = 1.f;
+  // (se: the last step's S in exact mode, g2: its squared growth, wmin, wmax: the squared norms met)
+  float vv = 1.f, s1 = 1.f, se = 1.f, g2 = 0.f, wmin = 1.f, wmax = 1.f;
   float2 l32 = make_float2(0.f, 0.f);
-  bool done = lane >= nq, pconv = false;
+  bool done = false, pconv = false, exact = false;
   float2 pr1 = l32, pr2 = l32;
   auto book32 = [&](int j) {                         // step j of the FP32 phase
     if (lane < Q) {
@@ -162,12 +212,15 @@ lambda_kernel(Dims dm, int ch0, int a0, int na, double tol, const double2* __res
       for (int w = 0; w < NW; ++w)
 #pragma unroll
         for (int m = 0; m < 5; ++m) r[m] += part[j & 1][w][lane][m];
-      const float yy = r[2], sj = j < 2 ? 1.f : s1;  // S used to form the iterate after step j
+      const float yy = r[2], sj = exact ? se : j < 2 ? 1.f : s1;   // S used to form the iterate after step j
       const float2 ln = cscale(make_float2(r[0], r[1]), vv > 0.f ? __fdividef(1.f, vv) : 0.f), d = ln - l32;
       if (cabs2(d) <= 4e-12f * cabs2(ln)) done = true;
       l32 = ln;
+      g2 = vv > 0.f ? __fdividef(yy, vv) : 0.f;
+      wmin = fminf(wmin, fminf(yy, vv));
+      wmax = fmaxf(wmax, fmaxf(yy, vv));
       const float sj1 = j < 1 ? 1.f : scal[(j + 1) & 1][lane];   // S of step j + 1 (published one step ago)
-      scal[j & 1][lane] = eig_scale(yy, vv, sj, sj1);            // S of step j + 2
+      scal[j & 1][lane] = eig_scale(yy, g2, sj, sj1);            // S of step j + 2
       float* h = hist + ((size_t)j * Q + lane) * 8;              // for the pair's fit
       h[0] = r[0];
       h[1] = r[1];
@@ -180,6 +233,15 @@ lambda_kernel(Dims dm, int ch0, int a0, int na, double tol, const double2* __res
     }
     const int all = __all_sync(0xffffffffu, done || lane >= Q);
     if (lane == 0) stop_s[j & 1] = all;
+  };
+  auto scale_now = [&](int j) {                      // exact mode: S of step j from its own norm
+    if (lane < Q) {
+      float yy = 0.f;
+#pragma unroll
+      for (int w = 0; w < NW; ++w) yy += part[j & 1][w][lane][2];
+      se = eig_pow2(yy);
+      scal[j & 1][lane] = se;
+    }
   };
   // The dominant pair from span{v_prev, v} of step j > 0: A v_prev = v / S_{j-1}, fit A v ~ al v +
   // be v_prev (least squares), l^2 - al l - be / S_{j-1} = 0.  For a pair the two iterates'
@@ -204,55 +266,88 @@ lambda_kernel(Dims dm, int ch0, int a0, int na, double tol, const double2* __res
     l2 = cscale(al - sq, 0.5f);
     return true;
   };
-  int it = 0;
-  for (;; ++it) {
-    if (owner) {
-      float2* u = uh + (it & 1) * 4 * US + uo;
+  int it;
+  for (;;) {
+    if (!book) {
 #pragma unroll
-      for (int k = 0; k < QL; ++k) u[k] = cmul(xh[k], v[k]);
+      for (int k = 0; k < QL; ++k) {
+        v[k] = make_float2(i < n ? rsqrtf((float)n) : 0.f, 0.f);
+        vp[k] = make_float2(0.f, 0.f);
+      }
+    } else if (lane < Q) {
+      scal[0][lane] = scal[1][lane] = 1.f;
+      if (lane < 2) stop_s[lane] = 0;
+      vv = s1 = 1.f;
+      l32 = make_float2(0.f, 0.f);
+      done = lane >= nq;
+    }
+    __syncthreads();                                 // (part's maxima are read)
+    for (it = 0;; ++it) {
+      if (owner) {
+        float2* u = uh + (it & 1) * 4 * US + uo;
+#pragma unroll
+        for (int k = 0; k < QL; ++k) u[k] = cmul(xh[k], v[k]);
+      }
+      __syncthreads();
+      // the flag of step it - 2 (written during step it - 1); the pair is for systems that never settle
+      if (it == kEigIter32 || (it >= 2 && stop_s[it & 1])) break;
+      float2 yo[QL];
+      if (book) {
+        if (it > 0) book32(it - 1);
+      } else {
+        float2 y[Q];
+#pragma unroll
+        for (int t = 0; t < Q; ++t) y[t] = make_float2(0.f, 0.f);
+        const float4* ub = reinterpret_cast<const float4*>(uh + (it & 1) * 4 * US + jb * US);
+#pragma unroll
+        for (int k = 0; k < CPL; ++k)
+#pragma unroll
+          for (int tp = 0; tp < Q / 2; ++tp) {
+            const float4 w = ub[k * (Q / 2) + tp];
+            y[2 * tp] = cfma(gh[k], make_float2(w.x, w.y), y[2 * tp]);
+            y[2 * tp + 1] = cfma(gh[k], make_float2(w.z, w.w), y[2 * tp + 1]);
+          }
+        eig_fold<Q, QL>(y, jb, yo);
+#pragma unroll
+        for (int k = 0; k < QL; ++k) {
+          const float2 rq = cmul(cconj(v[k]), yo[k]), g = cmul(cconj(vp[k]), yo[k]);
+          float p[5] = {rq.x, rq.y, cabs2(yo[k]), g.x, g.y};
+#pragma unroll
+          for (int m = 0; m < 5; ++m)
+#pragma unroll
+            for (int o = 4; o < 32; o <<= 1) p[m] += __shfl_xor_sync(0xffffffffu, p[m], o);
+          if (lane < 4 && owner) {
+#pragma unroll
+            for (int m = 0; m < 5; ++m) part[it & 1][warp][t0 + k][m] = p[m];
+          }
+        }
+      }
+      if (exact) {
+        __syncthreads();
+        if (book) scale_now(it);
+        __syncthreads();
+      }
+      if (!book) {
+#pragma unroll
+        for (int k = 0; k < QL; ++k) {
+          const float s = scal[it & 1][t0 + k];
+          vp[k] = v[k];
+          v[k] = cscale(yo[k], s);
+        }
+      }
+    }
+    __syncthreads();                                 // every thread has read the flag
+    // the last step's data (part of step it - 1 was complete at the barrier before)
+    if (book) {
+      book32(it - 1);
+      const int again = !exact && __any_sync(0xffffffffu, alive && !(wmin > kEigMin && wmax < kEigMax));
+      if (lane == 0) lost_s = again;
     }
     __syncthreads();
-    // the flag of step it - 2 (written during step it - 1); the pair is for systems that never settle
-    if (it == kEigIter32 || (it >= 2 && stop_s[it & 1])) break;
-    if (book) {
-      if (it > 0) book32(it - 1);
-      continue;
-    }
-    float2 y[Q];
-#pragma unroll
-    for (int t = 0; t < Q; ++t) y[t] = make_float2(0.f, 0.f);
-    const float4* ub = reinterpret_cast<const float4*>(uh + (it & 1) * 4 * US + jb * US);
-#pragma unroll
-    for (int k = 0; k < CPL; ++k)
-#pragma unroll
-      for (int tp = 0; tp < Q / 2; ++tp) {
-        const float4 w = ub[k * (Q / 2) + tp];
-        y[2 * tp] = cfma(gh[k], make_float2(w.x, w.y), y[2 * tp]);
-        y[2 * tp + 1] = cfma(gh[k], make_float2(w.z, w.w), y[2 * tp + 1]);
-      }
-    float2 yo[QL];
-    eig_fold<Q, QL>(y, jb, yo);
-#pragma unroll
-    for (int k = 0; k < QL; ++k) {
-      const float2 rq = cmul(cconj(v[k]), yo[k]), g = cmul(cconj(vp[k]), yo[k]);
-      float p[5] = {rq.x, rq.y, cabs2(yo[k]), g.x, g.y};
-#pragma unroll
-      for (int m = 0; m < 5; ++m)
-#pragma unroll
-        for (int o = 4; o < 32; o <<= 1) p[m] += __shfl_xor_sync(0xffffffffu, p[m], o);
-      if (lane < 4 && owner) {
-#pragma unroll
-        for (int m = 0; m < 5; ++m) part[it & 1][warp][t0 + k][m] = p[m];
-      }
-      const float s = it < 2 ? 1.f : scal[it & 1][t0 + k];
-      vp[k] = v[k];
-      v[k] = cscale(yo[k], s);
-    }
+    if (!lost_s) break;
+    exact = true;
   }
-  __syncthreads();                                   // every thread has read the flag
-  // the last step's data (part of step it - 1 was complete at the barrier before)
   if (book) {
-    book32(it - 1);
     // systems that never settled: the last two fits that count, settled when both
     // roots agree within 1e-4 (their order may swap)
     if (lane < Q && !done) {
@@ -270,7 +365,10 @@ lambda_kernel(Dims dm, int ch0, int a0, int na, double tol, const double2* __res
     }
     if (lane < Q) conv_s[lane] = lane < nq && done;
     if (lane < 2) stop_s[lane] = 0;
-    if (lane < Q) scal[0][lane] = scal[1][lane] = 1.f;
+    if (lane < Q) {                                  // the polish goes on at the last step's growth
+      scal[0][lane] = eig_pow2(g2 * vv);
+      scal[1][lane] = eig_pow2(g2);
+    }
   }
   __syncthreads();
   int any = 0;
@@ -281,7 +379,7 @@ lambda_kernel(Dims dm, int ch0, int a0, int na, double tol, const double2* __res
   const bool conv = book && lane < Q && conv_s[lane];
   double2 lo = mk(0.0, 0.0);
   bool dn = !conv;
-  s1 = 1.f;
+  const float sp0 = eig_pow2(g2 * vv), sp1 = eig_pow2(g2);
   auto book64 = [&](int j) {                         // step j of the polish
     if (lane < Q) {
       double r[4];
@@ -301,8 +399,9 @@ lambda_kernel(Dims dm, int ch0, int a0, int na, double tol, const double2* __res
         if (j > 0 && cabs2(d) <= tol * tol * cabs2(ln)) dn = true;
         lo = ln;
       }
-      const float sj = j < 2 ? 1.f : s1, sj1 = j < 1 ? 1.f : scal[(j + 1) & 1][lane];
-      scal[j & 1][lane] = eig_scale((float)r[2], (float)r[3], sj, sj1);
+      const float sj = j == 0 ? sp0 : j == 1 ? sp1 : s1, sj1 = j < 1 ? sp1 : scal[(j + 1) & 1][lane];
+      const float y2 = (float)r[2], v2 = (float)r[3];
+      scal[j & 1][lane] = eig_scale(y2, v2 > 0.f ? __fdividef(y2, v2) : 0.f, sj, sj1);
       s1 = sj1;
     }
     const int all = __all_sync(0xffffffffu, dn || lane >= Q);
@@ -392,7 +491,7 @@ lambda_kernel(Dims dm, int ch0, int a0, int na, double tol, const double2* __res
 #pragma unroll
           for (int m = 0; m < 8; ++m) part[ip & 1][warp][t0 + k][m] = p[m];
         }
-        const float s = ip < 2 ? 1.f : scal[ip & 1][t0 + k];
+        const float s = scal[ip & 1][t0 + k];
         // renormalise the pair, scale by the power of two (exact)
         const float hx = ys[k].x + yl[k].x, hy = ys[k].y + yl[k].y;
         vl[k] = make_float2((yl[k].x - (hx - ys[k].x)) * s, (yl[k].y - (hy - ys[k].y)) * s);
@@ -414,9 +513,10 @@ lambda_kernel(Dims dm, int ch0, int a0, int na, double tol, const double2* __res
       l = mk((double)lp.x, (double)lp.y);
       okv = 2;
     }
+    l = mk(scalbn(l.x, lexp), scalbn(l.y, lexp));
     lam[o] = l;
     ok[o] = okv;
-    if (cabs2(l) >= 1.0) atomicOr(flags, kFlagRadius);
+    if (!(cabs2(l) < 1.0)) atomicOr(flags, kFlagRadius);   // (a value that is not finite counts as outside)
   }
 }
 
