@@ -36,6 +36,13 @@ struct MixedCheck {
   int base;       // added to the system index in the list (the batch: point << 24)
 };
 
+// An exactly zero pivot of the FP32 inversion: such a ladder is not finite for the error control.  It may
+// still be regular in FP64 (condition number above 2^24), so where it is handed back the FP64 LU
+// decides; without a list it is reported.
+__device__ __forceinline__ void zero_pivot(const MixedCheck& mc, int* flags) {
+  if (!mc.redo) atomicOr(flags, kFlagSingular);
+}
+
 __device__ __forceinline__ void mixed_check_ladder(const MixedCheck& mc, float emax, float gmax, bool finite,
                                                    long sys, int* flags) {
   float rho2;

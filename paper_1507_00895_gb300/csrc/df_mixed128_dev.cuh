@@ -243,7 +243,8 @@ __device__ __forceinline__ bool m128_system(const Dims& dm, int c, int a, int q,
         float2 pv[kPanel];
 #pragma unroll
         for (int c2 = 0; c2 < kPanel; ++c2) pv[c2] = part ? swap[((part - 1) * kPanel + c2) * 32 + lane] : A[0][c2];
-        gj_panel_team<4>(pv, r, part, lane, kPanel * kp, wbuf + kp * kPanel * 128, cand, ckey, piv_s, rowstep, flags, 2);
+        gj_panel_team<4>(pv, r, part, lane, kPanel * kp, wbuf + kp * kPanel * 128, cand, ckey, piv_s, rowstep, mc, flags,
+                         badw, 2);
         if (part) {
 #pragma unroll
           for (int c2 = 0; c2 < kPanel; ++c2) swap[((part - 1) * kPanel + c2) * 32 + lane] = pv[c2];

@@ -270,10 +270,11 @@ __device__ __forceinline__ void m32_system(const Dims& dm, int c, int a, int q, 
       }
     }
   }
-  if ((kmin & ~0x1Fu) == 0u && lane == 0) atomicOr(flags, kFlagSingular);   // an exactly zero pivot
+  const bool zero = (kmin & ~0x1Fu) == 0u;                // an exactly zero FP32 pivot
+  if (zero && lane == 0) zero_pivot(mc, flags);
   // ---- S to shared memory in logical order: row `step`, column piv[c]; padding zero ----
   __syncwarp();
-  bool bad = false;
+  bool bad = zero;
   {
     int pc[CP];                                           // register r holds column lcol + 4 ((r + n / 4) mod CP)
     bool cz[CP];

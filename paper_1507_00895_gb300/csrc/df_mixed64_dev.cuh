@@ -194,8 +194,8 @@ __device__ __forceinline__ float rcp_approx(float x) {
 // pivot rows goes to wk [step][row].
 template <int WARPS>
 __device__ __forceinline__ void gj_panel_team(float2 (&pv)[kPanel], int r, int half, int lane, int k0, float2* wk,
-                                              float4* cand, unsigned* ckey, int* piv_s, int* rowstep, int* flags,
-                                              int bar) {
+                                              float4* cand, unsigned* ckey, int* piv_s, int* rowstep,
+                                              const MixedCheck& mc, int* flags, int* badw, int bar) {
   constexpr int kRows = 32 * WARPS;
   const bool taken = rowstep[r] >= 0;
   unsigned km = taken ? 0u : ~0x7Fu, kr = taken ? 0u : (unsigned)(127 - r);   // 0 once the row is a pivot
@@ -260,7 +260,10 @@ __device__ __forceinline__ void gj_panel_team(float2 (&pv)[kPanel], int r, int h
     rowstep[r] = k0 + step;
     piv_s[k0 + step] = r;
   }
-  if ((kmin & ~0x7Fu) == 0u && lane == 0) atomicOr(flags, kFlagSingular);   // an exactly zero pivot
+  if ((kmin & ~0x7Fu) == 0u && lane == 0) {                 // an exactly zero FP32 pivot
+    *badw = 1;
+    zero_pivot(mc, flags);
+  }
 }
 
 struct M64Group {
@@ -345,7 +348,8 @@ __device__ __forceinline__ void m64_system(const Dims& dm, int c, int a, int q, 
         float2 pv[kPanel];
 #pragma unroll
         for (int c = 0; c < kPanel; ++c) pv[c] = half ? swap[c * 32 + lane] : A[0][c];
-        gj_panel_team<2>(pv, r, half, lane, kPanel * kp, wbuf + kp * 512, cand, ckey, piv_s, rowstep, flags, 3 + gr.g);
+        gj_panel_team<2>(pv, r, half, lane, kPanel * kp, wbuf + kp * 512, cand, ckey, piv_s, rowstep, mc, flags, badw,
+                         3 + gr.g);
         if (half == 1) {
 #pragma unroll
           for (int c = 0; c < kPanel; ++c) swap[c * 32 + lane] = pv[c];

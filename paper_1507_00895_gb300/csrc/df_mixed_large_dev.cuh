@@ -64,7 +64,7 @@ __device__ __forceinline__ void x2_acc(float2& S, float2& L, float2 A, float2 nA
 
 // ghi, glo: gamma's (hi, lo) FP32 words [2][nb][n][n]; gth, gtl: gamma^T's;
 // gg: gamma o gamma^T (FP64); chi: chi~ [nb][n][N]; kc: the Eq. sd bracket
-// [2][nb][n][N]; flags bit 0: a zero FP32 pivot.
+// [2][nb][n][N]; a zero FP32 pivot: zero_pivot.
 __device__ __forceinline__ void gj_ir_system(const Dims& dm, int c, int a, int q, const float2* __restrict__ ghi,
                                              const float2* __restrict__ glo, const float2* __restrict__ gth,
                                              const float2* __restrict__ gtl, const double2* __restrict__ gg,
@@ -138,7 +138,10 @@ __device__ __forceinline__ void gj_ir_system(const Dims& dm, int c, int a, int q
     const bool zero = (pv.x == 0.f && pv.y == 0.f);
     const float2 inv = zero ? make_float2(0.f, 0.f) : gj_cinv(pv);
     if (tid == 0) {
-      if (zero) atomicOr(flags, kFlagSingular);
+      if (zero) {
+        sh.bad = 1;
+        zero_pivot(mc, flags);
+      }
       if (p != k) { const int t = sh.perm[k]; sh.perm[k] = sh.perm[p]; sh.perm[p] = t; }
     }
     // rows k and p exchanged, row k scaled by 1/pivot (its column-k entry

@@ -347,3 +347,40 @@ def test_single_hand_back_is_split(df, n_w):
         b64.iterate(1)
         b.iterate(1)
         assert nrel(b.get_sigma(0), b64.get_sigma(0)) < TOL_SIGMA
+
+
+def rounds_to_singular(n, m_max=0):
+    """Ladders that are exactly singular once D is rounded to FP32 and regular in FP64: g = Delta = 1,
+    t = 0, N_k = 2, beta = 4 give chi~ = -1/16 exactly, and D = 1 + gamma / 16 is the identity but for
+    [[2, 1], [2, 1 + 2^-30]] in its first and last rows and columns; every step of its LU is exact."""
+    gam = np.zeros((1, n, n), complex)
+    gam[0, 0, 0], gam[0, 0, n - 1], gam[0, n - 1, 0], gam[0, n - 1, n - 1] = 16.0, 16.0, 32.0, 16.0 * 2.0 ** -30
+    g = np.ones(n, complex)
+    return I.Workload("singular32", 1, 2, 0.0, 0.0, 1.0, 4.0, 0.0, n, 0, g, g, gam, np.zeros_like(gam))
+
+
+@pytest.mark.parametrize("n_w,sweep", [(2, 0), (16, 0), (18, 0), (32, 0), (34, 0), (64, 0), (66, 0), (128, 0), (96, 1)])
+def test_zero_fp32_pivot_is_left_to_the_fp64_solve(df, n_w, sweep):
+    w = rounds_to_singular(n_w)
+    with df.DualFermion.from_workload(w, eig_mode=0) as d:
+        assert d.iterate(1)[2] == df.DF_OK
+        ref, kref = d.get_sigma(), d.get_kernel()
+    with df.DualFermion.from_workload(w, precision=df.DF_FP32_IR, eig_mode=0, mixed_sweep=sweep) as d:
+        assert d.iterate(1)[2] == df.DF_OK
+        assert d.ladder_stats()[1] == 4                     # 2 channels x 1 plane x 2 momenta
+        assert nrel(d.get_kernel(), kref) < 1e-12 and nrel(d.get_sigma(), ref) < 1e-12
+    # without the second solve it is reported
+    with df.DualFermion.from_workload(w, precision=df.DF_FP32_IR, eig_mode=0, mixed_sweep=sweep, ladder_fallback=0) as d:
+        with pytest.raises(df.DFError) as e:
+            d.iterate(1)
+        assert e.value.status == df.DF_ERR_SINGULAR
+
+
+def test_zero_fp32_pivot_in_a_batch(df):
+    ws = [rounds_to_singular(n) for n in (2, 18, 34, 66)]
+    with df.DualFermionBatch(ws, precision=df.DF_FP32_IR) as b:
+        b.iterate(1)
+        for i, w in enumerate(ws):
+            with df.DualFermion.from_workload(w, eig_mode=0) as d:
+                d.iterate(1)
+                assert nrel(b.get_sigma(i), d.get_sigma()) < 1e-12, w.n_w
