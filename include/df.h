@@ -431,6 +431,13 @@ df_status df_bse_noalloc(const double* gamma, const double* chi, int n_w, int n_
  * DF_ERR_CUDA. */
 df_status df_selftest_wait(int arrive, int spins);
 
+/* Self-test of the same waits where they are used: one df_bse of the handle (DF_FP32_IR,
+ * 33 <= n_w <= 64; chi~ as df_bubble left it) with every completion wait of the ladder kernel limited to
+ * `spins` polls.  A wait that gives up ends its block's work after a bounded wait for the
+ * products in flight, and the call returns DF_ERR_TIMEOUT (brackets not valid until the
+ * next df_bse); DF_OK when every wait saw its completion.  Synchronous.  Errors: DF_ERR_ARG (other handles, spins < 0). */
+df_status df_selftest_ladder_wait(df_ctx* c, int spins);
+
 /* Measured arithmetic peak of the current device, the denominator of the
  * ladder kernels' roofline fractions (the paper has no counterpart: this is
  * measurement support).  kind 0: FP32 fma.rn.f32, 1: FP32 packed

@@ -537,6 +537,17 @@ df_status df_selftest_wait(int arrive, int spins) {
   return (h & kFlagTcTimeout) ? DF_ERR_TIMEOUT : DF_OK;
 }
 
+df_status df_selftest_ladder_wait(df_ctx* c, int spins) {
+  if (!c || spins < 0 || c->opts.precision != DF_FP32_IR || c->dm.n_w <= 32 || c->dm.n_w > 64) return DF_ERR_ARG;
+  c->wait_spins = (unsigned)spins;
+  const df_status s = df_bse(c, 3);
+  c->wait_spins = kMbarSpin;
+  if (s != DF_OK) return s;
+  int flags = 0;
+  const df_status r = read_scalars(c, nullptr, &flags);
+  return r != DF_OK ? r : flag_error(c, flags & kFlagTcTimeout);
+}
+
 static bool full_range(const df_ctx* c) { return c->dm.a0 == 0 && c->dm.na == c->dm.nb; }
 
 // the end of a pass: the residual and the ladder flags of the pass, if asked for

@@ -329,23 +329,27 @@ batch_bse_mixed64_kernel(const PointDev* __restrict__ pts, const int* __restrict
   extern __shared__ __align__(1024) unsigned char sm64[];
   __shared__ uint64_t mbar_s[2 * kM64Groups];
   __shared__ unsigned tslot_s;
+  __shared__ int fail_s[kM64Groups];
   __shared__ unsigned long long item_s;
   if (smem_u32(sm64) & 1023u) {                  // the swizzled operand tiles need 1024-byte alignment
     if (threadIdx.x == 0) atomicOr(pts[0].flags, kFlagTcLayout);
     return;
   }
   M64Block blk;
-  m64_setup(blk, sm64, mbar_s, &tslot_s);
+  m64_setup(blk, sm64, mbar_s, &tslot_s, fail_s);
   const long total = start[nseg];
   long cur = -1;                       // (point, channel, W) whose gamma digits are in shared memory
-  for (;;) {
+  bool ok = true, go = true;           // of this group (a completion wait gave up), of the block
+  while (go) {
     __syncthreads();
+    go = !m64_failed(blk);
     if (threadIdx.x == 0) item_s = atomicAdd(counter, (unsigned long long)(kBatch64Take * chunk));
     __syncthreads();
+    if (!go) break;
     long s = (long)item_s;
     if (s >= total) break;
     const long last = min(s + (long)(kBatch64Take * chunk), total);
-    while (s < last) {
+    while (s < last && go) {
       const int k = find_segment(start, nseg, s);
       const PointDev& P = pts[order[k]];
       const Dims& dm = P.ldm;
@@ -355,13 +359,16 @@ batch_bse_mixed64_kernel(const PointDev* __restrict__ pts, const int* __restrict
         const int c = (int)(plane / dm.na), a = dm.a0 + (int)(plane % dm.na), key = c * dm.nb + a;
         const long id = (long)k * 256 + key;
         const unsigned char* gd = P.gdig + (size_t)key * kM64DigBytes;
-        if (id != cur) m64_load_digits(blk, gd);
+        if (id != cur) go = m64_load_digits(blk, gd);
         cur = id;
+        if (!go) break;
         const size_t mat = (size_t)key * dm.n_w * dm.n_w;
-        for (long x = s + blk.gr.g; x < end; x += kM64Groups)
-          m64_system(dm, c, a, (int)(x - base), reinterpret_cast<const float4*>(gd + kM64Shared), P.gg_hi + mat,
-                     P.gg_lo + mat, P.lchi, P.lkc, P.flags, blk.gr, smem_u32(sm64), reinterpret_cast<const float*>(sm64 + kM64Gexp),
-                     batch_check(redo, order[k]));
+        for (long x = s + blk.gr.g; x < end && ok; x += kM64Groups) {
+          ok = m64_system(dm, c, a, (int)(x - base), reinterpret_cast<const float4*>(gd + kM64Shared), P.gg_hi + mat,
+                          P.gg_lo + mat, P.lchi, P.lkc, P.flags, blk.gr, smem_u32(sm64),
+                          reinterpret_cast<const float*>(sm64 + kM64Gexp), batch_check(redo, order[k]));
+          if (!ok && threadIdx.x % kM64Group == 0) atomicOr(P.flags, kFlagTcTimeout);
+        }
       }
       s = end;
     }

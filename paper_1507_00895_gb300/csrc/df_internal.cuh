@@ -20,6 +20,8 @@ constexpr int kFlagTcTimeout = 4;   // a bounded tensor-core completion wait gav
 constexpr int kFlagTcLayout = 8;    // tensor-core operands not 1024-byte aligned (no MMA issued)
 constexpr int kFlagRefine = 16;     // a mixed-precision ladder missed its error bound and was not re-solved
 
+constexpr unsigned kMbarSpin = 1u << 22;   // polls of a bounded wait on a shared-memory barrier before it gives up
+
 // Per-ladder error control of the mixed-precision ladder solves.  After the
 // one correction E of X0 ~ D^-1 gamma, rho = max_j |E_jj| / max_j |Gamma_jj|
 // (|re| + |im|) is the relative size of the correction; with a fixed FP32
@@ -289,6 +291,7 @@ struct df_ctx {
                                // df_init: the hand-back list before it is sized for the full grid)
   size_t bse_ws_bytes = 0;
   int bse_grid = 0;
+  unsigned wait_spins = df::kMbarSpin;   // polls of the order 33-64 kernel's completion waits (df_selftest_ladder_wait)
   int iter_done = 0;
   int sigma_valid = 0;         // gk/gr reflect sigma
   double last_resid = -1.0;

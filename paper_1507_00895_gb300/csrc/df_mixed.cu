@@ -67,16 +67,17 @@ bse_mixed32_kernel(Dims dm, int ch0, int nch, const float2* __restrict__ gg_hi, 
 __global__ void __launch_bounds__(kM64Threads, 1)
 bse_mixed64_kernel(Dims dm, int ch0, int nch, const float2* __restrict__ gg_hi, const float2* __restrict__ gg_lo,
                    const double2* __restrict__ chi, double2* __restrict__ kc, const unsigned char* __restrict__ gdig,
-                   int* __restrict__ flags, MixedCheck mc) {
+                   int* __restrict__ flags, MixedCheck mc, unsigned spins) {
   extern __shared__ __align__(1024) unsigned char sm64[];
   __shared__ uint64_t mbar_s[2 * kM64Groups];
   __shared__ unsigned tslot_s;
+  __shared__ int fail_s[kM64Groups];
   if (smem_u32(sm64) & 1023u) {                  // the swizzled operand tiles need 1024-byte alignment
     if (threadIdx.x == 0) atomicOr(flags, kFlagTcLayout);
     return;
   }
   M64Block blk;
-  m64_setup(blk, sm64, mbar_s, &tslot_s);
+  m64_setup(blk, sm64, mbar_s, &tslot_s, fail_s, spins);
   const int N = dm.N, nb = dm.nb, na = dm.na;
   const long systems = (long)nch * na * N;
   const long s1 = systems * (blockIdx.x + 1) / gridDim.x;
@@ -85,11 +86,13 @@ bse_mixed64_kernel(Dims dm, int ch0, int nch, const float2* __restrict__ gg_hi, 
     const long plane = s / N, end = min(s1, (plane + 1) * N);
     const int c = ch0 + (int)(plane / na), a = dm.a0 + (int)(plane % na), key = c * nb + a;
     const unsigned char* gd = gdig + (size_t)key * kM64DigBytes;
-    m64_load_digits(blk, gd);
+    if (!m64_load_digits(blk, gd)) break;
     const size_t mat = (size_t)key * dm.n_w * dm.n_w;
-    for (long x = s + blk.gr.g; x < end; x += kM64Groups)
-      m64_system(dm, c, a, (int)(x - plane * N), reinterpret_cast<const float4*>(gd + kM64Shared), gg_hi + mat,
+    bool ok = true;
+    for (long x = s + blk.gr.g; x < end && ok; x += kM64Groups)
+      ok = m64_system(dm, c, a, (int)(x - plane * N), reinterpret_cast<const float4*>(gd + kM64Shared), gg_hi + mat,
                  gg_lo + mat, chi, kc, flags, blk.gr, smem_u32(sm64), reinterpret_cast<const float*>(sm64 + kM64Gexp), mc);
+    if (!ok && threadIdx.x % kM64Group == 0) atomicOr(flags, kFlagTcTimeout);
     s = end;
   }
   m64_teardown(blk);
@@ -209,7 +212,8 @@ static cudaError_t launch_bse_mixed64(df_ctx* c, int channel_mask, int* flags) {
   const int nch = (channel_mask & 1) + ((channel_mask >> 1) & 1), ch0 = (channel_mask & 1) ? 0 : 1;
   const long pairs = ((long)nch * dm.na * dm.N + kM64Groups - 1) / kM64Groups;
   bse_mixed64_kernel<<<(int)(pairs < sms ? pairs : sms), kM64Threads, kM64Smem, c->stream>>>(
-      dm, ch0, nch, hi + 2 * count, hi + 3 * count, c->chi, c->kc, gdig_ptr(c), flags, mc);
+      dm, ch0, nch, hi + 2 * count, hi + 3 * count, c->chi, c->kc, gdig_ptr(c), flags, mc,
+      c->wait_spins);
   return cudaGetLastError();
 }
 

@@ -272,12 +272,15 @@ struct M64Group {
   uint64_t* mbar;         // completion barrier of its MMAs
   unsigned phase;
   int g;
+  unsigned spins;         // polls of a completion wait
+  volatile int* fail;     // shared, per group: a completion wait gave up
 };
 
 // One ladder by the kM64Group threads of group gr.  gdig: the block's gamma
 // digits in shared memory (their address), gwt the columns' weights 2^(e_j - 8).
-// Writes kc[c][a][:][q].
-__device__ __forceinline__ void m64_system(const Dims& dm, int c, int a, int q, const float4* __restrict__ words,
+// Writes kc[c][a][:][q].  False when a completion wait gave up (the same in the whole group, which then must
+// not start another ladder: its MMAs may still read its operands until the tear-down).
+__device__ __forceinline__ bool m64_system(const Dims& dm, int c, int a, int q, const float4* __restrict__ words,
                                            const float2* __restrict__ GGh, const float2* __restrict__ GGl,
                                            const double2* __restrict__ chi,
                                            double2* __restrict__ kc, int* __restrict__ flags, M64Group& gr,
@@ -512,7 +515,13 @@ __device__ __forceinline__ void m64_system(const Dims& dm, int c, int a, int q, 
       umma_commit(gr.mbar);
     }
     __syncwarp();
-    if (!mbar_wait(gr.mbar, gr.phase) && t == 0) atomicOr(flags, kFlagTcTimeout);
+    // a warp that saw the completion may overwrite the operands (with the exchange): the MMAs are done; one that gave up
+    // leaves them and the accumulators alone, and after the fold's barrier the whole group knows
+    if (!__all_sync(0xffffffffu, mbar_wait(gr.mbar, gr.phase, gr.spins))) {
+      *gr.fail = 1;
+      m64_sync(gr.g);
+      return false;
+    }
     gr.phase ^= 1u;
     tc05_fence_after();
     // fold: warp w reads lane quadrant w % 4 (lanes 0-63: gamma_re column j, 64-127:
@@ -565,6 +574,7 @@ __device__ __forceinline__ void m64_system(const Dims& dm, int c, int a, int q, 
         }
       }
       m64_sync(gr.g);
+      if (*gr.fail) return false;
       if (!zi) {
         float2* Eo = E + h * 16 * kM64ELd + j;
 #pragma unroll
@@ -661,6 +671,7 @@ __device__ __forceinline__ void m64_system(const Dims& dm, int c, int a, int q, 
     fin = __all_sync(0xffffffffu, fin);
     if (lane == 0) mixed_check_ladder(mc, emax, gmax, fin, ((long)c * nb + a) * N + q, flags);
   }
+  return true;
 }
 
 // Block-level state: set up by all threads (warp 0 allocates the tensor memory).
@@ -668,9 +679,17 @@ struct M64Block {
   unsigned char* sm;      // dynamic shared memory, 1024-aligned
   uint64_t* mbar;         // [kM64Groups] the groups' completion barriers, then their tear-down barriers
   unsigned tmem;
+  volatile int* fail;     // [kM64Groups]
   M64Group gr;            // this thread's group
 };
-__device__ __forceinline__ void m64_setup(M64Block& b, unsigned char* sm, uint64_t* mbar, unsigned* tslot) {
+// some group of the block gave up (read by all threads while no ladder runs)
+__device__ __forceinline__ bool m64_failed(const M64Block& b) {
+  int f = 0;
+  for (int i = 0; i < kM64Groups; ++i) f |= b.fail[i];
+  return f != 0;
+}
+__device__ __forceinline__ void m64_setup(M64Block& b, unsigned char* sm, uint64_t* mbar, unsigned* tslot,
+                                          volatile int* fail, unsigned spins = kMbarSpin) {
   if ((threadIdx.x >> 5) == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(tslot)) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -678,6 +697,7 @@ __device__ __forceinline__ void m64_setup(M64Block& b, unsigned char* sm, uint64
   if (threadIdx.x == 0) {
     for (int i = 0; i < 2 * kM64Groups; ++i)
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(mbar + i)) : "memory");
+    for (int i = 0; i < kM64Groups; ++i) fail[i] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   tc05_fence_before();
@@ -687,7 +707,8 @@ __device__ __forceinline__ void m64_setup(M64Block& b, unsigned char* sm, uint64
   b.sm = sm;
   b.mbar = mbar;
   b.tmem = *tslot;
-  b.gr = M64Group{sm + kM64Base + g * kM64GroupBytes, b.tmem + 256u * g, mbar + g, 0u, g};
+  b.fail = fail;
+  b.gr = M64Group{sm + kM64Base + g * kM64GroupBytes, b.tmem + 256u * g, mbar + g, 0u, g, spins, fail + g};
 }
 // each group's issuing thread commits once more, which completes after every
 // MMA it queued (also after a wait that gave up); the wait for it is bounded
@@ -703,14 +724,19 @@ __device__ __forceinline__ void m64_teardown(const M64Block& b) {
   if ((threadIdx.x >> 5) == 0)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(b.tmem) : "memory");
 }
-// gamma's digits of one (channel, W) into shared memory (all threads; no ladder running)
-__device__ __forceinline__ void m64_load_digits(const M64Block& b, const unsigned char* __restrict__ gdig) {
+// gamma's digits of one (channel, W) into shared memory (all threads; no ladder running).  False, the same in
+// the whole block, once a group gave up: its MMAs may still read the old ones.
+__device__ __forceinline__ bool m64_load_digits(const M64Block& b, const unsigned char* __restrict__ gdig) {
   __syncthreads();
-  const uint4* src = reinterpret_cast<const uint4*>(gdig);
-  uint4* dst = reinterpret_cast<uint4*>(b.sm);
-  for (int i = threadIdx.x; i < kM64Shared / 16; i += kM64Threads) dst[i] = __ldg(src + i);
-  fence_async_smem();
+  const bool go = !m64_failed(b);
+  if (go) {
+    const uint4* src = reinterpret_cast<const uint4*>(gdig);
+    uint4* dst = reinterpret_cast<uint4*>(b.sm);
+    for (int i = threadIdx.x; i < kM64Shared / 16; i += kM64Threads) dst[i] = __ldg(src + i);
+    fence_async_smem();
+  }
   __syncthreads();
+  return go;
 }
 
 }  // namespace df

@@ -51,8 +51,6 @@ __device__ __forceinline__ int swz(int row, int k) {
 // 1024 bytes apart, group base 1024-aligned) -- the layout swz() writes.  The
 // FP32 accumulators live in tensor memory (TMEM): row i of D in TMEM lane i,
 // column j in TMEM column (base + j).
-constexpr unsigned kMbarSpin = 1u << 22;   // try_wait rounds before giving up
-
 __device__ __forceinline__ unsigned smem_u32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
 
 // shared-memory matrix descriptor: K-major, 128-byte swizzle, 8-row groups 1024 B apart

@@ -42,7 +42,7 @@ EXPORTS = (
     "df_batch_reset", "df_batch_autotune", "df_batch_last_error", "df_batch_destroy", "df_mlp_create",
     "df_mlp_param_count", "df_mlp_forward", "df_mlp_gradients", "df_mlp_adam_step", "df_mlp_train_step",
     "df_mlp_params", "df_mlp_grads", "df_mlp_last_error", "df_mlp_destroy", "df_warmstart_sigma", "df_last_error",
-    "df_status_string", "df_destroy", "df_selftest_wait", "df_peak_probe", "df_wedge",
+    "df_status_string", "df_destroy", "df_selftest_wait", "df_selftest_ladder_wait", "df_peak_probe", "df_wedge",
 )
 
 
@@ -112,6 +112,7 @@ def load(path: str = LIB_PATH):
         "df_synchronize": [P],
         "df_bse_noalloc": [P, P, C.c_int, C.c_int, C.c_int, P, P],
         "df_selftest_wait": [C.c_int, C.c_int],
+        "df_selftest_ladder_wait": [P, C.c_int],
         "df_peak_probe": [C.c_int, D],
         "df_wedge": [C.c_int, C.c_int, P, P, I],
         "df_batch_init": [C.POINTER(P), C.c_int, C.c_void_p, C.c_int, C.c_double, C.c_double, P],

@@ -50,3 +50,20 @@ def test_device_usable_after_a_timeout(df):
     assert it == 1
     err = np.max(np.abs(sig - ref.sigma)) / np.max(np.abs(ref.sigma))
     assert err < 1e-8, err
+
+
+def test_ladder_kernel_gives_up_and_the_next_pass_is_right(df):
+    # every completion wait of the order 33-64 kernel gives up at once: its blocks stop after the products in
+    # flight, the call reports it, and the handle's next pass agrees with the oracle
+    w = I.workload("square32_tp", nk=4, n_w=64, m_max=1)
+    ref = O.run_workload(w, n_iter=1)
+    lib = df.load()
+    with df.DualFermion.from_workload(w, precision=df.DF_FP32_IR) as d:
+        d.bubble()
+        assert lib.df_selftest_ladder_wait(d.h, 0) == df.DF_ERR_TIMEOUT
+        assert lib.df_selftest_ladder_wait(d.h, -1) == df.DF_ERR_ARG
+        assert lib.df_selftest_ladder_wait(d.h, 1 << 22) == df.DF_OK
+        assert lib.df_selftest_ladder_wait(d.h, 0) == df.DF_ERR_TIMEOUT
+        assert d.iterate(1)[0] == 1
+        sig = d.get_sigma()
+    assert np.max(np.abs(sig - ref.sigma)) < 1e-8 * np.max(np.abs(ref.sigma))
