@@ -14,18 +14,22 @@
 //     orders 33-64), 8 x 8 (4 x 8) entries of it per thread in registers, where it stays:
 //     a solve is one matrix-vector product, not two serial triangular substitutions.
 //   * FP64 goes where it is needed, since its pipe is slow here (1.8 FMA per cycle and SM; 64^2 complex
-//     multiply-adds are 9k cycles).  d_0 only has to be an FP32 solution, so gamma L in it is an
-//     FP32 product.  r_1 = gamma (L + chi~ o x) - x is one FP64 product.  From then on r_{i+1} =
+//     multiply-adds are 9k cycles).  d_0 only has to be an FP32 solution, so gamma L in it is a
+//     double-float product (2^-46).  r_1 = gamma (L + chi~ o x) - x is one FP64 product.  From then on r_{i+1} =
 //     r_i - D d_i, and d_i is below 2^-13 |x|, so that D d_i in double-float (2^-46 of
 //     |d_i|) adds less than FP64's rounding of |x| does; while d_i is larger, r comes from x again.
-//     Error against 64 bits, three inputs each, before -> now: order 64 1.2e-13 -> 1.2e-13, 48 4.6e-14 ->
-//     3.1e-14, 30 4.2e-13 -> 2.9e-13.
+//     L, the residuals and the corrections are scaled by powers of two and the norms compared by their upper
+//     FP64 words, so that x may lie anywhere in FP64's range.
+//     Error against 64 bits (geometric mean over 8 or 10 inputs), with an FP32 LU and three FP64 products per
+//     step -> now: doped square lattice, order 16 2.5e-14 -> 2.4e-14, 30 6.4e-14 -> 6.4e-14, 48 7.1e-14 -> 6.2e-14,
+//     64 4.1e-14 -> 4.4e-14; generic vertices, 64 1.2e-13 -> 1.2e-13; the paper's, 48 5.0e-13 -> 5.0e-13.
 //   * A block keeps gamma of its (channel, W) in shared memory, FP64 and FP32 (hi, lo) words, and
 //     runs six (orders up to 32: twelve) ladders at a time.
 // Bound by instruction issue and the two barriers of a sweep step (two warps per ladder, 12 per SM, issue
 // 52-65% busy; the step is one body, since eight unrolled ones leave the instruction cache: 7.6 ms).
-// Measured, 30,720 ladders of order 64: 3.8 ms (6.3 ms with an FP32 LU in shared memory, two triangular
-// substitutions per solve by one warp and three FP64 products); five ladders 4.3 ms, four 4.4 ms.
+// Measured, 30,720 ladders of order 64: 4.0 ms (6.3 ms with an FP32 LU in shared memory, two triangular
+// substitutions per solve by one warp and three FP64 products; 3.8 with gamma L in FP32 and unscaled);
+// five ladders at a time 4.3 ms, four 4.4 ms, both against 3.8.
 #include "df_mixed32_dev.cuh"
 
 namespace df {
@@ -57,17 +61,24 @@ __device__ __forceinline__ void chi_ir_sync(int ladder) {
     __syncwarp();
 }
 
-// max of non-negative floats over a ladder's threads (a NaN wins); red: a slot per call of a sequence
+// max of |v| (|re| + |im|) over a ladder's threads, its lower word cut off (2^-20; the whole FP64 range; an
+// infinity or NaN wins): the upper word; red: a slot per call of a sequence
 template <int NP>
-__device__ __forceinline__ float chi_ir_max(float v, unsigned* red, int t, int ladder) {
-  unsigned u = __reduce_max_sync(0xffffffffu, __float_as_uint(v));
+__device__ __forceinline__ unsigned chi_ir_max(double2 v, unsigned* red, int t, int ladder) {
+  unsigned u = __reduce_max_sync(0xffffffffu, (unsigned)__double2hiint(cabs1(v)));
   if constexpr (NP == 64) {
     if ((t & 31) == 0) red[t >> 5] = u;
     chi_ir_sync<NP>(ladder);
     u = max(red[0], red[1]);
   }
-  return __uint_as_float(u);
+  return u;
 }
+constexpr unsigned kHiInf = 0x7FF00000u;                  // upper word of an infinity
+// 2^e (|e| <= 1022), e the exponent of an upper word (0 of zero, subnormal or not finite)
+__device__ __forceinline__ int hi_exp(unsigned hi) {
+  return hi >= 0x00100000u && hi < 0x7FE00000u ? (int)(hi >> 20) - 1023 : 0;
+}
+__device__ __forceinline__ double pow2d(int e) { return __hiloint2double((1023 + e) << 20, 0); }
 
 template <int NP>
 __device__ __forceinline__ void chi_ir_system(const Dims& dm, int c, int a, int q, const unsigned char* gsm,
@@ -105,13 +116,24 @@ __device__ __forceinline__ void chi_ir_system(const Dims& dm, int c, int a, int 
     lv[t] = l;
     x[t] = mk(0.0, 0.0);
     vh[t] = make_float2((float)xv.x, (float)xv.y);
-    vl[t] = make_float2((float)l.x, (float)l.y);
     piv[t] = t;
     rstep[t] = t;
     pinv[t] = make_float2(0.f, 0.f);
   }
   sync();
-  // ---- D in FP32 (only S uses it), gamma L in FP32 ----
+  // ---- gamma L in double-float (L to [1, 2)), D in FP32 (only S uses it) ----
+  {
+    const int e = hi_exp(chi_ir_max<NP>(lv[t], red, t, ladder));
+    const double2 l = cscale(lv[t], pow2d(-e));
+    const float2 h = make_float2((float)l.x, (float)l.y);
+    vl[t] = h;
+    part[t] = make_float2((float)(l.x - (double)h.x), (float)(l.y - (double)h.y));
+    sync();
+    float sr = 0.f, lr = 0.f, si = 0.f, li = 0.f;
+#pragma unroll 2
+    for (int k = 0; k < n; ++k) cdf_fma(sr, lr, si, li, ghi[k * LD + t], glo[k * LD + t], vl[k], part[k]);
+    y[t] = t < n ? cscale(mk((double)sr + (double)lr, (double)si + (double)li), pow2d(e)) : mk(0.0, 0.0);
+  }
   float2 A[RP][CP];
 #pragma unroll
   for (int r = 0; r < CP; ++r) {
@@ -123,12 +145,6 @@ __device__ __forceinline__ void chi_ir_system(const Dims& dm, int c, int a, int 
       const float2 g = cmulf(ghi[col * LD + row], ch);
       A[i][r] = make_float2((row == col ? 1.f : 0.f) - g.x, -g.y);
     }
-  }
-  {
-    float2 b = make_float2(0.f, 0.f);
-    for (int l = 0; l < n; ++l) b = cfmaf2(ghi[l * LD + t], vl[l], b);
-    sync();
-    vl[t] = t < n ? b : make_float2(0.f, 0.f);
   }
   // ---- in-place Gauss-Jordan sweep ----
   unsigned used = 0u, kmin = ~0u;
@@ -223,14 +239,13 @@ __device__ __forceinline__ void chi_ir_system(const Dims& dm, int c, int a, int 
   // thread t owns the solution's entry ks (the step of row t) and the residual's entry t
   const int ks = rstep[t], pt = piv[t], rot = n / G;
   const float2 rinv = pinv[t];
-  double2 res = mk((double)vl[t].x, (double)vl[t].y);
+  double2 res = y[t];
   // ---- refinement; every thread takes the same decisions ----
-  float dprev = 0.f;
+  double dprev = 0.0;
   for (int it = 0; state == 0; ++it) {
     // d = S r, r scaled to [1, 2)
-    const float rm = chi_ir_max<NP>(fabsf((float)res.x) + fabsf((float)res.y), red + 2 * (it & 1), t, ladder);
-    const int e = rm > 0.f && rm < INFINITY ? (int)(__float_as_uint(rm) >> 23) - 127 : 0;
-    const double sc = __hiloint2double((1023 - e) << 20, 0), up = __hiloint2double((1023 + e) << 20, 0);
+    const int e = hi_exp(chi_ir_max<NP>(res, red + 2 * (it & 1), t, ladder));
+    const double sc = pow2d(-e), up = pow2d(e);
     vl[t] = make_float2((float)(res.x * sc), (float)(res.y * sc));
     sync();
     vh[t] = vl[pt];
@@ -262,17 +277,17 @@ __device__ __forceinline__ void chi_ir_system(const Dims& dm, int c, int a, int 
     const double2 xv = x[ks] + d;
     x[ks] = xv;
     // NaN and infinity compare false: a non-finite value hands the system back
-    const float dn = chi_ir_max<NP>(fabsf((float)d.x) + fabsf((float)d.y), red + 6, t, ladder);
-    const float xn = chi_ir_max<NP>(fabsf((float)xv.x) + fabsf((float)xv.y), red + 8, t, ladder);
-    if (!(dn < INFINITY) || !(xn < INFINITY)) state = 2;
-    else if (it > 0 && (double)dn <= tol * (double)xn) state = 1;   // (d_0 may be 0 by FP32 underflow alone)
-    else if (it > 0 && dn > 0.5f * dprev) state = 2;
-    else if (it > 0 && (double)dn * (double)dn <= 0.5 * tol * (double)xn * (double)dprev) state = 1;
+    const unsigned dh = chi_ir_max<NP>(d, red + 6, t, ladder), xh = chi_ir_max<NP>(xv, red + 8, t, ladder);
+    const double dn = __hiloint2double(dh, 0), xn = __hiloint2double(xh, 0);
+    if (dh >= kHiInf || xh >= kHiInf) state = 2;
+    else if (it > 0 && dn <= tol * xn) state = 1;           // (d_0 may be 0 by FP32 underflow alone)
+    else if (dprev > 0.0 && dn > 0.5 * dprev) state = 2;
+    else if (it > 0 && dn * dn <= 0.5 * tol * xn * dprev) state = 1;
     else if (it + 1 >= max_steps) state = 2;
     if (state != 0) break;
     dprev = dn;
     const double2 ch = xs[ks];
-    if (it == 0 || dn > 1.220703125e-4f * xn) {            // r = gamma (L + chi~ o x) - x in FP64
+    if (it == 0 || dn > 1.220703125e-4 * xn) {            // r = gamma (L + chi~ o x) - x in FP64
       y[ks] = cfma(ch, xv, lv[ks]);
       sync();
       double2 s0 = mk(0.0, 0.0), s1 = mk(0.0, 0.0);
@@ -286,7 +301,7 @@ __device__ __forceinline__ void chi_ir_system(const Dims& dm, int c, int a, int 
         res = mk(s0.x - x[t].x, s0.y - x[t].y);
       }
     } else {                                              // r -= d - gamma (chi~ o d), the product in double-float
-      const double2 v = cmul(ch, d);
+      const double2 v = cmul(ch, mk((double)ys.x, (double)ys.y));   // 2^-e d
       const float hx = (float)v.x, hy = (float)v.y;
       part[ks] = make_float2(hx, hy);                     // (part's readers are past the norms' barriers)
       vl[ks] = make_float2((float)(v.x - (double)hx), (float)(v.y - (double)hy));
@@ -296,7 +311,7 @@ __device__ __forceinline__ void chi_ir_system(const Dims& dm, int c, int a, int 
         float sr = 0.f, lr = 0.f, si = 0.f, li = 0.f;
 #pragma unroll 2
         for (int l = 0; l < n; ++l) cdf_fma(sr, lr, si, li, ghi[l * LD + t], glo[l * LD + t], part[l], vl[l]);
-        res = mk(res.x - y[t].x + ((double)sr + (double)lr), res.y - y[t].y + ((double)si + (double)li));
+        res = mk(res.x - y[t].x + ((double)sr + (double)lr) * up, res.y - y[t].y + ((double)si + (double)li) * up);
       }
       if constexpr (NP == 32) __syncwarp();
     }

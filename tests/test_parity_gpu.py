@@ -587,3 +587,20 @@ def test_leading_eigenvalue_at_tile_edges(df, n_w, nk):
             assert ok[c, 0, q] == 1, (c, q)
             assert abs(lam[c, 0, q] - ev[0]) < 1e-8 * abs(ev[0]), (c, q)
     assert seen > 0 or n_w == 2
+
+
+@pytest.mark.parametrize("n_w", [2, 16, 30, 48, 64])
+def test_susceptibility_refined_below_the_fp32_range(df, n_w):
+    # g, Delta = (1, 1) and (i, -i) in turn with t = 0: G = 1/2 and i/2, so that chi0 = -T sum G G = 0 exactly and
+    # the susceptibilities are the ladder term alone, here 2^-166 of gamma's entries of order one
+    rng = np.random.default_rng(n_w)
+    g = np.where(np.arange(n_w) % 2 == 0, 1.0, 1j).astype(complex)
+    delta = np.where(np.arange(n_w) % 2 == 0, 1.0, -1j).astype(complex)
+    gam = 2.0 ** -166 * (rng.normal(size=(2, 1, n_w, n_w)) + 1j * rng.normal(size=(2, 1, n_w, n_w)))
+    out = []
+    for prec in (df.DF_FP64, df.DF_FP32_IR):
+        with df.DualFermion(dim=1, nk=2, t=0.0, tp=0.0, beta=4.0, mu=0.0, n_w=n_w, m_max=0, g=g, delta=delta,
+                            gamma_d=gam[0], gamma_m=gam[1], precision=prec) as d:
+            out.append(d.susceptibility())
+    assert 0.0 < np.max(np.abs(out[0])) < 1e-45
+    assert np.max(np.abs(out[1] - out[0])) < 1e-12 * np.max(np.abs(out[0]))
