@@ -56,6 +56,9 @@ struct PointDev {
   int* flags;    // [4]
 };
 
+// the right-hand-side chunk of the FP64 solve at an order
+__host__ __device__ inline int default_nc(int n) { return n <= 32 ? n : (n <= 64 ? 32 : 16); }
+
 __device__ __forceinline__ int find_segment(const long* start, int nseg, long x) {
   // largest k with start[k] <= x (start[0] = 0, start[nseg] = total)
   int lo = 0, hi = nseg - 1;
@@ -217,23 +220,26 @@ batch_bse_f64_kernel(const PointDev* __restrict__ pts, const int* __restrict__ o
 // the FP64 LU over the mixed ladders handed back this pass (redo[0] entries)
 __global__ void __launch_bounds__(kBseThreads)
 batch_bse_f64_list_kernel(const PointDev* __restrict__ pts, const int* __restrict__ redo, double2* __restrict__ ws,
-                          size_t ws_stride) {
+                          size_t ws_stride, int wave, int long_list) {
   extern __shared__ double2 sm[];
   __shared__ BseF64Shared sh;
   const int count = redo[0];
+  // one launch for lists of up to a wave of its blocks (shared memory, kListSmemOrder), one for longer ones
+  if ((count > wave) != (long_list != 0)) return;
   // a short list is spread over the grid as ranges of right-hand sides (bse_f64_kernel)
   const int parts = count > 0 && (int)gridDim.x > count ? min((int)gridDim.x / count, 8) : 1;
   for (int s = blockIdx.x; s < count * parts; s += gridDim.x) {
     const int code = redo[1 + s / parts], part = s % parts;
     const PointDev& P = pts[code >> 24];
     const Dims& dm = P.ldm;
-    const int nc = min(dm.n_w, kListChunk), chunks = (dm.n_w + nc - 1) / nc, cpp = (chunks + parts - 1) / parts;
+    const int nc = long_list ? default_nc(dm.n_w) : min(dm.n_w, kListChunk);
+    const int chunks = (dm.n_w + nc - 1) / nc, cpp = (chunks + parts - 1) / parts;
     const int jb = part * cpp * nc, je = min(jb + cpp * nc, dm.n_w);
     if (jb >= je) continue;
     const int sys = code & 0xFFFFFF;
     const int c = sys / (dm.nb * dm.N), rem = sys - c * dm.nb * dm.N;
     const int a = rem / dm.N, q = rem - a * dm.N;
-    const bool lu_smem = dm.n_w <= kListSmemOrder;
+    const bool lu_smem = dm.n_w <= (long_list ? kLuSmemOrder : kListSmemOrder);
     const BseSmem L = bse_layout(dm.n_w, nc, lu_smem);
     double2* LU = lu_smem ? sm + L.lu : ws + blockIdx.x * ws_stride;
     bse_f64_system(dm, c, a, q, nc, P.gam, P.gg, P.lchi, P.lkc, LU, sm + L.y, sm + L.xs, sm + L.invu, sh, P.flags, 0,
@@ -488,8 +494,8 @@ struct df_batch {
   double2* ws = nullptr;                       // global LU scratch (FP64, n > 96)
   size_t ws_stride = 0;
   int* d_redo = nullptr;                       // mixed ladders handed back to the FP64 LU: count, list
-  int redo_grid = 0;
-  size_t redo_smem = 0;
+  int redo_grid[2] = {0, 0};            // short, long list
+  size_t redo_smem[2] = {0, 0};
   double* d_out = nullptr;                     // [3 npts] residual, active, flags
   bool any_sym = false;                        // some point uses the point-group reduction
   double* h_out = nullptr;
@@ -522,7 +528,6 @@ df_status bfail(df_batch* b, df_status s, const char* what, cudaError_t e = cuda
       return bfail((b), e__ == cudaErrorMemoryAllocation ? DF_ERR_OOM : DF_ERR_CUDA, (what), e__); \
   } while (0)
 
-int default_nc(int n) { return n <= 32 ? n : (n <= 64 ? 32 : 16); }
 
 size_t align_up(size_t x) { return (x + 255) & ~(size_t)255; }
 
@@ -556,9 +561,11 @@ df_status record_pass(df_batch* b) {
     B_CUDA(b, cudaGetLastError(), "batch ladder");
   }
   if (b->d_redo) {
-    batch_bse_f64_list_kernel<<<b->redo_grid, kBseThreads, b->redo_smem, s>>>(b->d_pts, b->d_redo, b->ws,
-                                                                              b->ws_stride);
-    B_CUDA(b, cudaGetLastError(), "batch hand-back ladders");
+    for (int k = 0; k < 2; ++k) {
+      batch_bse_f64_list_kernel<<<b->redo_grid[k], kBseThreads, b->redo_smem[k], s>>>(b->d_pts, b->d_redo, b->ws,
+                                                                                      b->ws_stride, b->redo_grid[0], k);
+      B_CUDA(b, cudaGetLastError(), "batch hand-back ladders");
+    }
   }
   if (b->any_sym) {
     batch_wedge_scatter_kernel<<<dim3(kWedgeBlocks, b->npts), 256, 0, s>>>(b->d_pts);
@@ -981,20 +988,23 @@ df_status df_batch_init(df_batch** out, int npts, const df_point* pts, int preci
     }
     if (mixed_ladders > 0) {
       BALLOC(b->d_redo, sizeof(int) * (1 + (size_t)mixed_ladders), "hand-back list");
-      size_t sm_max = 0;
       for (auto& g : b->groups)
         if (g.mixed)
           for (int p : g.order) {
             const int n = b->host_pts[p].dm.n_w;
-            sm_max = std::max(sm_max, sizeof(double2) * (size_t)bse_layout(n, std::min(n, kListChunk), n <= kListSmemOrder).total);
+            const int sm0 = bse_layout(n, std::min(n, kListChunk), n <= kListSmemOrder).total;
+            const int sm1 = bse_layout(n, default_nc(n), n <= kLuSmemOrder).total;
+            b->redo_smem[0] = std::max(b->redo_smem[0], sizeof(double2) * (size_t)sm0);
+            b->redo_smem[1] = std::max(b->redo_smem[1], sizeof(double2) * (size_t)sm1);
           }
-      b->redo_smem = sm_max;
       e = cudaFuncSetAttribute((const void*)batch_bse_f64_list_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)sm_max);
-      int per = 0;
-      if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, batch_bse_f64_list_kernel, kBseThreads, sm_max);
-      b->redo_grid = b->sms * std::min(std::max(per, 1), kLuScratchPerSm);   // the scratch has that many slices
+                               (int)std::max(b->redo_smem[0], b->redo_smem[1]));
+      for (int k = 0; k < 2; ++k) {
+        int per = 0;
+        if (e == cudaSuccess)
+          e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, batch_bse_f64_list_kernel, kBseThreads, b->redo_smem[k]);
+        b->redo_grid[k] = b->sms * std::min(std::max(per, 1), kLuScratchPerSm);   // the scratch has that many slices
+      }
       if (e != cudaSuccess) { st = bfail(b, DF_ERR_CUDA, "hand-back kernel", e); goto bad; }
     }
   }

@@ -30,18 +30,31 @@ __global__ void gamma_gt_kernel(int n, int count, const double2* __restrict__ ga
   }
 }
 
+// The hand-back list of a launch (list NULL: every system of the planes), whose length only the
+// device knows: the launch takes lists of above < length <= up_to, in ranges of nc right-hand sides up
+// to a length of short_up_to and of nc_long beyond it.
+struct LadderList {
+  const int* list = nullptr;
+  int spread = 0;
+  int above = -1, up_to = 0x7FFFFFFF, short_up_to = 0x7FFFFFFF, nc_long = 0;
+};
+
 template <bool LU_SMEM>
 __global__ void __launch_bounds__(kBseThreads)
 bse_f64_kernel(Dims dm, int ch0, int nch, int nc, const double2* __restrict__ gam,
                const double2* __restrict__ gg, const double2* __restrict__ chi,
                double2* __restrict__ kc, double2* __restrict__ ws, int* __restrict__ flags, int radius_K,
-               const double2* __restrict__ lam, const int* __restrict__ list, int spread) {
+               const double2* __restrict__ lam, LadderList ll) {
   extern __shared__ double2 sm[];
   __shared__ BseF64Shared sh;
   const int n = dm.n_w, N = dm.N, nb = dm.nb, na = dm.na;
+  const int* __restrict__ list = ll.list;
+  const int spread = ll.spread;
+  if (list && (list[0] <= ll.above || list[0] > ll.up_to)) return;
+  if (list && list[0] > ll.short_up_to) nc = ll.nc_long;
   const BseSmem L = bse_layout(n, nc, LU_SMEM);
   double2* LU = LU_SMEM ? sm + L.lu : ws + (size_t)blockIdx.x * n * n;
-  // the handle's planes of channels ch0 .. ch0 + nch - 1, or with `list` the
+  // the handle's planes of channels ch0 .. ch0 + nch - 1, or with a list its
   // list[0] systems (c N_W + a) N + q that follow it (ladders the mixed-precision
   // kernels handed back).  A short list is spread over up to `spread` blocks:
   // each ladder's right-hand-side chunks are split into `parts` column ranges,
@@ -213,11 +226,11 @@ cudaError_t launch_bse(df_ctx* c, int channel_mask) {
     const int grid = (int)(systems < c->bse_grid ? systems : c->bse_grid);
     if (bse_lu_in_smem(n)) {
       bse_f64_kernel<true><<<grid, kBseThreads, smem, c->stream>>>(dm, ch, nch, nc, c->gam, gg_ptr(c), c->chi,
-                                                                   c->kc, nullptr, flag_ptr(c), K, lam, nullptr, 0);
+                                                                   c->kc, nullptr, flag_ptr(c), K, lam, LadderList{});
     } else {
       bse_f64_kernel<false><<<grid, kBseThreads, smem, c->stream>>>(dm, ch, nch, nc, c->gam, gg_ptr(c), c->chi,
                                                                     c->kc, lu_ws_ptr(c), flag_ptr(c), K, lam,
-                                                                    nullptr, 0);
+                                                                    LadderList{});
     }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (both) break;
@@ -225,30 +238,52 @@ cudaError_t launch_bse(df_ctx* c, int channel_mask) {
   return cudaSuccess;
 }
 
-// the FP64 LU over the ladders the mixed-precision kernels handed back: list[0]
-// (read on the device) systems (c N_W + a) N + q, on the persistent grid; a
-// list shorter than the SM count is spread over the SMs by right-hand-side ranges
-cudaError_t launch_bse_f64_list(df_ctx* c, const int* list) {
-  const Dims& dm = c->dm;
-  const int n = dm.n_w;
-  const int nc = n < kListChunk ? n : kListChunk;
-  const bool in_smem = n <= kListSmemOrder;
-  const size_t smem = sizeof(double2) * (size_t)bse_layout(n, nc, in_smem).total;
-  int sms = 0;
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
-  const void* fn = in_smem ? (const void*)bse_f64_kernel<true> : (const void*)bse_f64_kernel<false>;
+template <bool LU_SMEM>
+static cudaError_t launch_list(df_ctx* c, int nc, int nc_smem, int max_grid, LadderList ll) {
+  const size_t smem = sizeof(double2) * (size_t)bse_layout(c->dm.n_w, nc_smem, LU_SMEM).total;
+  const void* fn = (const void*)bse_f64_kernel<LU_SMEM>;
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  int per_sm = 0;
-  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kBseThreads, smem)) != cudaSuccess) return e;
-  const int grid = in_smem ? sms * (per_sm < 1 ? 1 : per_sm) : c->bse_grid;   // (the scratch has bse_grid slices)
-  if (in_smem)
-    bse_f64_kernel<true><<<grid, kBseThreads, smem, c->stream>>>(dm, 0, 2, nc, c->gam, gg_ptr(c), c->chi, c->kc, nullptr,
-                                                                 flag_ptr(c), 0, nullptr, list, grid);
-  else
-    bse_f64_kernel<false><<<grid, kBseThreads, smem, c->stream>>>(dm, 0, 2, nc, c->gam, gg_ptr(c), c->chi, c->kc,
-                                                                  lu_ws_ptr(c), flag_ptr(c), 0, nullptr, list, grid);
+  const int grid = max_grid < ll.up_to ? max_grid : ll.up_to;
+  ll.spread = grid;
+  bse_f64_kernel<LU_SMEM><<<grid, kBseThreads, smem, c->stream>>>(c->dm, 0, 2, nc, c->gam, gg_ptr(c), c->chi, c->kc,
+                                                                  LU_SMEM ? nullptr : lu_ws_ptr(c), flag_ptr(c), 0,
+                                                                  nullptr, ll);
   return cudaGetLastError();
+}
+
+// blocks of a shared-memory list launch that run at once (asked once per handle)
+static int list_wave(df_ctx* c, int nc) {
+  if (c->list_wave > 0) return c->list_wave;
+  const size_t smem = sizeof(double2) * (size_t)bse_layout(c->dm.n_w, nc, true).total;
+  int sms = 0, per_sm = 0;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
+  cudaFuncSetAttribute((const void*)bse_f64_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, bse_f64_kernel<true>, kBseThreads, smem);
+  return c->list_wave = sms * (per_sm < 1 ? 1 : per_sm);
+}
+
+// the FP64 LU over the ladders the mixed-precision kernels handed back: list[0]
+// (read on the device) systems (c N_W + a) N + q, on the persistent grid; a
+// list shorter than the grid is spread over it by right-hand-side ranges.  How the list is solved
+// follows from its length (kListSmemOrder): of the two launches of orders 41-96 one returns at once.
+cudaError_t launch_bse_f64_list(df_ctx* c, const int* list) {
+  const int n = c->dm.n_w, nc = n < kListChunk ? n : kListChunk, nc_long = bse_chunk(n);
+  LadderList ll;
+  ll.list = list;
+  ll.nc_long = nc_long;
+  if (n > kListSmemOrder) return launch_list<false>(c, nc_long, nc_long, c->bse_grid, ll);   // (the scratch has bse_grid slices)
+  const int wave = list_wave(c, n <= kLuSmemOrder ? nc_long : nc);
+  if (n <= kLuSmemOrder) {
+    ll.short_up_to = kListShort;
+    return launch_list<true>(c, nc, nc_long, wave, ll);
+  }
+  ll.up_to = wave;
+  const cudaError_t e = launch_list<true>(c, nc, nc, wave, ll);
+  if (e != cudaSuccess) return e;
+  ll.above = wave;
+  ll.up_to = 0x7FFFFFFF;
+  return launch_list<false>(c, nc_long, nc_long, c->bse_grid, ll);
 }
 
 // the ladder term of the susceptibilities for both channels: FP64 LU on the
@@ -308,7 +343,7 @@ cudaError_t launch_bse_both_raw(const Dims& dm, const double2* gam, const double
   const long systems = 2L * dm.nb * dm.N;
   const int grid = (int)(systems < grid_max ? systems : grid_max);
   bse_f64_kernel<true><<<grid, kBseThreads, smem, stream>>>(dm, 0, 2, nc, gam, gg, chi, kc, nullptr, flags, 0,
-                                                            nullptr, nullptr, 0);
+                                                            nullptr, LadderList{});
   return cudaGetLastError();
 }
 

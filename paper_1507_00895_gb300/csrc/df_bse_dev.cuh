@@ -15,13 +15,20 @@ constexpr int kBseThreads = 256;
 // Measured fractions of the FP64 peak (shared / global): order 40 64.6 / 63.8%,
 // 48 67.4 / 70.2%, 64 71.4 / 78.4%, 96 57 / 83%.
 constexpr int kLuSmemOrder = 40;
-// The hand-back lists are short, so that a ladder's own latency counts, not the blocks per
-// SM: shared memory as far as it reaches, and ranges of kListChunk right-hand sides
+// Hand-back lists are usually short, so that a ladder's own latency counts, not the blocks per
+// SM: shared memory as far as it reaches (kListSmemOrder), and ranges of kListChunk right-hand sides
 // spread over the idle blocks.  Measured, order 64: about 150 ladders 831 -> 587 us, about 30 390 -> 370 us
 // (the FP64 pipe of one SM needs 175 us for one range: the factorisation is repeated per range);
-// a 24-point batch's list 657 -> 366 us (it was not split before).
+// a 24-point batch's list 657 -> 366 us (it was not split before).  A list of more ladders than blocks in shared
+// memory run at once (a tight ladder_tol, inputs far outside the radius) is solved as the FP64 path solves its
+// ladders: global scratch beyond order 40 and default chunks.  Measured, us, shared memory / global
+// scratch: order 48, 640 ladders 816 / 799, 4,608 4455 / 4379; order 64 (one wave: 304), 192 727 / 955, 384 1260 / 1262, 4,608
+// 11050 / 9527; order 80 (152), 128 940 / 1502, 192 1878 / 1536, 4,608 29074 / 18125; order 96 (152), 128 1472 / 2425, 192
+// 2940 / 2478, 4,608 45534 / 30503.  Up to order 40 only the chunk changes, beyond kListShort ladders: order 32,
+// chunks of 16 / 32, 32 ladders 106 / 115, 64 119 / 115, 4,608 1636 / 1526.
 constexpr int kListSmemOrder = 96;
 constexpr int kListChunk = 16;
+constexpr int kListShort = 48;
 
 struct BseSmem {
   // offsets in double2 units inside the dynamic shared block

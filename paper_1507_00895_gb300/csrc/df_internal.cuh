@@ -291,6 +291,7 @@ struct df_ctx {
                                // df_init: the hand-back list before it is sized for the full grid)
   size_t bse_ws_bytes = 0;
   int bse_grid = 0;
+  int list_wave = 0;           // blocks of the hand-back list's shared-memory launch that run at once
   unsigned wait_spins = df::kMbarSpin;   // polls of the order 33-64 kernel's completion waits (df_selftest_ladder_wait)
   int iter_done = 0;
   int sigma_valid = 0;         // gk/gr reflect sigma

@@ -384,3 +384,54 @@ def test_zero_fp32_pivot_in_a_batch(df):
             with df.DualFermion.from_workload(w, eig_mode=0) as d:
                 d.iterate(1)
                 assert nrel(b.get_sigma(i), d.get_sigma()) < 1e-12, w.n_w
+
+
+@pytest.mark.parametrize("n_w,m_max", [(24, 3), (32, 3), (40, 4), (42, 4), (48, 4), (64, 3), (66, 2), (96, 2), (98, 2)])
+def test_long_hand_back_list(df, n_w, m_max):
+    """Lists longer than the blocks that run at once with their factors in shared memory (order 24: chunk lists only),
+    and one just as long as a plane: every ladder is the FP64 path's, bit for bit, on a handle, and the batch's
+    Sigma~ is within the FP64 parity bound."""
+    w = I.random_nonsymmetric(n_w, m_max, 1, 64, seed=n_w, scale=0.5)
+    with df.DualFermion.from_workload(w, eig_mode=0) as d64, \
+            df.DualFermion.from_workload(w, precision=df.DF_FP32_IR, eig_mode=0, ladder_tol=1e-300) as d:
+        d64.iterate(1)
+        d.bubble()
+        for mask, count in ((1, w.n_bos * w.N), (3, 2 * w.n_bos * w.N)):
+            d.bse(mask)
+            assert d.ladder_stats()[1] == count
+            k, k64 = d.get_kernel(), d64.get_kernel()
+            assert np.array_equal(k if mask == 3 else k[:1], k64 if mask == 3 else k64[:1])
+        d.sigma()
+        assert np.array_equal(d.get_sigma(), d64.get_sigma())
+
+
+def test_long_hand_back_list_in_a_batch(df):
+    # ladders near the edge of FP32 (square32_tp's critical planes at every momentum): hundreds are handed back, of
+    # several orders at once, some of them beyond the shared-memory order
+    ws = [I.workload("square32_tp", nk=16, n_w=n, m_max=1) for n in (24, 48, 64, 80, 98)]
+    for w in ws:                                            # W = 0 scaled to |lambda| ~ 1e7: the list takes the plane
+        w.gamma_uu[1] *= 1e4
+        w.gamma_ud[1] *= 1e4
+    with df.DualFermionBatch(ws) as b64, df.DualFermionBatch(ws, precision=df.DF_FP32_IR) as b:
+        b64.iterate(1)
+        b.iterate(1)
+        for i in range(len(ws)):
+            assert nrel(b.get_sigma(i), b64.get_sigma(i)) < TOL_SIGMA, ws[i].n_w
+
+
+def test_long_hand_back_list_takes_the_fp64_path_s_time(df):
+    # order 96, 3,200 ladders, all handed back: the second solve takes the FP64 path's time (22 ms; shared-memory
+    # factors, one block per SM, took 1.45 times as long), beside the mixed kernel's own 3.4 ms
+    w = I.random_nonsymmetric(96, 12, 1, 64, seed=1, scale=0.5)
+    t = []
+    for kw in (dict(), dict(precision=df.DF_FP32_IR), dict(precision=df.DF_FP32_IR, ladder_tol=1e-300)):
+        with df.DualFermion.from_workload(w, eig_mode=0, **kw) as d:
+            d.bubble()
+            d.bse(3)
+            best = 1e30
+            for _ in range(3):
+                d.set_timing(True)
+                d.bse(3)
+                best = min(best, d.get_timing()["bse"][0])
+            t.append(best)
+    assert t[2] - t[1] < 1.2 * t[0], t
