@@ -156,7 +156,9 @@ gemm_tc_kernel(const GemmArgs g) {
   unsigned char* gsm = reinterpret_cast<unsigned char*>(((uintptr_t)gsm_raw + 1023) & ~(uintptr_t)1023);
   constexpr int kA = TM * 128 * KB, kB = TN * 128 * KB, kStage = kA + kB;
   constexpr int kTmem = TN < 32 ? 32 : TN;
-  const int m0 = blockIdx.x * TM, n0 = blockIdx.y * TN;
+  // (tiles in a one-dimensional grid, those of one column block together: the other dimensions end at 65,535)
+  const int mtiles = (g.M + TM - 1) / TM, bm = blockIdx.x % mtiles, bn = blockIdx.x / mtiles;
+  const int m0 = bm * TM, n0 = bn * TN;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int nit = (g.nkb + KB - 1) / KB;
   if (warp == 0) tmem_alloc_cols<kTmem>(&tslot_s);
@@ -246,7 +248,7 @@ gemm_tc_kernel(const GemmArgs g) {
           const uint2 v = make_uint2(pack_bf16(w[e].x, w[e].y), pack_bf16(w[e].z, w[e].w));
           const unsigned o = (unsigned)((k & 7) * 128 + ((((c & 63) >> 3) ^ (k & 7)) << 4) + (c & 4) * 2);
           *reinterpret_cast<uint2*>(bt + (c >> 6) * 8192 + (k >> 3) * 1024 + o) = v;
-          if (g.wsh && blockIdx.x == 0)
+          if (g.wsh && bm == 0)
             *reinterpret_cast<uint2*>(g.wsh + ((size_t)((n0 + c) >> 6) * g.wsh_rg + it * 8 + (k >> 3)) * 1024 + o) = v;
         }
         if (it + 1 < nit) fetch(it + 1);
@@ -256,7 +258,8 @@ gemm_tc_kernel(const GemmArgs g) {
       }
       if (!ok) fail_s = 1;
     }
-    if (!mbar_wait(&done_s, 0u)) fail_s = 1;
+    // (the whole sum's products: the limit grows with their number)
+    if (!mbar_wait(&done_s, 0u, kMbarSpin * (1u + min(nit >> 12, 1000)))) fail_s = 1;
     tc05_fence_after();
   }
   __syncthreads();
@@ -326,7 +329,7 @@ gemm_tc_kernel(const GemmArgs g) {
                 s += z;
               }
             }
-            g.part_col[(size_t)(blockIdx.x * 4 + q) * g.N + n] = s;
+            g.part_col[(size_t)(bm * 4 + q) * g.N + n] = s;
           }
         }
         if (dz) {
@@ -359,7 +362,7 @@ gemm_tc_kernel(const GemmArgs g) {
   if (!fail && g.epi == kEpiLoss && tid == 0) {
     float s = 0.f;
     for (int w = 0; w < 8; ++w) s += loss_s[w];
-    g.part_loss[blockIdx.y * gridDim.x + blockIdx.x] = s;
+    g.part_loss[blockIdx.x] = s;
   }
   if (warp == 0) tmem_dealloc_cols<kTmem>(tmem);
 }
@@ -492,8 +495,9 @@ cudaError_t launch_gemm(cudaStream_t s, const GemmArgs& g) {
   auto fn = gemm_tc_kernel<TM, TN, KB, NS, AMN, BMN, WF32>;
   cudaError_t e = cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
-  const dim3 grid((g.M + TM - 1) / TM, (g.N + TN - 1) / TN);
-  fn<<<grid, kGemmThreads, smem, s>>>(g);
+  const long grid = (long)((g.M + TM - 1) / TM) * (((long)g.N + TN - 1) / TN);
+  if (grid > 0x7FFFFFFFL) return cudaErrorInvalidConfiguration;
+  fn<<<(unsigned)grid, kGemmThreads, smem, s>>>(g);
   return cudaGetLastError();
 }
 

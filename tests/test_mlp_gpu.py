@@ -152,3 +152,27 @@ def test_products_at_tile_edges(env, dims, batch, max_batch):
         for part in (slice(o, o + nw), slice(o + nw, o + nw + dims[l + 1])):
             assert nrel(g[part], ref[part]) < 1e-2, (l, part)
         o += nw + dims[l + 1]
+
+
+def test_more_columns_than_a_grid_s_second_dimension_holds(env):
+    """65,536 column tiles of 128 outputs: forward, loss and the output layer's gradient against the oracle, bounds as
+    above."""
+    df, torch = env
+    dims = (1, 1, 1, 1, 65535 * 128 + 1)
+    net = df.MLP(dims[0], dims[-1], width=dims[1], max_batch=1, seed=3)
+    rng = np.random.default_rng(7)
+    x = rng.normal(size=(1, 1)).astype(np.float32)
+    t = rng.normal(size=(1, dims[-1])).astype(np.float32)
+    xd, td = torch.from_numpy(x).cuda(), torch.from_numpy(t).cuda()
+    p = net.params().astype(np.float64)
+    y = torch.empty((1, dims[-1]), dtype=torch.float32, device="cuda")
+    net.forward(xd, y)
+    torch.cuda.synchronize()
+    assert nrel(y.cpu().numpy(), M.forward(p, dims, x, rounding=True)[-1]) < 5e-3
+    loss = net.gradients(xd, td)
+    g = net.grads()
+    ref_loss, ref = M.loss_and_grads(p, dims, x, t, rounding=True)
+    assert abs(loss - ref_loss) < 1e-3 * ref_loss
+    last = slice(len(g) - 2 * dims[-1], len(g) - dims[-1]), slice(len(g) - dims[-1], len(g))
+    for part in last:
+        assert nrel(g[part], ref[part]) < 1e-2
