@@ -74,9 +74,10 @@ typedef enum df_status {
 
 typedef enum df_precision {
   DF_FP64 = 0,       /* every step in FP64 (complex128) */
-  DF_FP32_IR = 1     /* ladder solves factorised in FP32 (complex64) and refined by
-                        one correction with an extended-precision residual (exact
-                        digit products on the tensor cores; below order 17 double-float).  Per ladder, rho = max|correction| / max|diag Gamma|
+  DF_FP32_IR = 1     /* ladder solves inverted in FP32 (complex64) and refined by
+                        one correction from a product held to ~2^-47 (exact digit
+                        products on the tensor cores; mixed_sweep = 1: double-float).  Per
+                        ladder, rho = max|correction| / max|diag Gamma|
                         predicts the error left (~rho^2 of diag Gamma's largest entry);
                         a ladder with rho^2 > ladder_tol is solved again by the FP64 LU
                         (ladder_fallback = 1) or reported (DF_ERR_REFINE_STALL).  Bubble,
@@ -422,7 +423,7 @@ df_status df_bse_noalloc(const double* gamma, const double* chi, int n_w, int n_
                          double* kernel, void* stream);
 
 /* Self-test of the bounded device-side wait used by the tensor-core
- * residual of the mixed path (n_w 33-64): a one-warp kernel on the current
+ * products of the mixed path (n_w > 32): a one-warp kernel on the current
  * device initialises a shared-memory barrier, completes it only when
  * arrive != 0, and waits for it with a limit of `spins` polls.  Returns
  * DF_ERR_TIMEOUT when the wait gave up (arrive = 0), DF_OK when it saw the

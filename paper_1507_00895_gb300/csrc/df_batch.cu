@@ -50,8 +50,8 @@ struct PointDev {
   int active;    // 1 until converged
   double mix, tol, resid;
   double2 *g, *delta, *gam, *gg, *g0, *gk, *gr, *chi, *kc, *prod, *sigma;
-  float2 *gam_hi, *gam_lo, *gg_hi, *gg_lo;   // mixed: FP32 (hi, lo) of gam and gg
-  unsigned char* gdig;                         // mixed: gamma's digits
+  float2 *gg_hi, *gg_lo;      // mixed: FP32 (hi, lo) of gg
+  unsigned char* gdig;        // mixed: gamma's digits, column weights and (hi, lo) words
   double* red;   // [2 n_w + 4]
   int* flags;    // [4]
 };
@@ -128,7 +128,7 @@ batch_residual_kernel(PointDev* __restrict__ pts, double* __restrict__ out) {
   }
 }
 
-// per-point set-up: Eq. gd0, gamma o gamma^T, gamma (hi, lo), Dyson + FFT
+// per-point set-up: Eq. gd0, gamma o gamma^T and its (hi, lo) words, gamma's digits
 __global__ void batch_setup_elem_kernel(const PointDev* __restrict__ pts, int p) {
   const PointDev& P = pts[p];
   const int total = P.dm.ne * P.dm.N;
@@ -143,12 +143,8 @@ __global__ void batch_setup_elem_kernel(const PointDev* __restrict__ pts, int p)
     const double2* G = P.gam + mat * n * n;
     const double2 w = cmul(G[i * n + j], G[j * n + i]);
     P.gg[idx] = w;
-    if (P.gam_hi) {
-      const double2 v = P.gam[idx];
-      float hx = (float)v.x, hy = (float)v.y;
-      P.gam_hi[idx] = make_float2(hx, hy);
-      P.gam_lo[idx] = make_float2((float)(v.x - (double)hx), (float)(v.y - (double)hy));
-      hx = (float)w.x; hy = (float)w.y;
+    if (P.gg_hi) {
+      const float hx = (float)w.x, hy = (float)w.y;
       P.gg_hi[idx] = make_float2(hx, hy);
       P.gg_lo[idx] = make_float2((float)(w.x - (double)hx), (float)(w.y - (double)hy));
     }
@@ -782,7 +778,7 @@ df_status df_batch_init(df_batch** out, int npts, const df_point* pts, int preci
     total += align_up(sizeof(double2) * (size_t)dm.n_w * dm.N);  // sigma
     total += align_up(sizeof(double) * (2 * dm.n_w + 4));
     total += align_up(sizeof(int) * 4);
-    if (P.mixed) total += align_up(sizeof(float2) * nv) * 4;      // gam hi, lo; gg hi, lo
+    if (P.mixed) total += align_up(sizeof(float2) * nv) * 2;      // gg hi, lo
     if (P.mixed) total += align_up((size_t)2 * dm.nb * batch_digit_bytes(dm.n_w));   // gamma's digits
     if (P.sym) {
       const size_t nw = (size_t)dm.nb * dm.n_w * P.n_orb;
@@ -828,8 +824,6 @@ df_status df_batch_init(df_batch** out, int npts, const df_point* pts, int preci
     P.red = (double*)take(sizeof(double) * (2 * dm.n_w + 4));
     P.flags = (int*)take(sizeof(int) * 4);
     if (P.mixed) {
-      P.gam_hi = (float2*)take(sizeof(float2) * nv);
-      P.gam_lo = (float2*)take(sizeof(float2) * nv);
       P.gg_hi = (float2*)take(sizeof(float2) * nv);
       P.gg_lo = (float2*)take(sizeof(float2) * nv);
       P.gdig = (unsigned char*)take((size_t)2 * dm.nb * batch_digit_bytes(dm.n_w));

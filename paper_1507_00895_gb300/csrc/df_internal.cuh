@@ -22,11 +22,10 @@ constexpr int kFlagRefine = 16;     // a mixed-precision ladder missed its error
 
 constexpr unsigned kMbarSpin = 1u << 22;   // polls of a bounded wait on a shared-memory barrier before it gives up
 
-// Per-ladder error control of the mixed-precision ladder solves.  After the
-// one correction E of X0 ~ D^-1 gamma, rho = max_j |E_jj| / max_j |Gamma_jj|
-// (|re| + |im|) is the relative size of the correction; with a fixed FP32
-// factorisation each correction shrinks the error by about the same factor,
-// so the error left in diag Gamma is about rho^2 of its largest entry.  A
+// Per-ladder error control of the mixed-precision ladder solves.  With S ~ D^-1 in FP32, T = S gamma and
+// R = 1 - S D, Gamma = T + R T + R^2 Gamma; E = diag(R T) is the one correction taken, rho = max_j
+// |E_jj| / max_j |Gamma_jj| (|re| + |im|) its relative size, and what is left out, diag(R^2 Gamma),
+// is about rho^2 of diag Gamma's largest entry.  A
 // ladder with rho^2 above rho2_max (or a non-finite value) is appended to
 // the hand-back list (redo[0] = count, redo[1 + i] = (c N_W + a) N + q) for
 // the FP64 LU, or, without a list, flagged kFlagRefine.  worst receives the

@@ -98,7 +98,7 @@ bse_mixed64_kernel(Dims dm, int ch0, int nch, const float2* __restrict__ gg_hi, 
   m64_teardown(blk);
 }
 
-// Self-test of the bounded wait the tensor-core residual uses: one warp
+// Self-test of the bounded wait the ladder kernels' tensor-core products use: one warp
 // initialises an mbarrier (one arrival expected), arrives on it only when
 // `arrive` is set, and waits for its first phase with a limit of `spins`
 // polls; a wait that gives up sets kFlagTcTimeout.  Nothing else runs.
@@ -128,8 +128,8 @@ static int mixed_np(int n) { return mixed_pad(n); }
 
 bool mixed_supported(int n_w) { return mixed_np(n_w) <= 128; }
 
-// gamma hi, lo; gamma o gamma^T hi, lo (orders > 64: gamma^T hi, lo); gamma's
-// digits (tensor-core residual); then the error control's words: the call's
+// gamma hi, lo (df_chi.cu and mixed_sweep = 1); gamma o gamma^T hi, lo (mixed_sweep = 1: gamma^T hi, lo); gamma's
+// digits, weights and words (orders <= 64); then the error control's words: the call's
 // largest rho^2 and the hand-back list (count + 2 N_W N system indices)
 static size_t mixed_check_offset(const Dims& dm) {
   const int np = mixed_np(dm.n_w);

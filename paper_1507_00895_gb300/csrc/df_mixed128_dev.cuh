@@ -13,6 +13,12 @@
 //     slice), the accumulators 192 columns of tensor memory;
 //   * T's leading words stay in tensor memory (lane j, 2 x 128 columns) until
 //     all rows of R are there: lane j then sums R_jm T_mj.
+// The digit sums: a weight 2^-9d of d + 1 pairs reaches (d + 1) x 128 x 2^16, so that d <= 1 is
+// exact (2^24).  d = 2 and 3 could pass 2^24 (by at most 1.5 and 2) where a row of S and a column of gamma
+// have digits near 256 of equal sign throughout; a K step beyond rounds by a unit or two, so that the bound on T
+// is 2^-28 of max|S_i| max|gamma_j| there.  Measured on matrices a (+-1), Sylvester's of order 128, with a
+// chosen to pass 2^24 by a fifth: error 1.9e-12 of the bracket, 1.3e-12 with an a that does not: the
+// remainder of the sweep, not these roundings.
 // Tile t's finishing lanes 64 t .. 64 t + 63 are the columns j themselves: the
 // digit rows are [gamma_re; gamma_im] in tile 0 and [gamma_im; gamma_re] in tile 1.
 //

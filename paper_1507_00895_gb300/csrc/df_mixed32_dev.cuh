@@ -270,7 +270,8 @@ __device__ __forceinline__ void m32_system(const Dims& dm, int c, int a, int q, 
       }
     }
   }
-  const bool zero = (kmin & ~0x1Fu) == 0u;                // an exactly zero FP32 pivot
+  // an exactly zero FP32 pivot (a used row may then have been taken again, so that rows of S collide: not used)
+  const bool zero = (kmin & ~0x1Fu) == 0u;
   if (zero && lane == 0) zero_pivot(mc, flags);
   // ---- S to shared memory in logical order: row `step`, column piv[c]; padding zero ----
   __syncwarp();

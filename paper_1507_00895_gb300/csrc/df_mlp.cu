@@ -467,7 +467,6 @@ struct df_mlp {
   float* part_loss = nullptr;
   long loss_blocks = 0;         // capacity of part_loss
   int* d_timeout = nullptr;  // set by a tensor-core GEMM whose bounded wait gave up
-  float* h_loss = nullptr;
   long step = 0;
 };
 
@@ -502,7 +501,9 @@ cudaError_t launch_gemm(cudaStream_t s, const GemmArgs& g) {
 }
 
 // forward and weight-gradient tiles: 128 columns, or 64 when 128 leave the
-// 152 SMs without a block each (the width-512 layers)
+// 152 SMs without a block each (the width-512 layers).  The activation gradient takes 64 x 16 at every size: at
+// 256 x 512 outputs that is 128 blocks (8 with 128 x 128); larger batches and widths, whose operands
+// wider tiles would read less often, are not tuned
 bool wide_tiles(int M, int N) { return (long)((M + 127) / 128) * ((N + 127) / 128) >= 152; }
 
 int rg_of(long rows) { return (int)(pad128(rows) / 8); }
