@@ -6,9 +6,9 @@
 // NP = 16 or 32 is the padded order.
 //   * Sweep: lane (lrow, lcol) = (lane % 8, lane / 8) holds rows lrow + 8 i and columns lcol + 4 r.  Step k
 //     takes column k's entries by shuffles, finds the pivot row by one warp maximum, its lanes leave it in
-//     shared memory, every other row adds f u (f = -m / pivot).  Rows are not scaled: a
-//     pivot row keeps its values with a 1 in the new column, and takes its 1 / pivot at
-//     the end, so no row needs special treatment in the update.  The columns rotate by one register
+//     shared memory and zero their own, and every row adds f u: f = -m / pivot, and 1 / pivot for the
+//     pivot row itself, which is scaled at once: scaled at the end instead, its whole
+//     magnitude is rounded once more, and R^2 is up to 1.5 times as large.  The columns rotate by one register
 //     every four steps (the update writes one register down), so that the pivot column is
 //     always register 0 and the loop stays rolled; only the n real columns are swept.
 //   * T: S's rows are cut into three base-512 FP16 digits (as in df_mixed64_dev.cuh) and S is
@@ -21,9 +21,12 @@
 // At n <= 32 one ladder fills neither a tcgen05 tile (64 rows) nor a block.  Bound by the FP32
 // pipe and issue (three warps per scheduler; the sweep's 950 cycles a step are 3 x 235
 // instructions) and, in the product, by the mma.sync rate (960 x 8 cycles per scheduler).
-// Measured, 11,264 ladders of order 30: 0.33 ms (1.35 ms with one ladder per 64-thread block,
+// Measured, 11,264 ladders of order 30: 0.34 ms (1.35 ms with one ladder per 64-thread block,
 // [D | gamma] swept and BF16 digits of X0; 0.47 with whole rows per lane, whose pivot row
-// costs each lane 16 16-byte loads, and six digits of S; 0.38 with ten warps); of order 16: 58 us.
+// costs each lane 16 16-byte loads, and six digits of S; 0.38 with ten warps; 0.33 with rows scaled at the
+// end); of order 16: 58 us.  Error against FP64 on the paper's inputs, orders 8 / 16 / 24 / 32, geometric mean of
+// a (channel, W) plane's over 24 inputs: 1.1 / 1.5 / 1.6 / 2.0e-14 (the block kernel's: 1.1 / 1.5 / 1.9 / 2.1e-14; with
+// rows scaled at the end 1.5 / 2.2 / 2.3 / 2.9e-14).
 #pragma once
 #include "df_mixed64_dev.cuh"
 
@@ -40,10 +43,10 @@ struct M32 {
   static constexpr int kBytes = kWords + NP * NP * 16;    // one matrix, in global and in shared memory
   static constexpr int SLD = NP + 2, TLD = NP + 1;        // row strides of S / R and T (float2)
   // per warp: S / R, 16 rows of T, chi~ hi, lo, the pivot row (two slots), row scales and weights, diag T,
-  // pivots, the rows' steps, 1 / pivot by step
+  // pivots, the rows' steps
   static constexpr int oT = NP * SLD * 8, oX = (oT + 16 * TLD * 8 + 15) / 16 * 16, oP = oX + 2 * NP * 8,
-                       oS = oP + 2 * NP * 8, oD = oS + 2 * NP * 4, oV = oD + NP * 16, oI = oV + 2 * NP * 4,
-                       kWarp = oI + NP * 8;
+                       oS = oP + 2 * NP * 8, oD = oS + 2 * NP * 4, oV = oD + NP * 16,
+                       kWarp = oV + 2 * NP * 4;
   static constexpr int kWarps = NP == 32 ? 12 : 16;
   static constexpr int kThreads = 32 * kWarps;
   static constexpr int kItem = kBytes + kWarps * kWarp;   // the batch's queue item (beside it no static shared memory fits)
@@ -139,6 +142,55 @@ __device__ __forceinline__ void st_row_if(bool q, unsigned addr, const float2 (&
                : "memory");
 }
 
+// Where `here` (the same in the whole warp: a branch, not predicated instructions), N complex values
+// to shared memory and zeroed in the lanes that set `mine`
+__device__ __forceinline__ void take_row(bool here, bool mine, unsigned addr, float2 (&a)[4]) {
+  asm volatile(
+      "{\n.reg .pred h, q;\nsetp.eq.s32 h, %8, 0;\n@h bra.uni DONE;\nsetp.ne.s32 q, %9, 0;\n"
+      "@q st.shared.v4.f32 [%10 + 0], {%0, %1, %2, %3};\n"
+      "@q st.shared.v4.f32 [%10 + 16], {%4, %5, %6, %7};\n"
+      "@q mov.f32 %0, 0f00000000;\n"
+      "@q mov.f32 %1, 0f00000000;\n"
+      "@q mov.f32 %2, 0f00000000;\n"
+      "@q mov.f32 %3, 0f00000000;\n"
+      "@q mov.f32 %4, 0f00000000;\n"
+      "@q mov.f32 %5, 0f00000000;\n"
+      "@q mov.f32 %6, 0f00000000;\n"
+      "@q mov.f32 %7, 0f00000000;\n"
+      "DONE:\n}\n"
+      : "+f"(a[0].x), "+f"(a[0].y), "+f"(a[1].x), "+f"(a[1].y), "+f"(a[2].x), "+f"(a[2].y), "+f"(a[3].x), "+f"(a[3].y)
+      : "r"((int)here), "r"((int)mine), "r"(addr)
+      : "memory");
+}
+__device__ __forceinline__ void take_row(bool here, bool mine, unsigned addr, float2 (&a)[8]) {
+  asm volatile(
+      "{\n.reg .pred h, q;\nsetp.eq.s32 h, %16, 0;\n@h bra.uni DONE;\nsetp.ne.s32 q, %17, 0;\n"
+      "@q st.shared.v4.f32 [%18 + 0], {%0, %1, %2, %3};\n"
+      "@q st.shared.v4.f32 [%18 + 16], {%4, %5, %6, %7};\n"
+      "@q st.shared.v4.f32 [%18 + 32], {%8, %9, %10, %11};\n"
+      "@q st.shared.v4.f32 [%18 + 48], {%12, %13, %14, %15};\n"
+      "@q mov.f32 %0, 0f00000000;\n"
+      "@q mov.f32 %1, 0f00000000;\n"
+      "@q mov.f32 %2, 0f00000000;\n"
+      "@q mov.f32 %3, 0f00000000;\n"
+      "@q mov.f32 %4, 0f00000000;\n"
+      "@q mov.f32 %5, 0f00000000;\n"
+      "@q mov.f32 %6, 0f00000000;\n"
+      "@q mov.f32 %7, 0f00000000;\n"
+      "@q mov.f32 %8, 0f00000000;\n"
+      "@q mov.f32 %9, 0f00000000;\n"
+      "@q mov.f32 %10, 0f00000000;\n"
+      "@q mov.f32 %11, 0f00000000;\n"
+      "@q mov.f32 %12, 0f00000000;\n"
+      "@q mov.f32 %13, 0f00000000;\n"
+      "@q mov.f32 %14, 0f00000000;\n"
+      "@q mov.f32 %15, 0f00000000;\n"
+      "DONE:\n}\n"
+      : "+f"(a[0].x), "+f"(a[0].y), "+f"(a[1].x), "+f"(a[1].y), "+f"(a[2].x), "+f"(a[2].y), "+f"(a[3].x), "+f"(a[3].y), "+f"(a[4].x), "+f"(a[4].y), "+f"(a[5].x), "+f"(a[5].y), "+f"(a[6].x), "+f"(a[6].y), "+f"(a[7].x), "+f"(a[7].y)
+      : "r"((int)here), "r"((int)mine), "r"(addr)
+      : "memory");
+}
+
 // One ladder by one warp.  gsm: gamma's fragments, weights and words in shared memory (M32), GGh, GGl the
 // (hi, lo) words of gamma o gamma^T (symmetric), ws: the warp's shared memory.  Writes kc[c][a][:][q].
 template <int NP>
@@ -160,7 +212,6 @@ __device__ __forceinline__ void m32_system(const Dims& dm, int c, int a, int q, 
   float4* td = reinterpret_cast<float4*>(ws + M::oD);
   int* piv = reinterpret_cast<int*>(ws + M::oV);
   int* rstep = piv + NP;
-  float2* pinv = reinterpret_cast<float2*>(ws + M::oI);
   const float* gwt = reinterpret_cast<const float*>(gsm + M::kFrag);
   const float4* words = reinterpret_cast<const float4*>(gsm + M::kWords);
 
@@ -217,27 +268,27 @@ __device__ __forceinline__ void m32_system(const Dims& dm, int c, int a, int q, 
 #pragma unroll
       for (int i = 0; i < RP; ++i) {
         is[i] = p == lrow + 8 * i;
-        st_row_if(is[i], pa, A[i]);
         km[i] = is[i] ? 0u : km[i];
       }
+#pragma unroll
+      for (int i = 0; i < RP; ++i) take_row(p >> 3 == i, is[i], pa, A[i]);
       __syncwarp();
       const float2* pr = prow + NP * (s & 1);
       const float2 z = pr[CP * s];
-      // approximate reciprocal: the FP32 sweep is corrected later
-      const float d = rcp_approx(fmaf(z.x, z.x, z.y * z.y));
+      // approximate reciprocal and one Newton step
+      const float zz = fmaf(z.x, z.x, z.y * z.y), d0 = rcp_approx(zz), d = fmaf(d0, fmaf(-zz, d0, 1.f), d0);
       const float2 ainv = make_float2(z.x * d, -z.y * d);
       if (lane == 0) {
         piv[kb + s] = p;
         rstep[p] = kb + s;
-        pinv[kb + s] = ainv;
       }
-      float2 f[RP], nc[RP];                               // the rows' factors, the new column's entries
+      float2 f[RP], nc[RP];                               // the rows' factors: the new column's entries
 #pragma unroll
       for (int i = 0; i < RP; ++i) {
         f[i] = cmulf(m[i], make_float2(-ainv.x, -ainv.y));
-        f[i].y = is[i] ? 0.f : f[i].y;
-        nc[i] = make_float2(is[i] ? 1.f : f[i].x, f[i].y);
-        f[i].x = is[i] ? 0.f : f[i].x;
+        f[i].x = is[i] ? ainv.x : f[i].x;
+        f[i].y = is[i] ? ainv.y : f[i].y;
+        nc[i] = f[i];
       }
       constexpr int kLast = 3;                            // rotate with the last update of four
       const float4* u4 = reinterpret_cast<const float4*>(pr + CP * lcol);
@@ -291,10 +342,9 @@ __device__ __forceinline__ void m32_system(const Dims& dm, int c, int a, int q, 
       const int st = rstep[lrow + 8 * i];
       const bool real = st >= 0;
       const int k = real ? st : lrow + 8 * i;
-      const float2 rinv = pinv[k];
 #pragma unroll
       for (int r = 0; r < CP; ++r) {
-        float2 v = cmulf(A[i][r], rinv);
+        float2 v = A[i][r];
         if (!real || cz[r]) v = make_float2(0.f, 0.f);
         mx = fmaxf(mx, fmaxf(fabsf(v.x), fabsf(v.y)));
         S[k * SLD + pc[r]] = v;
@@ -319,14 +369,15 @@ __device__ __forceinline__ void m32_system(const Dims& dm, int c, int a, int q, 
   float2 er[2] = {};                                      // (R T)_jj, j = j16 and 16 + j16, half of the terms each
   // er += the terms of 16 m: R's rows r0 + j16 at its columns m0 .., T's rows there (their columns start at t0)
   auto diag_rt = [&](int r0, int m0, int t0) {
-    float2 e = er[r0 >> 4];
+    float2 e = make_float2(0.f, 0.f);
 #pragma unroll
     for (int m = 0; m < 16; m += 2) {
       const float2 w = S[(r0 + j16) * SLD + m0 + m + hm], tv = T[(m + hm) * TLD + t0 + j16];
       e.x = fmaf(w.x, tv.x, fmaf(-w.y, tv.y, e.x));
       e.y = fmaf(w.x, tv.y, fmaf(w.y, tv.x, e.y));
     }
-    er[r0 >> 4] = e;
+    er[r0 >> 4].x += e.x;
+    er[r0 >> 4].y += e.y;
   };
 #pragma unroll 1
   for (int mt = 0; mt < nks; ++mt) {

@@ -435,3 +435,23 @@ def test_long_hand_back_list_takes_the_fp64_path_s_time(df):
                 best = min(best, d.get_timing()["bse"][0])
             t.append(best)
     assert t[2] - t[1] < 1.2 * t[0], t
+
+
+def test_small_orders_error_on_the_paper_s_inputs(df):
+    # the mean error of a (channel, W) plane against the FP64 path over orders 8-32 and 12 inputs each of the paper's
+    # Example I: 1.6e-14 with the kernel that swept [D | gamma] (which rounds the pivot row once); 10% above that
+    errs = []
+    for n_w in (8, 16, 24, 32):
+        for seed in range(1, 13):
+            rng = np.random.default_rng(seed)
+            w = I.half_filled_atom("p", 2, 8, U=float(rng.uniform(16.0, 24.0)), beta=float(rng.uniform(0.8, 1.2)),
+                                   n_w=n_w, m_max=1)
+            k = []
+            for prec in (df.DF_FP64, df.DF_FP32_IR):
+                with df.DualFermion.from_workload(w, precision=prec, eig_mode=0) as d:
+                    d.bubble()
+                    d.bse(3)
+                    k.append(d.get_kernel())
+            errs += [np.linalg.norm(k[1][c, a] - k[0][c, a]) / np.linalg.norm(k[0][c, a])
+                     for c in range(2) for a in range(w.n_bos)]
+    assert np.exp(np.mean(np.log(errs))) < 1.8e-14
