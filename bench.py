@@ -515,14 +515,14 @@ def observables_bench(df, I, torch, reps: int = 20):
             "susceptibility_fp32_ir": {"ms_per_call": ir_s * 1e3, "ladders": 2 * w.n_bos * w.N,
                                        "lu_flop_fp64_equivalent": lu_flop,
                                        "fp64_equivalent_GFLOP_per_s": lu_flop / ir_s / 1e9,
-                                       "note": "the same call under DF_FP32_IR: FP32 LU + FP64 refinement "
+                                       "note": "the same call under DF_FP32_IR: FP32 inverse + FP64 refinement "
                                                "(chi_ladder_ir_kernel), FP64 LU for the systems handed back"}}
 
 
 def large_order_bench(df, I, passes: int = 2):
     """The 3D critical workload (16^3, n_w = 96, N_W = 21: 172,032 ladders of order 96) one
-    pass at a time from Sigma~ = 0, FP64 and DF_FP32_IR (orders 64 < n_w <= 96: the Gauss-Jordan
-    inversion and the residual on the tensor cores); ladder time from libdf's own events, the
+    pass at a time from Sigma~ = 0, FP64 and DF_FP32_IR (orders 65-128: the Gauss-Jordan
+    sweep in registers, the digit product on the tensor cores); ladder time from libdf's own events, the
     CUDA-core sweep's time beside it (mixed_sweep = 1), and the normwise difference of the two
     paths' Sigma~ after the first pass."""
     import numpy as np

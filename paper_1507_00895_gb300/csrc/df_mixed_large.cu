@@ -2,7 +2,7 @@
 // df_mixed128_dev.cuh, and with mixed_sweep = 1 the shared-memory Gauss-Jordan kernel
 // (df_mixed_large_dev.cuh: one CTA of 2n threads per ladder, FP32 inversion with row
 // exchanges in shared memory, double-float residual on the CUDA cores), which the default
-// one beats at every order (3D workload, n = 96: 482 ms of ladders per pass against 195) and
+// one beats at every order (3D workload, n = 96: 482 ms of ladders per pass against 182) and
 // which shares no code with it.
 #include "df_mixed128_dev.cuh"
 #include "df_mixed_large_dev.cuh"
