@@ -192,7 +192,7 @@ df_status df_bubble(df_ctx* c);
  * opts.precision); keeps c (Gamma_{W,w,w} - Gamma^(2)_{W,w,w}/2) with
  * Gamma^(2) = gamma chi~ gamma (the double-counting term of Eq. sd).  With
  * eig_mode != 0 also estimates the leading eigenvalue of gamma chi~ (FP64
- * power iteration).  Asynchronous: a zero pivot or |lambda| >= 1 is
+ * power iteration).  Asynchronous: a zero pivot or |lambda| >= 1 (an eigenvalue that is not finite counts) is
  * recorded on the device and reported by the next df_sigma with a residual
  * pointer (DF_ERR_SINGULAR / DF_WARN_LADDER_RADIUS) or by df_iterate.
  * Needs df_bubble first. */

@@ -186,7 +186,8 @@ __device__ __forceinline__ void take_row(bool here, bool mine, unsigned addr, fl
       "@q mov.f32 %14, 0f00000000;\n"
       "@q mov.f32 %15, 0f00000000;\n"
       "DONE:\n}\n"
-      : "+f"(a[0].x), "+f"(a[0].y), "+f"(a[1].x), "+f"(a[1].y), "+f"(a[2].x), "+f"(a[2].y), "+f"(a[3].x), "+f"(a[3].y), "+f"(a[4].x), "+f"(a[4].y), "+f"(a[5].x), "+f"(a[5].y), "+f"(a[6].x), "+f"(a[6].y), "+f"(a[7].x), "+f"(a[7].y)
+      : "+f"(a[0].x), "+f"(a[0].y), "+f"(a[1].x), "+f"(a[1].y), "+f"(a[2].x), "+f"(a[2].y), "+f"(a[3].x), "+f"(a[3].y),
+        "+f"(a[4].x), "+f"(a[4].y), "+f"(a[5].x), "+f"(a[5].y), "+f"(a[6].x), "+f"(a[6].y), "+f"(a[7].x), "+f"(a[7].y)
       : "r"((int)here), "r"((int)mine), "r"(addr)
       : "memory");
 }
