@@ -26,7 +26,7 @@
 // from the growth two steps earlier, so |v| stays near 1 without waiting for
 // this step's norm.
 //
-// Range: chi~ of a system is scaled by the power of two that brings max|gamma|
+// Range: chi~ of a system (and gamma, where it is far from one) is scaled by the power of two that brings max|gamma|
 // max|chi~| to [1/4, 1) (exact; lambda is scaled back in FP64), so that the first two steps, which
 // have no growth to go by, and the squared norms stay within FP32 whatever lambda's size.
 // A growth that changes by many orders of magnitude within two steps (a start vector
@@ -141,59 +141,90 @@ lambda_kernel(Dims dm, int ch0, int a0, int na, double tol, const double2* __res
   // gamma's words, chi~, the start vector
   float2 gh[CPL];
   float2 xh[QL], xl[QL], v[QL], vp[QL];
+  auto split = [](double2 z, float2& hi, float2& lo) {
+    hi = make_float2((float)z.x, (float)z.y);
+    lo = make_float2((float)(z.x - (double)hi.x), (float)(z.y - (double)hi.y));
+  };
+  auto top = [](double2 z) {
+    return (unsigned)max(__double2hiint(z.x) & 0x7FFFFFFF, __double2hiint(z.y) & 0x7FFFFFFF);
+  };
   if (!book) {
+    unsigned gm = 0u, xm[QL];
 #pragma unroll
     for (int k = 0; k < CPL; ++k) {
       const int j = CPL * jb + k;
       const double2 g = (i < n && j < n) ? Gg[(size_t)i * n + j] : mk(0.0, 0.0);
-      gh[k] = make_float2((float)g.x, (float)g.y);
-      glo[jb * LS + k * NP + i] = make_float2((float)(g.x - (double)gh[k].x), (float)(g.y - (double)gh[k].y));
+      float2 lo;
+      split(g, gh[k], lo);
+      glo[jb * LS + k * NP + i] = lo;
+      gm = max(gm, top(g));
     }
 #pragma unroll
     for (int k = 0; k < QL; ++k) {
       const double2 x = (i < n && t0 + k < nq) ? chi[((size_t)a * n + i) * N + q0 + t0 + k] : mk(0.0, 0.0);
-      xh[k] = make_float2((float)x.x, (float)x.y);
-      xl[k] = make_float2((float)(x.x - (double)xh[k].x), (float)(x.y - (double)xh[k].y));
+      split(x, xh[k], xl[k]);
+      xm[k] = top(x);
     }
-    // the largest |gamma| of the warp's rows, the largest |chi~| of its systems' entries
-    unsigned gm = 0u;
-#pragma unroll
-    for (int k = 0; k < CPL; ++k) gm = max(gm, __float_as_uint(fmaxf(fabsf(gh[k].x), fabsf(gh[k].y))));
+    // the largest upper FP64 words of |gamma| in the warp's rows, of |chi~| in its systems' entries
     gm = __reduce_max_sync(0xffffffffu, gm);
     if (lane == 0) part[0][warp][0][7] = __uint_as_float(gm);
 #pragma unroll
     for (int k = 0; k < QL; ++k) {
-      float m = fmaxf(fabsf(xh[k].x), fabsf(xh[k].y));
 #pragma unroll
-      for (int o = 4; o < 32; o <<= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-      if (lane < 4 && owner) part[0][warp][t0 + k][6] = m;
+      for (int o = 4; o < 32; o <<= 1) xm[k] = max(xm[k], __shfl_xor_sync(0xffffffffu, xm[k], o));
+      if (lane < 4 && owner) part[0][warp][t0 + k][6] = __uint_as_float(xm[k]);
     }
   }
   __syncthreads();
-  // chi~ of system t by 2^-e: lambda of the scaled problem is 2^-e lambda (e of an infinite or NaN
-  // product: 0); false for A = 0
-  auto range_exp = [&](int t, int& e) {
-    float g = 0.f, x = 0.f;
+  // exponents of the block's gamma and of system t's chi~ (|value| < 2^e; 0 for an infinite or NaN one): lambda
+  // of the problem with both brought to 2^0 is 2^-(eg + ex) lambda.  False for A = 0
+  int eg = 0;                                        // (the block's)
+  auto range_exp = [&](int t, int& ex) {
+    unsigned g = 0u, x = 0u;
 #pragma unroll
     for (int w = 0; w < NW; ++w) {
-      g = fmaxf(g, part[0][w][0][7]);
-      x = fmaxf(x, part[0][w][t][6]);
+      g = max(g, __float_as_uint(part[0][w][0][7]));
+      x = max(x, __float_as_uint(part[0][w][t][6]));
     }
-    e = g < INFINITY && x < INFINITY ? exp_bound_f32(g) + exp_bound_f32(x) : 0;
-    return g > 0.f && x > 0.f;
+    eg = g != 0u && g < 0x7FF00000u ? (int)(g >> 20) - 1022 : 0;
+    ex = x < 0x7FF00000u ? (int)(x >> 20) - 1022 : 0;
+    return g != 0u && x != 0u;
   };
-  int lexp = 0;                                      // e of the bookkeeping lane's system
+  int lexp = 0;                                      // eg + ex of the bookkeeping lane's system
   bool alive = false;
   if (book) {
-    if (lane < nq && !(alive = range_exp(lane, lexp))) lexp = 0;
+    if (lane < nq) {
+      alive = range_exp(lane, lexp);
+      lexp = alive ? lexp + eg : 0;
+    }
   } else {
+    // far from one, the words are made anew from the scaled FP64 value (their trailing ones would leave FP32's
+    // range); else chi~'s alone take both powers of two
+    constexpr int kFar = 40;
 #pragma unroll
     for (int k = 0; k < QL; ++k) {
-      int e;
-      if (!range_exp(t0 + k, e)) e = 0;
-      const float s1 = pow2f(-(e >> 1)), s2 = pow2f((e >> 1) - e);   // (2^-e itself may leave FP32's range)
-      xh[k] = cscale(cscale(xh[k], s1), s2);
-      xl[k] = cscale(cscale(xl[k], s1), s2);
+      int ex;
+      if (!range_exp(t0 + k, ex)) continue;
+      int r = ex + (eg > kFar || eg < -kFar ? 0 : eg);
+      if (ex > kFar || ex < -kFar) {
+        const double2 x = (i < n && t0 + k < nq) ? chi[((size_t)a * n + i) * N + q0 + t0 + k] : mk(0.0, 0.0);
+        split(mk(scalbn(x.x, -ex), scalbn(x.y, -ex)), xh[k], xl[k]);
+        r -= ex;
+      }
+      xh[k] = cscale(xh[k], pow2f(-r));
+      xl[k] = cscale(xl[k], pow2f(-r));
+    }
+    if (eg > kFar || eg < -kFar) {
+      for (int k = 0; k < CPL; ++k) {
+        const int j = CPL * jb + k;
+        const double2 g = (i < n && j < n) ? Gg[(size_t)i * n + j] : mk(0.0, 0.0);
+        float2 hi, lo;
+        split(mk(scalbn(g.x, -eg), scalbn(g.y, -eg)), hi, lo);
+#pragma unroll
+        for (int m = 0; m < CPL; ++m)
+          if (m == k) gh[m] = hi;
+        glo[jb * LS + k * NP + i] = lo;
+      }
     }
   }
 

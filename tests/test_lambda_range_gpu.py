@@ -105,3 +105,44 @@ def test_zero_vertex(df):
         assert d.iterate(1)[2] == df.DF_OK
         lam, ok = d.get_lambda()
     assert np.all(lam == 0.0) and np.all(ok == 1)
+
+
+def test_product_at_the_end_of_the_fp32_range(df):
+    # chi~ = -T G0~^2 = -2^127 (g = 2^63, Delta = 1 / g: G0~ = -g / 2) and gamma = -2^126 diag(1, 1/4): lambda = 2^253
+    g = np.full(2, 2.0 ** 63, complex)
+    d_ = np.full(2, 2.0 ** -63, complex)
+    gam = np.diag([-(2.0 ** 126), -(2.0 ** 124)]).astype(complex)[None]
+    for up in (1.0, 2.0, 1.75):
+        with df.DualFermion(dim=1, nk=2, t=0.0, tp=0.0, beta=0.125, mu=0.0, n_w=2, m_max=0, g=g, delta=d_,
+                            gamma_d=up * gam, gamma_m=gam, eig_mode=2) as d:
+            d.bubble()
+            chi = d.get_chi()
+            d.bse(3)
+            lam, ok = d.get_lambda()
+        assert np.all(chi == chi[0, 0, 0]) and chi[0, 0, 0] == -(2.0 ** 127)
+        ref = up * gam[0, 0, 0] * chi[0, 0, 0]
+        assert np.max(np.abs(lam[0] - ref)) < 1e-8 * abs(ref), (lam[0], ref)
+
+
+@pytest.mark.parametrize("n_w", [8, 48, 128])
+@pytest.mark.parametrize("p,q", [(-290, 0), (-60, 40), (45, -45), (60, 60), (250, 20), (41, 39)])
+def test_vertex_and_bubble_far_from_one(df, n_w, p, q):
+    """gamma by 2^p and beta by 2^-q (chi~ has the prefactor T): lambda is scaled by 2^(p + q), FP64's
+    eigenvalues with it, wherever gamma's or chi~'s FP32 words would lie."""
+    w = I.random_nonsymmetric(n_w, 0, 1, 4, seed=500 + n_w, scale=0.7)
+    w.gamma_uu[:] += 3.0 * np.linspace(0.5, 1.0, n_w)[:, None]
+    w.gamma_ud[:] *= 0.2
+    lam = []
+    for a, b in ((0, 0), (p, q)):
+        v = w.scaled(2.0 ** a)
+        v.beta = w.beta * 2.0 ** -b
+        with df.DualFermion.from_workload(v, eig_mode=2) as d:
+            d.bubble()
+            chi = d.get_chi()
+            d.bse(3)
+            lam.append(d.get_lambda())
+    ref = lam[0][0] * 2.0 ** p * 2.0 ** q
+    assert np.array_equal(lam[0][1], lam[1][1])
+    m = lam[0][1] == 1
+    assert np.any(m)
+    assert np.max(np.abs(lam[1][0] - ref)[m] / np.abs(ref)[m]) < 1e-8
